@@ -132,11 +132,13 @@ __device__ __forceinline__ float u01_from_u32(uint32_t raw)
 }
 
 // Ran2 uniform: min(fl(AM * fl(iy)), RNMX), AM = fl(1/m1), RNMX < 1.
+// iy <= m1 - 1 = 2147483562, whose binary32 neighbour is 2^31 - 128, so
+// AM fl(iy) never exceeds RNMX = 1 - 2^-24 and the minimum selects nothing.
+static_assert((float)kR2Imm1 * 0x1p-31f == 0x1.fffffep-1f, "AM fl(m1 - 1) is RNMX");
 __device__ __forceinline__ float u01_from_ran2(int32_t iy)
 {
     const float am = 0x1p-31f;   // fl32(1/2147483563) rounds to 2^-31 exactly
-    const float rnmx = 0x1.fffffep-1f;
-    return fminf(__fmul_rn(am, __int2float_rn(iy)), rnmx);
+    return __fmul_rn(am, __int2float_rn(iy));
 }
 
 // Open-interval Box-Muller input ((raw >> 9) + 1/2) * 2^-23, exact in
@@ -205,7 +207,7 @@ __device__ __forceinline__ float neg2log(float u)
 __device__ __forceinline__ float sqrt_pos(float y)
 {
     float r;
-    asm("sqrt.approx.f32 %0, %1;" : "=f"(r) : "f"(y));
+    asm("sqrt.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(y));
     return r;
 }
 
