@@ -116,6 +116,8 @@ int fill_uniform_pt(Handle* h, float* dst, int64_t n, cudaStream_t st);
 int fill_normal_pt(Handle* h, float* dst, int64_t n, cudaStream_t st);
 int ld_init_pt(const ld_system* s, cudaStream_t st);
 int ld_run_pt(const ld_system* s, int64_t n_steps, ld_stats* out, cudaStream_t st);
+// Small systems, Hybrid Taus and the LCG, n_steps >= 1 (team.cu).
+int ld_team(const ld_system* s, int64_t n_steps, bool want_stats, int64_t* blocks_out, cudaStream_t st);
 
 // Lagged Fibonacci entry points (lfg.cu)
 int lfg_seed(Handle* h, cudaStream_t st);
@@ -143,6 +145,8 @@ int lfg_ou(const ou_system* s, int64_t n_steps, int64_t every, double* mean, dou
            cudaStream_t st);
 int ou_finish(Handle* h, int64_t n, int64_t n_rec, int64_t blocks, double* mean, double* corr,
               cudaStream_t st);
+
+int ou_team(const ou_system* s, int64_t n_steps, int64_t every, bool rec, int64_t* blocks_out, cudaStream_t st);
 
 // Statistics: reduce `blocks` partials (4 doubles each) into h->dstats and
 // copy to the host (synchronising st).

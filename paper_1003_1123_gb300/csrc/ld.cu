@@ -222,14 +222,12 @@ __global__ void __launch_bounds__(32) ld_pair_kernel(LdArgs a, int64_t n_pairs)
 }
 
 // Pair-kernel grid: one full resident wave of one-warp blocks (16 a SM for
-// Taus, 20 for Ran2 at 1e6 oscillators).  Measured at 1e6 oscillators x 1000
-// steps (scalar arithmetic): 5.90 ms for Hybrid Taus against 6.13 ms for one
-// oscillator a thread; 64-, 128- and 256-thread blocks 6.06-6.60 ms; a grid
-// trimmed so that every thread gets the same number of pairs (fewer warps a
-// SM) 6.36 ms.  With the paired instructions: Taus 4.9 ms, Ran2 6.3 ms (64-
-// thread blocks for Ran2 equal).  Returns 0 (and launches nothing) when the
-// pairs do not fill one resident wave, where one oscillator a thread spreads
-// better.
+// Taus, 20 for Ran2 at 1e6 oscillators), fewer where the pairs do not fill it.
+// Measured at 1e6 oscillators x 1000 steps (scalar arithmetic): 5.90 ms for
+// Hybrid Taus against 6.13 ms for one oscillator a thread; 64-, 128- and
+// 256-thread blocks 6.06-6.60 ms; a grid trimmed so that every thread gets the
+// same number of pairs (fewer warps a SM) 6.36 ms.  With the paired
+// instructions: Taus 4.7 ms, Ran2 6.0 ms (64-thread blocks for Ran2 equal).
 template <int KIND>
 static int launch_pairs(const ld_system* s, int64_t n_steps, bool want_stats, int64_t* blocks_out,
                         cudaStream_t st)
@@ -241,10 +239,9 @@ static int launch_pairs(const ld_system* s, int64_t n_steps, bool want_stats, in
     const size_t smem = KIND == GBRNG_RAN2 ? sizeof(int32_t) * 2 * 32 * T : 0;
     int occ = 0;
     GB_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, ld_pair_kernel<KIND>, T, smem));
-    if (occ < 1) return 0;
-    const int64_t pairs = (s->n + 1) / 2, wave = (int64_t)di.sms * occ * T;
-    if (pairs < wave) return 0;
-    const int64_t blocks = wave / T;
+    if (occ < 1) occ = 1;
+    const int64_t pairs = (s->n + 1) / 2;
+    const int64_t blocks = std::min<int64_t>((int64_t)di.sms * occ, (pairs + T - 1) / T);
     if (want_stats) GB_CHECK(ensure_partials(h, blocks));
     LdArgs a;
     a.n = s->n;
@@ -261,7 +258,7 @@ static int launch_pairs(const ld_system* s, int64_t n_steps, bool want_stats, in
     ld_pair_kernel<KIND><<<(unsigned)blocks, T, smem, st>>>(a, pairs);
     GB_CUDA(cudaGetLastError());
     *blocks_out = blocks;
-    return 1;
+    return GBRNG_OK;
 }
 
 // Grid shape: threads per block T and one full resident wave (SMs x blocks
@@ -315,6 +312,36 @@ int ld_init_pt(const ld_system* s, cudaStream_t st)
     return launch_ld<GBRNG_RAN2, true>(s, 0, false, &blocks, st);
 }
 
+// Which kernel runs a system.  A run's time is the steps' times the time of a
+// step, which for the thread-per-oscillator kernels goes by the warps on the
+// busiest scheduler (w1 with one oscillator a thread, w2 with two) and for the
+// teams by the oscillators a SM holds.  Measured for Hybrid Taus, ns a step:
+// one a thread 134, 206, 313, 408, 505, 602, 698, 795 for w1 = 1 .. 8; two a
+// thread 212, 377, 551, 723 for w2 = 1 .. 4 (16 warps a SM: a full wave); teams
+// 28 + 0.79 per oscillator a SM, and 8 us + 5.5 us per 1e4 oscillators more at
+// their start than the others.  The LCG's (87, 142, 210, 275, 340, 405 / 152,
+// 255, 377, 491 / 0.52) and Ran2's (763 against 740 at w1 = 6, 1000 against 957
+// at w1 = 8) stand to each other alike.
+enum LdPath { LD_ONE, LD_PAIRS, LD_TEAM };
+static LdPath pick_path(int kind, int64_t n, int64_t n_steps, int sms)
+{
+    const int64_t w1 = (n + 128ll * sms - 1) / (128ll * sms), w2 = (n + 256ll * sms - 1) / (256ll * sms);
+    if (w1 > 8) return LD_PAIRS;
+    const double one = w1 <= 2 ? 62 + 72.0 * (double)w1 : 5 + 100.0 * (double)w1;
+    const double pairs = 38 + 172.0 * (double)w2;
+    const double team = 28 + 0.79 * (double)n / sms + (8000 + 0.55 * (double)n) / (double)std::max<int64_t>(n_steps, 1);
+    if (kind != GBRNG_RAN2 && team < std::min(one, pairs)) return LD_TEAM;
+    return pairs < one ? LD_PAIRS : LD_ONE;
+}
+
+template <int KIND>
+static int run_kind(const ld_system* s, LdPath path, int64_t n_steps, bool want, int64_t* blocks,
+                    cudaStream_t st)
+{
+    if (path == LD_PAIRS) return launch_pairs<KIND>(s, n_steps, want, blocks, st);
+    return launch_ld<KIND, false>(s, n_steps, want, blocks, st);
+}
+
 int ld_run_pt(const ld_system* s, int64_t n_steps, ld_stats* out, cudaStream_t st)
 {
     if (s->n == 0) {
@@ -323,21 +350,17 @@ int ld_run_pt(const ld_system* s, int64_t n_steps, ld_stats* out, cudaStream_t s
     }
     int64_t blocks = 0;
     const bool want = out != nullptr;
-    int rc = 0;
-    if (s->rng->kind == GBRNG_TAUS)
-        rc = launch_pairs<GBRNG_TAUS>(s, n_steps, want, &blocks, st);
+    DevInfo di;
+    GB_CHECK(dev_info(s->rng->device, &di));
+    const LdPath path = pick_path(s->rng->kind, s->n, n_steps, di.sms);
+    if (path == LD_TEAM)
+        GB_CHECK(ld_team(s, n_steps, want, &blocks, st));
+    else if (s->rng->kind == GBRNG_TAUS)
+        GB_CHECK(run_kind<GBRNG_TAUS>(s, path, n_steps, want, &blocks, st));
     else if (s->rng->kind == GBRNG_LCG)
-        rc = launch_pairs<GBRNG_LCG>(s, n_steps, want, &blocks, st);
-    else if (s->rng->kind == GBRNG_RAN2)
-        rc = launch_pairs<GBRNG_RAN2>(s, n_steps, want, &blocks, st);
-    if (rc < 0) return rc;
-    if (rc == 1) return finish_stats(s->rng, blocks, n_steps, out, st);
-    if (s->rng->kind == GBRNG_TAUS)
-        GB_CHECK((launch_ld<GBRNG_TAUS, false>(s, n_steps, want, &blocks, st)));
-    else if (s->rng->kind == GBRNG_LCG)
-        GB_CHECK((launch_ld<GBRNG_LCG, false>(s, n_steps, want, &blocks, st)));
+        GB_CHECK(run_kind<GBRNG_LCG>(s, path, n_steps, want, &blocks, st));
     else
-        GB_CHECK((launch_ld<GBRNG_RAN2, false>(s, n_steps, want, &blocks, st)));
+        GB_CHECK(run_kind<GBRNG_RAN2>(s, path, n_steps, want, &blocks, st));
     return finish_stats(s->rng, blocks, n_steps, out, st);
 }
 

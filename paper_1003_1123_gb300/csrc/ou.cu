@@ -184,6 +184,10 @@ int ou_run_pt(const ou_system* s, int64_t n_steps, int64_t every, double* mean, 
     const int64_t blocks = (s->n + T - 1) / T;
     const bool rec = mean != nullptr;
     const int64_t n_rec = n_steps / every + 1;
+    int64_t team_blocks = 0;
+    const int rc = ou_team(s, n_steps, every, rec, &team_blocks, st);
+    if (rc < 0) return rc;
+    if (rc == 1) return rec ? ou_finish(h, s->n, n_rec, team_blocks, mean, corr, st) : GBRNG_OK;
     if (rec) {
         if (n_rec > 0x7fffffff || (double)n_rec * blocks * 16.0 > 4.0 * (1 << 30))
             return fail(GBRNG_EINVAL, "%lld records x %lld blocks exceed the record scratch",

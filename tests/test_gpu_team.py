@@ -1,0 +1,67 @@
+"""Small systems of Hybrid Taus and the LCG run in teams (producer warps over
+jumped-ahead generators, one consumer warp): trajectories and generator states
+equal the thread-per-oscillator kernels' bit for bit at the edges of the blocks
+(8 and 16 oscillators), of a chunk (16 or 32 steps), a stage and a pass."""
+import numpy as np
+import pytest
+import torch
+
+from paper_1003_1123_gb300 import workloads as W
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def G():
+    if not torch.cuda.is_available():
+        pytest.skip("needs a CUDA GPU")
+    from paper_1003_1123_gb300 import gbrng
+    gbrng.lib()
+    return gbrng
+
+
+def system(G, kind, n):
+    s = G.LdSystem(G.rng_init(kind, 17, n), torch.zeros((n, 3), device="cuda"),
+                   torch.zeros((n, 3), device="cuda"),
+                   K_per=torch.from_numpy(W.spring_constants(n, n)).cuda())
+    G.ld_init_equilibrium(s)
+    return s
+
+
+@pytest.mark.parametrize("kind", ["taus", "lcg"])
+@pytest.mark.parametrize("n,steps", [(1, 200), (8, 511), (9, 512), (1000, 513), (1000, 1041), (4864, 128),
+                                     (4865, 255), (4865, 257), (14593, 600), (30001, 700)])
+def test_team_equals_paper_form(G, kind, n, steps):
+    """ld_run against ld_run_stepwise, whose x, v and states are the same binary32
+    operations one launch a step."""
+    a, b = system(G, kind, n), system(G, kind, n)
+    sa, sb = G.ld_run(a, steps), G.ld_run_stepwise(b, steps)
+    assert torch.equal(a.x, b.x) and torch.equal(a.v, b.v)
+    assert G.rng_get_state(a.rng) == G.rng_get_state(b.rng)
+    # binary64 sums of the same binary32 values, and two compensated binary32 sums
+    assert abs(sa["sum_x2"] / sb["sum_x2"] - 1) < 1e-12
+    assert abs(sa["energy_time_avg"] / sb["energy_time_avg"] - 1) < 1e-6
+
+
+@pytest.mark.parametrize("kind", ["taus", "lcg"])
+@pytest.mark.parametrize("n,steps,every", [(1, 100, 1), (7, 1024, 512), (9, 1025, 31), (2433, 511, 33),
+                                           (2433, 513, 100), (20001, 300, 300)])
+def test_overdamped_team_equals_short_runs(G, kind, n, steps, every):
+    """One long overdamped run against runs of at most 40 steps (one particle a
+    thread): positions and states bit for bit, records to binary64 rounding."""
+    R0 = torch.linspace(-3, 4, n, device="cuda")
+    kw = dict(k_sp=0.01, xi=16.568, kT=4.142, dt=1.0)
+    a = G.OuSystem(G.rng_init(kind, 5, n), R0.clone(), **kw)
+    b = G.OuSystem(G.rng_init(kind, 5, n), R0.clone(), **kw)
+    mean, corr = G.ou_run(a, steps, every)
+    m, c = [], []
+    for t in range(steps + 1):
+        if t % every == 0:
+            Rd = b.R.double()
+            m.append(Rd.mean().item())
+            c.append((Rd * R0.double()).mean().item())
+        if t < steps:
+            G.ou_run(b, 1)
+    assert torch.equal(a.R, b.R)
+    assert G.rng_get_state(a.rng) == G.rng_get_state(b.rng)
+    assert np.allclose(mean, m, rtol=0, atol=1e-12) and np.allclose(corr, c, rtol=0, atol=1e-11)
