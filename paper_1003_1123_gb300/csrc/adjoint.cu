@@ -46,7 +46,7 @@ struct AdjArgs {
     float* gbuf;        // [S][3][n] history (hist) or [P][3][n] segment scratch
     int hist;
     float* dK;          // [n] or null
-    double* partials;   // [grid][4]: loss, dgamma, dkT, unused
+    StatsSink sink;     // loss, dgamma, dkT, unused
 };
 
 // 64-thread blocks with an 85-register budget: twelve blocks per SM (116736
@@ -231,9 +231,7 @@ __global__ void __launch_bounds__(64, 12) adjoint_kernel(AdjArgs a)
         acc[2] += dT.value();
     }
     block_reduce_sum<4>(acc, red);
-    if (threadIdx.x == 0)
-#pragma unroll
-        for (int k = 0; k < 4; ++k) a.partials[4 * blockIdx.x + k] = acc[k];
+    if (threadIdx.x < 32) store_stats(a.sink, acc);
 }
 
 // Largest noise history (bytes) ld_backward keeps; -1: half the free device
@@ -301,8 +299,8 @@ extern "C" int ld_backward(ld_system* sys, int64_t n_steps, int ckpt_every, floa
     if (e != cudaSuccess || occ < 1) occ = 1;
     // one full resident wave at most; oscillators i, i + W, ... per thread
     const int64_t blocks = std::min<int64_t>((int64_t)di.sms * occ, (n + T - 1) / T);
-    GB_CHECK(ensure_partials(h, blocks));
     AdjArgs a;
+    GB_CHECK(make_sink(h, blocks, true, &a.sink));
     a.n = n;
     a.S = n_steps;
     a.P = P;
@@ -323,7 +321,6 @@ extern "C" int ld_backward(ld_system* sys, int64_t n_steps, int ckpt_every, floa
     a.gbuf = scratch + ck_bytes / sizeof(float);
     a.hist = hist ? 1 : 0;
     a.dK = dK_per;
-    a.partials = h->partials;
     if (h->kind == GBRNG_TAUS)
         adjoint_kernel<GBRNG_TAUS><<<(unsigned)blocks, T, smem, st>>>(a);
     else
@@ -331,7 +328,7 @@ extern "C" int ld_backward(ld_system* sys, int64_t n_steps, int ckpt_every, floa
     e = cudaGetLastError();
     if (e != cudaSuccess) return fail(GBRNG_ECUDA, "adjoint launch failed: %s", cudaGetErrorString(e));
     ld_stats tmp;
-    GB_CHECK(finish_stats(h, blocks, 1, &tmp, st));
+    GB_CHECK(finish_stats(h, a.sink, blocks, 1, &tmp, st));
     if (loss) *loss = tmp.sum_x2;
     if (dgamma) *dgamma = tmp.sum_v2;
     if (dkT) *dkT = tmp.sum_xv;

@@ -68,10 +68,9 @@ struct Handle {
     // scratch owned by the handle
     uint64_t* progress = nullptr;   // grid-barrier arrival counter (LFG)
     int64_t progress_cap = 0;
-    int* dstatus = nullptr;         // device status word
+    int* dstatus = nullptr;         // device status word, then the statistics' ticket
     double* partials = nullptr;     // per-block reduction partials
     int64_t partials_cap = 0;
-    double* dstats = nullptr;       // 8 doubles of final statistics
     float2* eacc = nullptr;         // paper-form runs: per-oscillator energy sum (Kahan s, c)
     int64_t eacc_cap = 0;
     float* adj = nullptr;           // adjoint checkpoints and noise (history or one segment)
@@ -117,7 +116,7 @@ int fill_normal_pt(Handle* h, float* dst, int64_t n, cudaStream_t st);
 int ld_init_pt(const ld_system* s, cudaStream_t st);
 int ld_run_pt(const ld_system* s, int64_t n_steps, ld_stats* out, cudaStream_t st);
 // Small systems, Hybrid Taus and the LCG, n_steps >= 1 (team.cu).
-int ld_team(const ld_system* s, int64_t n_steps, bool want_stats, int64_t* blocks_out, cudaStream_t st);
+int ld_team(const ld_system* s, int64_t n_steps, ld_stats* out, cudaStream_t st);
 
 // Lagged Fibonacci entry points (lfg.cu)
 int lfg_seed(Handle* h, cudaStream_t st);
@@ -148,9 +147,19 @@ int ou_finish(Handle* h, int64_t n, int64_t n_rec, int64_t blocks, double* mean,
 
 int ou_team(const ou_system* s, int64_t n_steps, int64_t every, bool rec, int64_t* blocks_out, cudaStream_t st);
 
-// Statistics: reduce `blocks` partials (4 doubles each) into h->dstats and
-// copy to the host (synchronising st).
-int finish_stats(Handle* h, int64_t blocks, int64_t n_steps, ld_stats* out, cudaStream_t st);
+// Pinned mapped memory of this host thread for a call's results (at most
+// kHostBlock bytes): a call that has kernels write there reads it, synchronised,
+// before it returns.  Null if it cannot be allocated.
+constexpr size_t kHostBlock = 65536;
+void* host_block();
+
+// Statistics.  make_sink: where a launch of `blocks` blocks leaves its sums
+// (partials grown if needed).  finish_stats: add them up if the launch has not,
+// synchronise st and fill out (no-op for out == null).
+struct StatsSink;
+int make_sink(Handle* h, int64_t blocks, bool want, StatsSink* out);
+int finish_stats(Handle* h, const StatsSink& sink, int64_t blocks, int64_t n_steps, ld_stats* out,
+                 cudaStream_t st);
 
 // Lagged Fibonacci Table I (row 4 as sl = 13470).
 int lfg_lags(int row, int32_t* sl, int32_t* ll);

@@ -22,7 +22,7 @@ struct LdArgs {
     int32_t* r2;       // Ran2 state [35][streams]
     uint32_t* lcg;     // LCG state [streams]
     int64_t S;         // streams of the generator (row stride of r2)
-    double* partials;  // [gridDim.x][4]
+    StatsSink sink;
 };
 
 // Register budget (128-thread blocks per SM, measured at 1e6 oscillators):
@@ -108,11 +108,9 @@ __global__ void __launch_bounds__(128, KIND == GBRNG_LCG ? 7 : 6) ld_pt_kernel(L
         acc[2] += (double)x0 * v0 + (double)x1 * v1 + (double)x2 * v2;
         acc[3] += es.value(hK, c.hm);
     }
-    if (a.partials) {
+    if (a.sink.partials) {
         block_reduce_sum<4>(acc, red);
-        if (threadIdx.x == 0)
-#pragma unroll
-            for (int k = 0; k < 4; ++k) a.partials[4 * blockIdx.x + k] = acc[k];
+        if (threadIdx.x < 32) store_stats(a.sink, acc);
     }
 }
 
@@ -213,11 +211,9 @@ __global__ void __launch_bounds__(32) ld_pair_kernel(LdArgs a, int64_t n_pairs)
             acc[3] += es.value(j, hK[j], c.hm);
         }
     }
-    if (a.partials) {
+    if (a.sink.partials) {
         block_reduce_sum<4>(acc, red);
-        if (threadIdx.x == 0)
-#pragma unroll
-            for (int k = 0; k < 4; ++k) a.partials[4 * blockIdx.x + k] = acc[k];
+        if (threadIdx.x < 32) store_stats(a.sink, acc);
     }
 }
 
@@ -229,8 +225,7 @@ __global__ void __launch_bounds__(32) ld_pair_kernel(LdArgs a, int64_t n_pairs)
 // same number of pairs (fewer warps a SM) 6.36 ms.  With the paired
 // instructions: Taus 4.7 ms, Ran2 6.0 ms (64-thread blocks for Ran2 equal).
 template <int KIND>
-static int launch_pairs(const ld_system* s, int64_t n_steps, bool want_stats, int64_t* blocks_out,
-                        cudaStream_t st)
+static int launch_pairs(const ld_system* s, int64_t n_steps, ld_stats* out, cudaStream_t st)
 {
     Handle* h = s->rng;
     DevInfo di;
@@ -242,7 +237,6 @@ static int launch_pairs(const ld_system* s, int64_t n_steps, bool want_stats, in
     if (occ < 1) occ = 1;
     const int64_t pairs = (s->n + 1) / 2;
     const int64_t blocks = std::min<int64_t>((int64_t)di.sms * occ, (pairs + T - 1) / T);
-    if (want_stats) GB_CHECK(ensure_partials(h, blocks));
     LdArgs a;
     a.n = s->n;
     a.n_steps = n_steps;
@@ -254,11 +248,10 @@ static int launch_pairs(const ld_system* s, int64_t n_steps, bool want_stats, in
     a.r2 = h->r2;
     a.lcg = h->lcg;
     a.S = h->n;
-    a.partials = want_stats ? h->partials : nullptr;
+    GB_CHECK(make_sink(h, blocks, out != nullptr, &a.sink));
     ld_pair_kernel<KIND><<<(unsigned)blocks, T, smem, st>>>(a, pairs);
     GB_CUDA(cudaGetLastError());
-    *blocks_out = blocks;
-    return GBRNG_OK;
+    return finish_stats(h, a.sink, blocks, n_steps, out, st);
 }
 
 // Grid shape: threads per block T and one full resident wave (SMs x blocks
@@ -269,8 +262,7 @@ static int launch_pairs(const ld_system* s, int64_t n_steps, bool want_stats, in
 // cut to ceil(n / (oscillators per thread x T)) blocks leaves some SMs a block
 // short and others a block over, about 9% apart at 1e6 oscillators.)
 template <int KIND, bool INIT>
-static int launch_ld(const ld_system* s, int64_t n_steps, bool want_stats, int64_t* blocks_out,
-                     cudaStream_t st)
+static int launch_ld(const ld_system* s, int64_t n_steps, ld_stats* out, cudaStream_t st)
 {
     Handle* h = s->rng;
     DevInfo di;
@@ -285,7 +277,6 @@ static int launch_ld(const ld_system* s, int64_t n_steps, bool want_stats, int64
     if (occ < 1) occ = 1;
     int64_t blocks = std::min<int64_t>((int64_t)di.sms * occ, (s->n + T - 1) / T);
     if (blocks < 1) blocks = 1;
-    if (want_stats) GB_CHECK(ensure_partials(h, blocks));
     LdArgs a;
     a.n = s->n;
     a.n_steps = n_steps;
@@ -297,19 +288,17 @@ static int launch_ld(const ld_system* s, int64_t n_steps, bool want_stats, int64
     a.r2 = h->r2;
     a.lcg = h->lcg;
     a.S = h->n;
-    a.partials = want_stats ? h->partials : nullptr;
+    GB_CHECK(make_sink(h, blocks, out != nullptr, &a.sink));
     ld_pt_kernel<KIND, INIT><<<(unsigned)blocks, T, smem, st>>>(a);
     GB_CUDA(cudaGetLastError());
-    *blocks_out = blocks;
-    return GBRNG_OK;
+    return finish_stats(h, a.sink, blocks, n_steps, out, st);
 }
 
 int ld_init_pt(const ld_system* s, cudaStream_t st)
 {
-    int64_t blocks = 0;
-    if (s->rng->kind == GBRNG_TAUS) return launch_ld<GBRNG_TAUS, true>(s, 0, false, &blocks, st);
-    if (s->rng->kind == GBRNG_LCG) return launch_ld<GBRNG_LCG, true>(s, 0, false, &blocks, st);
-    return launch_ld<GBRNG_RAN2, true>(s, 0, false, &blocks, st);
+    if (s->rng->kind == GBRNG_TAUS) return launch_ld<GBRNG_TAUS, true>(s, 0, nullptr, st);
+    if (s->rng->kind == GBRNG_LCG) return launch_ld<GBRNG_LCG, true>(s, 0, nullptr, st);
+    return launch_ld<GBRNG_RAN2, true>(s, 0, nullptr, st);
 }
 
 // Which kernel runs a system.  A run's time is the steps' times the time of a
@@ -335,11 +324,10 @@ static LdPath pick_path(int kind, int64_t n, int64_t n_steps, int sms)
 }
 
 template <int KIND>
-static int run_kind(const ld_system* s, LdPath path, int64_t n_steps, bool want, int64_t* blocks,
-                    cudaStream_t st)
+static int run_kind(const ld_system* s, LdPath path, int64_t n_steps, ld_stats* out, cudaStream_t st)
 {
-    if (path == LD_PAIRS) return launch_pairs<KIND>(s, n_steps, want, blocks, st);
-    return launch_ld<KIND, false>(s, n_steps, want, blocks, st);
+    if (path == LD_PAIRS) return launch_pairs<KIND>(s, n_steps, out, st);
+    return launch_ld<KIND, false>(s, n_steps, out, st);
 }
 
 int ld_run_pt(const ld_system* s, int64_t n_steps, ld_stats* out, cudaStream_t st)
@@ -348,20 +336,13 @@ int ld_run_pt(const ld_system* s, int64_t n_steps, ld_stats* out, cudaStream_t s
         if (out) *out = ld_stats{0, 0, 0, 0, n_steps};
         return GBRNG_OK;
     }
-    int64_t blocks = 0;
-    const bool want = out != nullptr;
     DevInfo di;
     GB_CHECK(dev_info(s->rng->device, &di));
     const LdPath path = pick_path(s->rng->kind, s->n, n_steps, di.sms);
-    if (path == LD_TEAM)
-        GB_CHECK(ld_team(s, n_steps, want, &blocks, st));
-    else if (s->rng->kind == GBRNG_TAUS)
-        GB_CHECK(run_kind<GBRNG_TAUS>(s, path, n_steps, want, &blocks, st));
-    else if (s->rng->kind == GBRNG_LCG)
-        GB_CHECK(run_kind<GBRNG_LCG>(s, path, n_steps, want, &blocks, st));
-    else
-        GB_CHECK(run_kind<GBRNG_RAN2>(s, path, n_steps, want, &blocks, st));
-    return finish_stats(s->rng, blocks, n_steps, out, st);
+    if (path == LD_TEAM) return ld_team(s, n_steps, out, st);
+    if (s->rng->kind == GBRNG_TAUS) return run_kind<GBRNG_TAUS>(s, path, n_steps, out, st);
+    if (s->rng->kind == GBRNG_LCG) return run_kind<GBRNG_LCG>(s, path, n_steps, out, st);
+    return run_kind<GBRNG_RAN2>(s, path, n_steps, out, st);
 }
 
 }  // namespace gb

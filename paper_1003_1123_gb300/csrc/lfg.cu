@@ -1121,7 +1121,7 @@ int lfg_ld(const ld_system* s, int64_t n_steps, int init, ld_stats* out, cudaStr
             GB_CHECK(ensure_partials(h, 256));
             snapshot_kernel<<<256, 256, 0, st>>>(s->x, s->v, s->n, h->partials);
             GB_CUDA(cudaGetLastError());
-            return finish_stats(h, 256, 0, out, st);
+            return finish_stats(h, StatsSink{}, 256, 0, out, st);
         }
         return GBRNG_OK;
     }
@@ -1152,7 +1152,7 @@ int lfg_ld(const ld_system* s, int64_t n_steps, int init, ld_stats* out, cudaStr
     }
     GB_CHECK(read_status(h, st));
     h->pos += a.n_pos;
-    if (out) return finish_stats(h, G, n_steps, out, st);
+    if (out) return finish_stats(h, StatsSink{}, G, n_steps, out, st);
     return GBRNG_OK;
 }
 

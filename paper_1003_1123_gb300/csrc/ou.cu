@@ -162,12 +162,18 @@ OuCoef make_ou_coef(const ou_system* s)
 int ou_finish(Handle* h, int64_t n, int64_t n_rec, int64_t blocks, double* mean, double* corr,
               cudaStream_t st)
 {
-    double* out = h->partials + 2 * n_rec * blocks;
+    // the records' sums straight into mapped host memory; more than fit there by a copy
+    const size_t bytes = sizeof(double) * 2 * (size_t)n_rec;
+    double* host = bytes <= kHostBlock ? (double*)host_block() : nullptr;
+    double* out = host ? host : h->partials + 2 * n_rec * blocks;
     ou_finish_kernel<<<(unsigned)n_rec, 256, 0, st>>>(h->partials, blocks, 1.0 / (double)n, out);
     GB_CUDA(cudaGetLastError());
-    std::vector<double> host(2 * (size_t)n_rec);
-    GB_CUDA(cudaMemcpyAsync(host.data(), out, sizeof(double) * 2 * n_rec, cudaMemcpyDeviceToHost,
-                            st));
+    std::vector<double> copy;
+    if (!host) {
+        copy.resize(2 * (size_t)n_rec);
+        host = copy.data();
+        GB_CUDA(cudaMemcpyAsync(host, out, bytes, cudaMemcpyDeviceToHost, st));
+    }
     GB_CUDA(cudaStreamSynchronize(st));
     for (int64_t r = 0; r < n_rec; ++r) {
         mean[r] = host[2 * r];

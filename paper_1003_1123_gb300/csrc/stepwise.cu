@@ -73,7 +73,7 @@ __global__ void __launch_bounds__(256) step_pt_kernel(StepArgs a)
 
 // Final-state sums and the oscillators' energy sums, per block.
 __global__ void step_stats_kernel(const float* x, const float* v, const float2* eacc, int64_t n,
-                                  double* partials)
+                                  StatsSink sink)
 {
     __shared__ double red[4 * 32];
     double acc[4] = {0, 0, 0, 0};
@@ -88,18 +88,18 @@ __global__ void step_stats_kernel(const float* x, const float* v, const float2* 
         acc[3] += (double)eacc[i].x - (double)eacc[i].y;
     }
     block_reduce_sum<4>(acc, red);
-    if (threadIdx.x == 0)
-        for (int k = 0; k < 4; ++k) partials[4 * blockIdx.x + k] = acc[k];
+    if (threadIdx.x < 32) store_stats(sink, acc);
 }
 
 int stepwise_stats(Handle* h, const ld_system* s, int64_t n_steps, ld_stats* out, cudaStream_t st)
 {
     if (!out) return GBRNG_OK;
     const int64_t blocks = 256;
-    GB_CHECK(ensure_partials(h, blocks));
-    step_stats_kernel<<<(unsigned)blocks, 256, 0, st>>>(s->x, s->v, h->eacc, s->n, h->partials);
+    StatsSink sink;
+    GB_CHECK(make_sink(h, blocks, true, &sink));
+    step_stats_kernel<<<(unsigned)blocks, 256, 0, st>>>(s->x, s->v, h->eacc, s->n, sink);
     GB_CUDA(cudaGetLastError());
-    return finish_stats(h, blocks, n_steps, out, st);
+    return finish_stats(h, sink, blocks, n_steps, out, st);
 }
 
 int ld_run_stepwise_pt(const ld_system* s, int64_t n_steps, ld_stats* out, cudaStream_t st)

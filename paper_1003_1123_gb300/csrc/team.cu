@@ -56,7 +56,8 @@ struct TeamArgs {
     int64_t every;      // OU: steps between records
     uint4* taus;
     uint32_t* lcg;
-    double* partials;   // LD: [gridDim.x][4]; OU: [record][gridDim.x][2]; or null
+    StatsSink sink;     // LD
+    double* records;    // OU: [record][gridDim.x][2] or null
 };
 
 // PAIRS: oscillator pairs of a block; M: producer warps a stage.
@@ -80,15 +81,6 @@ struct TeamShape {
     static constexpr int kThreads = 32 * (kStages * M + 1);
     static constexpr size_t kBufBytes = sizeof(float) * kChunks * kChunkWords;
 };
-
-// Sum over a warp's first LANES lanes (a power of two), in lane 0.
-template <int LANES = 32>
-__device__ __forceinline__ double warp_sum(double v)
-{
-#pragma unroll
-    for (int o = LANES / 2; o > 0; o >>= 1) v += __shfl_down_sync(0xffffffffu, v, o);
-    return v;
-}
 
 // The cosine-branch normals of one step of two particles (lane j = particle j),
 // each lane ou_run's transform.
@@ -172,7 +164,7 @@ __device__ __forceinline__ void team_produce(const TeamArgs& a, float* buf, int 
     if (chunk & 8) jump(std::integral_constant<uint64_t, 8 * D>{});
     if (S::kChunks > 16 && (chunk & 16)) jump(std::integral_constant<uint64_t, 16 * D>{});
     static_assert(S::kChunks == 16 || S::kChunks == 32, "jumps of the chunk number's bits");
-    const bool energies = MODEL == TEAM_LD && a.partials;
+    const bool energies = MODEL == TEAM_LD && a.sink.partials;
     const float2 cs = splat2(a.c.cs), cdt = splat2(a.c.cdt), cva = splat2(a.c.cva);
     float2 nck = {0.f, 0.f};
     if (energies) {
@@ -381,10 +373,8 @@ __device__ __forceinline__ void team_consume_ld(const TeamArgs& a, float* buf, i
     if (lane < 2 * G && ie < a.n)
         acc[3] = (double)(lane < G ? 0.5f * (a.Kper ? a.Kper[ie] : c.K) : c.hm) * K.value();
 #pragma unroll
-    for (int k = 0; k < 4; ++k) {
-        const double sum = warp_sum(acc[k]);
-        if (lane == 0) a.partials[4 * (int64_t)blockIdx.x + k] = sum;
-    }
+    for (int k = 0; k < 4; ++k) acc[k] = warp_sum(acc[k]);
+    store_stats(a.sink, acc);
 }
 
 // Consumer of the overdamped particles, a lane each; records between steps.
@@ -404,14 +394,14 @@ __device__ __forceinline__ void team_consume_ou(const TeamArgs& a, float* buf, i
         const double m = warp_sum<G>(live ? (double)Rt : 0.0);
         const double q = warp_sum<G>(live ? (double)Rt * (double)R0 : 0.0);
         if (lane == 0) {
-            double* o = a.partials + 2 * (rec * gridDim.x + blockIdx.x);
+            double* o = a.records + 2 * (rec * gridDim.x + blockIdx.x);
             o[0] = m;
             o[1] = q;
         }
         ++rec;
         next_rec += a.every;
     };
-    if (a.partials) record(R);
+    if (a.records) record(R);
     else next_rec = INT64_MAX;
     auto one = [&](const float* p) {
         R = __fmaf_rn(cs, *p, __fmaf_rn(-c1, R, R));
@@ -451,7 +441,7 @@ __global__ void __launch_bounds__(TeamShape<MODEL, PAIRS, M>::kThreads) team_ker
         team_produce<MODEL, KIND, S>(a, team_sm, kBarThreads);
     else if constexpr (MODEL == TEAM_OU)
         team_consume_ou<S>(a, team_sm, kBarThreads);
-    else if (a.partials)
+    else if (a.sink.partials)
         team_consume_ld<S, true>(a, team_sm, kBarThreads);
     else
         team_consume_ld<S, false>(a, team_sm, kBarThreads);
@@ -477,14 +467,13 @@ static bool team_of_8(int64_t n, int64_t n_steps, int sms)
     return n <= (int64_t)32 * sms || (n <= (int64_t)96 * sms && n_steps >= 512);
 }
 
-int ld_team(const ld_system* s, int64_t n_steps, bool want_stats, int64_t* blocks_out, cudaStream_t st)
+int ld_team(const ld_system* s, int64_t n_steps, ld_stats* out, cudaStream_t st)
 {
     Handle* h = s->rng;
     DevInfo di;
     GB_CHECK(dev_info(h->device, &di));
     const bool small = team_of_8(s->n, n_steps, di.sms);
     const int64_t blocks = (s->n + (small ? 7 : 15)) / (small ? 8 : 16);
-    if (want_stats) GB_CHECK(ensure_partials(h, blocks));
     TeamArgs a{};
     a.n = s->n;
     a.n_steps = n_steps;
@@ -494,11 +483,12 @@ int ld_team(const ld_system* s, int64_t n_steps, bool want_stats, int64_t* block
     a.c = make_coef(s);
     a.taus = h->taus;
     a.lcg = h->lcg;
-    a.partials = want_stats ? h->partials : nullptr;
-    *blocks_out = blocks;
+    GB_CHECK(make_sink(h, blocks, out != nullptr, &a.sink));
     if (h->kind == GBRNG_TAUS)
-        return small ? launch_team<TEAM_LD, GBRNG_TAUS, 4, 1>(a, st) : launch_team<TEAM_LD, GBRNG_TAUS, 8, 1>(a, st);
-    return small ? launch_team<TEAM_LD, GBRNG_LCG, 4, 1>(a, st) : launch_team<TEAM_LD, GBRNG_LCG, 8, 1>(a, st);
+        GB_CHECK((small ? launch_team<TEAM_LD, GBRNG_TAUS, 4, 1>(a, st) : launch_team<TEAM_LD, GBRNG_TAUS, 8, 1>(a, st)));
+    else
+        GB_CHECK((small ? launch_team<TEAM_LD, GBRNG_LCG, 4, 1>(a, st) : launch_team<TEAM_LD, GBRNG_LCG, 8, 1>(a, st)));
+    return finish_stats(h, a.sink, blocks, n_steps, out, st);
 }
 
 // Overdamped runs of at most 448 particles a SM (6.8e4: above, one particle a
@@ -525,7 +515,7 @@ int ou_team(const ou_system* s, int64_t n_steps, int64_t every, bool rec, int64_
     a.every = every;
     a.taus = h->taus;
     a.lcg = h->lcg;
-    a.partials = rec ? h->partials : nullptr;
+    a.records = rec ? h->partials : nullptr;
     *blocks_out = blocks;
     if (h->kind == GBRNG_TAUS)
         GB_CHECK((small ? launch_team<TEAM_OU, GBRNG_TAUS, 4, 1>(a, st) : launch_team<TEAM_OU, GBRNG_TAUS, 8, 1>(a, st)));

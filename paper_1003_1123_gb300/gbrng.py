@@ -120,9 +120,16 @@ def _check(rc: int):
         raise GbrngError(rc, gbrng_last_error())
 
 
+def _current_stream() -> int:
+    """torch's current stream of the current device, as current_stream().cuda_stream gives it but without
+    building a Stream object (3 us a call)."""
+    torch.cuda.init()
+    return torch._C._cuda_getCurrentRawStream(torch._C._cuda_getDevice())
+
+
 def _stream(stream):
     if stream is None:
-        return C.c_void_p(torch.cuda.current_stream().cuda_stream)
+        return C.c_void_p(_current_stream())
     if isinstance(stream, torch.cuda.Stream):
         return C.c_void_p(stream.cuda_stream)
     return C.c_void_p(int(stream))
