@@ -19,7 +19,7 @@ INCLUDE = os.path.join(ROOT, "include")
 BUILD = os.path.join(HERE, "_build")
 LIB = os.path.join(HERE, "libgbrng.so")
 
-SOURCES = ["runtime.cu", "fill.cu", "ld.cu", "team.cu", "lfg.cu", "batched.cu", "adjoint.cu", "noalloc.cu",
+SOURCES = ["runtime.cu", "fill.cu", "ld.cu", "team.cu", "lfg.cu", "lfg_run.cu", "lfg_ou.cu", "lfg_team.cu", "batched.cu", "adjoint.cu", "noalloc.cu",
            "stepwise.cu", "ou.cu"]
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 FLAGS = ARCH + ["-O3", "-lineinfo", "-std=c++17", "-Xcompiler", "-fPIC", "-I", INCLUDE,

@@ -53,20 +53,19 @@ struct Handle {
     int32_t* r2 = nullptr;     // [35][n]: idum, idum2, iy, iv[0..31]
     uint32_t* lcg = nullptr;   // [n] Quick and Dirty LCG words
 
-    // Lagged Fibonacci: the sequence value at position p (p >= -order_max ll)
-    // lives in ring[p mod ring_size]; ring_size >= order_max (ll + (ll - sl)),
-    // where order_max (2 or 4) is the highest leap order the ring serves.  The
-    // allocation holds ring_size + ring_mirror(ring_size) words: the ring,
-    // then a copy of its first ring_mirror(ring_size) slots.
+    // Lagged Fibonacci: the sequence value at position p lives in
+    // ring[p mod ring_size], those of the last lfg_history() positions before pos
+    // always.  depth: the deepest fan the ring serves; order_max (2 or 4): the
+    // highest order a paper-form or overdamped step may need (lfg.cuh).
     int row = -1;
     int32_t sl = 0, ll = 0;
-    int order_max = 2;
+    int order_max = 2, depth = 0;
     uint32_t ring_size = 0;
     uint32_t* ring = nullptr;
     int64_t pos = 0;           // next position to generate
 
     // scratch owned by the handle
-    uint64_t* progress = nullptr;   // grid-barrier arrival counter (LFG)
+    uint64_t* progress = nullptr;   // grid-barrier arrival counter, status (LFG)
     int64_t progress_cap = 0;
     int* dstatus = nullptr;         // device status word, then the statistics' ticket
     double* partials = nullptr;     // per-block reduction partials
@@ -77,15 +76,8 @@ struct Handle {
     size_t adj_bytes = 0;
 };
 
-// Mirrored slots after a Lagged Fibonacci ring of R slots: 32768 (a resident
-// CTA's step region at 1e6 oscillators is 26368), at most a quarter of the
-// ring (so that small rings do not store every value twice), a multiple of
-// 32 (R >= 6620 for every Table I row, so never below 1632 >= one block).
-inline uint32_t ring_mirror(uint32_t R)
-{
-    const uint32_t q = (R / 4) & ~31u;
-    return q < 32768u ? q : 32768u;
-}
+// Positions before the next one that a handle's ring holds: D + depth sl.
+inline int64_t lfg_history(const Handle* h) { return (int64_t)h->ll - h->sl + (int64_t)h->depth * h->sl; }
 
 // Device attributes used for launch sizing (cached per device).
 struct DevInfo {
@@ -120,7 +112,7 @@ int ld_team(const ld_system* s, int64_t n_steps, ld_stats* out, cudaStream_t st)
 
 // Lagged Fibonacci entry points (lfg.cu)
 int lfg_seed(Handle* h, cudaStream_t st);
-int lfg_order_for_new_handle();   // highest leap order a new handle's ring serves
+void lfg_new_handle(Handle* h);   // order_max, depth and ring_size of a new handle
 int lfg_fill(Handle* h, void* dst, int64_t n, int mode, cudaStream_t st);  // mode 0 u32, 1 uniform, 2 normal
 int lfg_ld(const ld_system* s, int64_t n_steps, int init, ld_stats* out, cudaStream_t st);
 

@@ -213,17 +213,8 @@ static int alloc_state(Handle* h)
     } else if (h->kind == GBRNG_LCG) {
         e = cudaMalloc(&h->lcg, sizeof(uint32_t) * h->n);
     } else {
-        // ring size: k (ll + D) rounded up to 32 words for the highest leap
-        // order k the ring serves (2 unless order 4 was set before creation).
-        // The order-k leap reads back to p - k ll, and a round of W <= k D
-        // positions overwrites positions p - R, so R - k ll >= k D lets every
-        // round take its full width (the seeds' backward extension fills
-        // positions -k ll .. -1).
-        h->order_max = lfg_order_for_new_handle();
-        const uint64_t D = (uint64_t)(h->ll - h->sl);
-        const uint64_t R = ((uint64_t)h->order_max * ((uint64_t)h->ll + D) + 31) & ~(uint64_t)31;
-        h->ring_size = (uint32_t)R;
-        e = cudaMalloc(&h->ring, sizeof(uint32_t) * (R + ring_mirror(h->ring_size)));
+        if (h->depth == 0) lfg_new_handle(h);   // a clone has its source's ring
+        e = cudaMalloc(&h->ring, sizeof(uint32_t) * h->ring_size);
     }
     if (e == cudaSuccess) e = cudaMalloc(&h->dstatus, sizeof(int) * 2);
     if (e != cudaSuccess) {
@@ -449,6 +440,9 @@ int rng_clone(gbrng_t src, gbrng_t* out, void* stream)
     h->row = src->row;
     h->sl = src->sl;
     h->ll = src->ll;
+    h->order_max = src->order_max;
+    h->depth = src->depth;
+    h->ring_size = src->ring_size;
     h->pos = src->pos;
     int rc = alloc_state(h);
     if (rc != GBRNG_OK) {
@@ -465,9 +459,7 @@ int rng_clone(gbrng_t src, gbrng_t* out, void* stream)
     else if (h->kind == GBRNG_LCG)
         e = cudaMemcpyAsync(h->lcg, src->lcg, sizeof(uint32_t) * h->n, cudaMemcpyDeviceToDevice, st);
     else
-        e = cudaMemcpyAsync(h->ring, src->ring,
-                            sizeof(uint32_t) * ((size_t)h->ring_size + ring_mirror(h->ring_size)),
-                            cudaMemcpyDeviceToDevice, st);
+        e = cudaMemcpyAsync(h->ring, src->ring, sizeof(uint32_t) * h->ring_size, cudaMemcpyDeviceToDevice, st);
     if (e != cudaSuccess) {
         free_handle(h);
         return fail(GBRNG_ECUDA, "clone copy failed: %s", cudaGetErrorString(e));
@@ -531,14 +523,13 @@ int rng_get_state(gbrng_t rng, void* host, size_t bytes)
         for (int64_t s = 0; s < rng->n; ++s)
             for (int k = 0; k < 35; ++k) o[35 * s + k] = tmp[(size_t)k * rng->n + s];
     } else {
-        const int64_t R = rng->ring_size;
-        std::vector<uint32_t> ring(R);
-        GB_CUDA(cudaMemcpy(ring.data(), rng->ring, sizeof(uint32_t) * R, cudaMemcpyDeviceToHost));
-        uint32_t* o = (uint32_t*)dst;
-        for (int64_t k = 0; k < rng->ll; ++k) {
-            const int64_t r = (rng->pos - rng->ll + k) % R;
-            o[k] = ring[r < 0 ? r + R : r];
-        }
+        // the last ll values, in two pieces where they wrap
+        const int64_t R = rng->ring_size, ll = rng->ll;
+        const int64_t at = ((rng->pos - ll) % R + R) % R, first = ll < R - at ? ll : R - at;
+        GB_CUDA(cudaMemcpy(dst, rng->ring + at, sizeof(uint32_t) * first, cudaMemcpyDeviceToHost));
+        if (first < ll)
+            GB_CUDA(cudaMemcpy(dst + sizeof(uint32_t) * first, rng->ring, sizeof(uint32_t) * (ll - first),
+                               cudaMemcpyDeviceToHost));
     }
     return GBRNG_OK;
 }
@@ -569,26 +560,19 @@ int rng_set_state(gbrng_t rng, const void* host, size_t bytes)
             for (int k = 0; k < 35; ++k) tmp[(size_t)k * rng->n + s] = in[35 * s + k];
         GB_CUDA(cudaMemcpy(rng->r2, tmp.data(), pb, cudaMemcpyHostToDevice));
     } else {
-        // The blob holds x_{p-ll} .. x_{p-1}.  The leap forms of the recurrence
-        // also read x_{p-k ll} .. x_{p-ll-1} (k = the ring's highest order);
-        // they follow from the recurrence run backwards, x_q = x_{q+ll} -
-        // x_{q+sl}, which keeps the recurrence true at every index the leaps use.
-        const int64_t R = rng->ring_size;
-        const int64_t ll = rng->ll, sl = rng->sl, p = hd.position, k = rng->order_max;
-        std::vector<uint32_t> hist((size_t)k * ll);          // hist[j] = x_{p-k ll+j}
-        const uint32_t* in = (const uint32_t*)src;
-        for (int64_t i = 0; i < ll; ++i) hist[(k - 1) * ll + i] = in[i];
-        for (int64_t j = (k - 1) * ll - 1; j >= 0; --j) hist[j] = hist[j + ll] - hist[j + sl];
-        const int64_t M = ring_mirror(rng->ring_size);
-        std::vector<uint32_t> ring(R + M, 0u);
-        for (int64_t j = 0; j < k * ll; ++j) {
-            int64_t r = (p - k * ll + j) % R;
-            if (r < 0) r += R;
-            ring[r] = hist[j];
-            if (r < M) ring[r + R] = hist[j];
-        }
-        GB_CUDA(cudaMemcpy(rng->ring, ring.data(), sizeof(uint32_t) * (R + M),
-                           cudaMemcpyHostToDevice));
+        // The blob holds x_{p-ll} .. x_{p-1}.  The fans also read x_{p-H} ..
+        // x_{p-ll-1}; they follow from the recurrence run backwards, x_q = x_{q+ll} -
+        // x_{q+sl}, which keeps the recurrence true at every index the fans use.
+        const int64_t R = rng->ring_size, H = lfg_history(rng);
+        const int64_t ll = rng->ll, sl = rng->sl, p = hd.position;
+        std::vector<uint32_t> hist((size_t)H);               // hist[j] = x_{p-H+j}
+        memcpy(hist.data() + (H - ll), src, pb);
+        for (int64_t j = H - ll - 1; j >= 0; --j) hist[j] = hist[j + ll] - hist[j + sl];
+        // into the ring, in two pieces where it wraps
+        const int64_t at = ((p - H) % R + R) % R, first = H < R - at ? H : R - at;
+        GB_CUDA(cudaMemcpy(rng->ring + at, hist.data(), sizeof(uint32_t) * first, cudaMemcpyHostToDevice));
+        if (first < H)
+            GB_CUDA(cudaMemcpy(rng->ring, hist.data() + first, sizeof(uint32_t) * (H - first), cudaMemcpyHostToDevice));
         rng->pos = hd.position;
     }
     return GBRNG_OK;

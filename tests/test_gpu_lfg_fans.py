@@ -1,0 +1,121 @@
+"""The Lagged Fibonacci kernels that generate the sequence in fans, at the edges of
+their launch rules, against the paper form (one launch a step, every word from its
+own lag reads) and against the same work in pieces: same bits."""
+import numpy as np
+import pytest
+import torch
+
+from paper_1003_1123_gb300 import workloads as W
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def G():
+    if not torch.cuda.is_available():
+        pytest.skip("needs a CUDA GPU")
+    from paper_1003_1123_gb300 import gbrng
+    gbrng.lib()
+    yield gbrng
+    gbrng.gbrng_set_lfg_order(0)
+
+
+def system(G, n, row, skip):
+    r = G.rng_init_lfg(29, n, row)
+    if skip:
+        G.rng_fill_u32(r, skip)
+    x, v = W.initial_state(n, 3)
+    return G.LdSystem(r, torch.from_numpy(x).cuda(), torch.from_numpy(v).cuda(),
+                      K_per=torch.from_numpy(W.spring_constants(n, n)).cuda())
+
+
+@pytest.mark.parametrize("order", [0, 1, 2])
+@pytest.mark.parametrize("skip", [0, 1, 6])
+@pytest.mark.parametrize("n,row,steps", [
+    (1, 0, 9), (2, 2, 40), (777, 2, 37),     # small systems' kernel, odd N, slots off a multiple of 4
+    (400, 0, 7), (401, 0, 7), (402, 0, 7),   # order 1: rounds of half a step, x and v through global memory
+    (24320, -1, 45), (24321, -1, 45),        # the last N of the small systems' kernel, the next one's
+    (70001, -1, 30),                         # x and v in shared memory, several steps a round
+])
+def test_runs_equal_paper_form(G, n, row, steps, skip, order):
+    try:
+        G.gbrng_set_lfg_order(order)
+        a = system(G, n, row, skip)
+        st = G.ld_run(a, steps)
+        G.gbrng_set_lfg_order(0)
+        b = system(G, n, row, skip)
+        sb = G.ld_run_stepwise(b, steps)
+    finally:
+        G.gbrng_set_lfg_order(0)
+    assert torch.equal(a.x, b.x) and torch.equal(a.v, b.v)
+    assert G.rng_get_state(a.rng) == G.rng_get_state(b.rng)
+    assert abs(st["sum_v2"] / sb["sum_v2"] - 1) < 1e-12          # binary64 sums
+    assert abs(st["energy_time_avg"] / sb["energy_time_avg"] - 1) < 1e-6   # compensated binary32 sums
+
+
+@pytest.mark.parametrize("n,row", [(1, 0), (9, 2), (2000, 3), (2001, 3), (38000, -1), (38001, -1)])
+def test_overdamped_equals_single_steps(G, n, row):
+    """A run of many steps a round against one step a call, at both record cadences a
+    round can see; orders 0 (small systems' kernel) and 2 (few steps a round)."""
+    kw = dict(k_sp=0.01, xi=1.0, kT=4.1, dt=1.0)
+    R0 = torch.linspace(-3, 4, n, device="cuda")
+    steps = 61
+    b = G.OuSystem(G.rng_init_lfg(7, n, row), R0.clone(), **kw)
+    Rs = [R0.double()]
+    for _ in range(steps):
+        G.ou_run(b, 1)
+        Rs.append(b.R.double())
+    for order in (0, 2):
+        try:
+            G.gbrng_set_lfg_order(order)
+            for every in (1, 7):
+                a = G.OuSystem(G.rng_init_lfg(7, n, row), R0.clone(), **kw)
+                mean, corr = G.ou_run(a, steps, every)
+                assert torch.equal(a.R, b.R)
+                assert G.rng_get_state(a.rng) == G.rng_get_state(b.rng)
+                assert np.allclose(mean, [r.mean().item() for r in Rs[::every]], rtol=0, atol=1e-12)
+                assert np.allclose(corr, [(r * Rs[0]).mean().item() for r in Rs[::every]], rtol=0, atol=1e-11)
+        finally:
+            G.gbrng_set_lfg_order(0)
+
+
+@pytest.mark.parametrize("row", list(range(10)))
+@pytest.mark.parametrize("skip", [0, 3])
+def test_normals_are_the_transform_of_the_words(G, row, skip):
+    """A normal fill over several rounds against the FP64 transform of the same words
+    from a u32 fill: pairs across fans, units and CTAs."""
+    sl, ll = G.rng_lfg_lags(row)
+    n = min(40 * (ll - sl), 9 * 10**6) // 2 * 2
+    r, q = G.rng_init_lfg(5, 100, row), G.rng_init_lfg(5, 100, row)
+    if skip:
+        G.rng_fill_u32(r, skip)
+        G.rng_fill_u32(q, skip)
+    got = G.rng_fill_normal(r, n).double()
+    w = G.rng_fill_u32(q, n).to(torch.int64) & 0xFFFFFFFF
+    assert G.rng_get_state(r) == G.rng_get_state(q)
+    u = ((w >> 9).double() + 0.5) * 2.0**-23
+    rho, phi = torch.sqrt(-2 * torch.log(u[0::2])), 2 * np.pi * u[1::2]
+    for o, e in ((0, rho * torch.cos(phi)), (1, rho * torch.sin(phi))):
+        # 4 ulp (ln 0.8, sin and cos 1.9, the root 1) and the absolute error at the zeros
+        assert bool((torch.abs(got[o::2] - e) <= 4 * 2.0**-23 * torch.abs(e) + 1e-7 * (1 + rho)).all())
+
+
+def test_small_system_timeout(G):
+    """A CTA that never arrives at the grid barrier ends the small systems' kernel with
+    GBRNG_ETIMEOUT; the handle works again after a state is set."""
+    n = 10**4
+    s = system(G, n, -1, 0)
+    blob = G.rng_get_state(s.rng)
+    G.rng_set_wait_limit_ns(200_000_000)
+    G.gbrng_test_stall_chunk(3)
+    try:
+        with pytest.raises(G.GbrngError) as e:
+            G.ld_run(s, 200)
+        assert e.value.code == -4
+    finally:
+        G.gbrng_test_stall_chunk(-1)
+        G.rng_set_wait_limit_ns(2_000_000_000)
+    G.rng_set_state(s.rng, blob)
+    st = G.ld_run(s, 100)
+    xx = (s.x.double() ** 2).sum().item()
+    assert abs(st["sum_x2"] / xx - 1) < 1e-12
