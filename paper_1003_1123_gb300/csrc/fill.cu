@@ -1,9 +1,12 @@
-// Stand-alone fills for the per-thread generators (Hybrid Taus, Ran2):
+// Stand-alone fills for the per-thread generators (Hybrid Taus, the LCG, Ran2):
 // out[d*S + s] is the d-th draw of stream s.  One thread owns one stream at a
-// time and keeps its state in registers (Taus) or in a shared-memory column
-// (Ran2's shuffle table) for all of its draws; stores are coalesced across
-// the streams of a warp.
-#include "device.cuh"
+// time and keeps its state in registers (Taus, the LCG) or in a shared-memory
+// column (Ran2's shuffle table) for all of its draws, or, where the streams are
+// few, a segment of a stream's draws; stores are coalesced across the streams of
+// a warp.
+#include <algorithm>
+
+#include "jump.cuh"
 #include "internal.cuh"
 
 namespace gb {
@@ -26,7 +29,34 @@ __device__ __forceinline__ void emit_word(State& y, int64_t idx, void* out)
     }
 }
 
-// n_items = numbers (u32, uniform) or pairs (normal).
+// n_items = numbers (u32, uniform) or pairs (normal); the items idx, idx + S, ... <
+// end of one word chain.
+template <int MODE, class State>
+__device__ __forceinline__ void emit_chain(State& y, int64_t idx, int64_t S, int64_t end, void* out)
+{
+    // four draws in flight per iteration: independent stores, one state chain
+    for (; idx + 3 * S < end; idx += 4 * S) {
+        if (MODE == FILL_NORMAL) {
+            // the four pairs two at a time in the paired instructions' lanes
+            uint32_t r[8];
+#pragma unroll
+            for (int q = 0; q < 8; ++q) r[q] = next_word(y);
+            float2* o = (float2*)out;
+            float2 ga, gb;
+            box_muller_2pairs_u32(r[0], r[1], r[2], r[3], ga, gb);
+            o[idx] = ga, o[idx + S] = gb;
+            box_muller_2pairs_u32(r[4], r[5], r[6], r[7], ga, gb);
+            o[idx + 2 * S] = ga, o[idx + 3 * S] = gb;
+        } else {
+            emit_word<MODE>(y, idx, out);
+            emit_word<MODE>(y, idx + S, out);
+            emit_word<MODE>(y, idx + 2 * S, out);
+            emit_word<MODE>(y, idx + 3 * S, out);
+        }
+    }
+    for (; idx < end; idx += S) emit_word<MODE>(y, idx, out);
+}
+
 // Hybrid Taus (uint4 state) and the LCG (uint32 state): one word chain per stream.
 template <int MODE, class State>
 __global__ void __launch_bounds__(256) word_fill_kernel(State* __restrict__ st, int64_t S,
@@ -36,30 +66,51 @@ __global__ void __launch_bounds__(256) word_fill_kernel(State* __restrict__ st, 
     const int64_t stride = (int64_t)gridDim.x * blockDim.x;
     for (int64_t s = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; s < active; s += stride) {
         State y = st[s];
-        int64_t idx = s;
-        // four draws in flight per iteration: independent stores, one state chain
-        for (; idx + 3 * S < n_items; idx += 4 * S) {
-            if (MODE == FILL_NORMAL) {
-                // the four pairs two at a time in the paired instructions' lanes
-                uint32_t r[8];
-#pragma unroll
-                for (int q = 0; q < 8; ++q) r[q] = next_word(y);
-                float2* o = (float2*)out;
-                float2 ga, gb;
-                box_muller_2pairs_u32(r[0], r[1], r[2], r[3], ga, gb);
-                o[idx] = ga, o[idx + S] = gb;
-                box_muller_2pairs_u32(r[4], r[5], r[6], r[7], ga, gb);
-                o[idx + 2 * S] = ga, o[idx + 3 * S] = gb;
-            } else {
-                emit_word<MODE>(y, idx, out);
-                emit_word<MODE>(y, idx + S, out);
-                emit_word<MODE>(y, idx + 2 * S, out);
-                emit_word<MODE>(y, idx + 3 * S, out);
-            }
-        }
-        for (; idx < n_items; idx += S) emit_word<MODE>(y, idx, out);
+        emit_chain<MODE>(y, s, S, n_items, out);
         st[s] = y;
     }
+}
+
+// Few streams: one chain a stream leaves most of the GPU idle (a draw is about 25
+// cycles of latency), so a stream's items are cut into segments of L, each thread's
+// generator jumped ahead to its segment (jump.cuh: the same words as stepping
+// there).  All segments of a group of B streams are in one cluster of blocks, so
+// that the states are read, by the cluster's barrier, before any thread replaces
+// one; clusters keep B, the streams that a row of stores covers, at least 32 (2^27
+// uniforms of 4096 streams: 434 us with 16 in one block, 148 with 32, 181 with 64 and
+// twice the blocks a cluster).  One thread a stream / segments, us: 2^20 words of
+// 4096 streams 12.4 / 6.3; 2^24 uniforms of 1024 559 / 22.7; 2^27 of 4096 1118 / 148,
+// of 2e4 233 / 173, of 5e4 176 / 140; 2^27 normals of 4096 1868 / 208.  (From 7e4
+// streams on a thread a stream is faster: 115 against 123 us.)
+constexpr int kSplitThreads = 512, kSplitMax = 64, kSplitRow = 32;
+struct SplitArgs {
+    Jump lo[8], hi[kSplitMax / 8];   // g L items ahead for g = 0 .. 7, and 8g L
+    int64_t L;
+    int B;                           // streams of a cluster; kSplitThreads / B segments a block
+};
+
+template <int MODE, class State>
+__global__ void __launch_bounds__(kSplitThreads) word_split_kernel(State* st, int64_t S, int64_t n_items,
+                                                                   void* __restrict__ out,
+                                                                   const __grid_constant__ SplitArgs a)
+{
+    uint32_t rank, blocks;   // of the cluster
+    asm("mov.u32 %0, %%cluster_ctarank;" : "=r"(rank));
+    asm("mov.u32 %0, %%cluster_nctarank;" : "=r"(blocks));
+    const int64_t s = blockIdx.x / blocks * (int64_t)a.B + threadIdx.x % a.B;
+    const int g = (int)rank * (kSplitThreads / a.B) + threadIdx.x / a.B;
+    const int64_t first = s + g * a.L * S, end = min(n_items, first + a.L * S);
+    const bool live = s < S && first < n_items;
+    State y;
+    if (live) {
+        y = st[s];
+        if (g & 7) jump_ahead(y, a.lo[g & 7]);
+        if (g >> 3) jump_ahead(y, a.hi[g >> 3]);
+    }
+    asm volatile("barrier.cluster.arrive.aligned;\nbarrier.cluster.wait.aligned;" ::: "memory");
+    if (!live) return;
+    emit_chain<MODE>(y, first, S, end, out);
+    if (first + ((end - first - 1) / S) * S + S >= n_items) st[s] = y;   // the stream's last item
 }
 
 template <int MODE>
@@ -118,6 +169,43 @@ __global__ void __launch_bounds__(128) ran2_fill_kernel(int32_t* __restrict__ st
     }
 }
 
+// Segments for at most 400 streams a SM: powers of two that bring the threads to
+// about 1024 a SM, of at least 32 items (a jump costs a thread about as much as 15
+// draws).  Returns 1 when it has launched, 0 for one thread a stream, or an error.
+template <int MODE, class State>
+static int fill_split(Handle* h, State* states, void* dst, int64_t n_items, cudaStream_t st)
+{
+    const int64_t S = h->n, items = (n_items + S - 1) / S;   // of the longest chain
+    DevInfo di;
+    GB_CHECK(dev_info(h->device, &di));
+    int Q = 1;
+    while (S <= (int64_t)di.sms * 400 && Q < kSplitMax && S * Q < (int64_t)di.sms * 1024 && items / (2 * Q) >= 32) Q *= 2;
+    if (Q < 2) return 0;
+    const int C = std::max(1, Q * kSplitRow / kSplitThreads);   // blocks of a cluster
+    SplitArgs a;
+    a.B = kSplitThreads * C / Q;
+    a.L = (items + Q - 1) / Q;
+    const Jump one = jump_of((uint64_t)a.L * (MODE == FILL_NORMAL ? 2 : 1));
+    a.lo[0] = a.hi[0] = jump_of(0);
+    for (int g = 1; g < 8 && g < Q; ++g) a.lo[g] = jump_sum(a.lo[g - 1], one);
+    if (Q > 8) {
+        const Jump eight = jump_sum(a.lo[7], one);
+        for (int g = 1; g < Q / 8; ++g) a.hi[g] = jump_sum(a.hi[g - 1], eight);
+    }
+    cudaLaunchAttribute attr;
+    attr.id = cudaLaunchAttributeClusterDimension;
+    attr.val.clusterDim.x = (unsigned)C;
+    attr.val.clusterDim.y = attr.val.clusterDim.z = 1;
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = dim3((unsigned)((S + a.B - 1) / a.B * C));
+    cfg.blockDim = dim3(kSplitThreads);
+    cfg.stream = st;
+    cfg.attrs = &attr;
+    cfg.numAttrs = 1;
+    GB_CUDA(cudaLaunchKernelEx(&cfg, word_split_kernel<MODE, State>, states, S, n_items, dst, a));
+    return 1;
+}
+
 // Grid: one thread per stream (up to the streams a fill touches), in as many
 // waves as that takes, rather than one resident wave looping over streams:
 // the blocks then start, and load their streams' state, at staggered times
@@ -130,6 +218,9 @@ static int fill_pt(Handle* h, void* dst, int64_t n_items, cudaStream_t st)
 {
     const int64_t active = h->n < n_items ? h->n : n_items;
     if (h->kind == GBRNG_TAUS || h->kind == GBRNG_LCG) {
+        const int rc = h->kind == GBRNG_TAUS ? fill_split<MODE>(h, h->taus, dst, n_items, st)
+                                             : fill_split<MODE>(h, h->lcg, dst, n_items, st);
+        if (rc) return rc < 0 ? rc : GBRNG_OK;
         const int T = 256;
         const int64_t blocks = (active + T - 1) / T;
         if (h->kind == GBRNG_TAUS)

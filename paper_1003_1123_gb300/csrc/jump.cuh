@@ -23,29 +23,36 @@
 namespace gb {
 
 // x^m mod x^k + x^q + 1 over GF(2); bit i is the coefficient of x^i.
-__host__ __device__ constexpr uint64_t gf2_mulmod(uint64_t u, uint64_t v, int k, int q)
+__host__ __device__ constexpr uint32_t gf2_mulmod(uint32_t u, uint32_t v, int k, int q)
 {
     uint64_t p = 0;   // degree at most 2k - 2 <= 60
-    for (int i = 0; i < k; ++i)
-        if ((v >> i) & 1) p ^= u << i;
-    for (int i = 2 * k - 2; i >= k; --i)
-        if ((p >> i) & 1) p ^= (1ull << i) | (1ull << (i - k)) | (1ull << (i - k + q));
-    return p;
+    for (; v; v &= v - 1) {
+        const uint32_t low = v & (0u - v);
+        p ^= (uint64_t)u * low;   // u x^i
+    }
+    // x^{k+i} = x^{q+i} + x^i, twice: the first leaves a degree of at most k - 2 + q
+    const uint64_t mask = (1ull << k) - 1;
+    for (int r = 0; r < 2; ++r) {
+        const uint64_t h = p >> k;
+        p = (p & mask) ^ h ^ (h << q);
+    }
+    return (uint32_t)p;
 }
 
 __host__ __device__ constexpr uint32_t gf2_xpow(uint64_t m, int k, int q)
 {
-    uint64_t r = 1, b = 2;
+    uint32_t r = 1, b = 2;
     for (; m; m >>= 1) {
         if (m & 1) r = gf2_mulmod(r, b, k, q);
         b = gf2_mulmod(b, b, k, q);
     }
-    return (uint32_t)r;
+    return r;
 }
 
-// One word, moved on by the polynomial's number of bits.
-template <int K, int Q, uint32_t POLY>
-__device__ __forceinline__ uint32_t taus_word_jump(uint32_t y)
+// One word, moved on by the number of bits of the polynomial (a constant after
+// inlining, or not).
+template <int K, int Q>
+__device__ __forceinline__ uint32_t taus_word_jump(uint32_t y, uint32_t poly)
 {
     // bits b_n .. b_{n+63} from the K highest of y: the first application is
     // right up to bit 2K - Q - 1, which the second reads no further than
@@ -56,8 +63,7 @@ __device__ __forceinline__ uint32_t taus_word_jump(uint32_t y)
     const uint32_t hi = (uint32_t)(u >> 32), lo = (uint32_t)u;
     uint32_t r = 0;
 #pragma unroll
-    for (int i = 0; i < K; ++i)
-        if ((POLY >> i) & 1) r ^= __funnelshift_l(lo, hi, i);
+    for (int i = 0; i < K; ++i) r ^= __funnelshift_l(lo, hi, i) & (0u - ((poly >> i) & 1u));
     return r;
 }
 
@@ -86,10 +92,38 @@ template <uint64_t D>
 __device__ __forceinline__ void jump_ahead(uint4& y)
 {
     constexpr uint32_t p1 = gf2_xpow(12 * D, 31, 13), p2 = gf2_xpow(4 * D, 29, 2), p3 = gf2_xpow(17 * D, 28, 3);
-    y.x = taus_word_jump<31, 13, p1>(y.x);
-    y.y = taus_word_jump<29, 2, p2>(y.y);
-    y.z = taus_word_jump<28, 3, p3>(y.z);
+    y.x = taus_word_jump<31, 13>(y.x, p1);
+    y.y = taus_word_jump<29, 2>(y.y, p2);
+    y.z = taus_word_jump<28, 3>(y.z, p3);
     jump_ahead<D>(y.w);
+}
+
+// A jump whose distance is known at run time.
+struct Jump {
+    uint32_t p[3];   // the Tausworthe words' polynomials
+    LcgJump l;
+};
+
+inline Jump jump_of(uint64_t d)
+{
+    return Jump{{gf2_xpow(12 * d, 31, 13), gf2_xpow(4 * d, 29, 2), gf2_xpow(17 * d, 28, 3)}, lcg_jump(d)};
+}
+
+// The jump by both distances.
+inline Jump jump_sum(const Jump& a, const Jump& b)
+{
+    return Jump{{gf2_mulmod(a.p[0], b.p[0], 31, 13), gf2_mulmod(a.p[1], b.p[1], 29, 2),
+                 gf2_mulmod(a.p[2], b.p[2], 28, 3)},
+                LcgJump{a.l.a * b.l.a, a.l.a * b.l.c + a.l.c}};
+}
+
+__device__ __forceinline__ void jump_ahead(uint32_t& x, const Jump& j) { x = j.l.a * x + j.l.c; }
+__device__ __forceinline__ void jump_ahead(uint4& y, const Jump& j)
+{
+    y.x = taus_word_jump<31, 13>(y.x, j.p[0]);
+    y.y = taus_word_jump<29, 2>(y.y, j.p[1]);
+    y.z = taus_word_jump<28, 3>(y.z, j.p[2]);
+    jump_ahead(y.w, j);
 }
 
 }  // namespace gb
