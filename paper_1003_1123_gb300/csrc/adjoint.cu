@@ -43,20 +43,41 @@ struct AdjArgs {
     int32_t* r2;
     int64_t streams;
     float* ckpt;        // [nseg][6 + state words][n]
-    float* gbuf;        // [S][3][n] history (hist) or [P][3][n] segment scratch
-    int hist;
+    float* gbuf;        // [S][3][n] the run's noise, or [P][3][n] a segment's
     float* dK;          // [n] or null
     StatsSink sink;     // loss, dgamma, dkT, unused
 };
 
-// 64-thread blocks with an 85-register budget: twelve blocks per SM (116736
-// threads on 152 SMs), so 1e5 oscillators fit one resident wave with one
-// oscillator per thread and the SMs differ by at most one block; 1% faster
-// than fourteen blocks at 72 registers (at 96 registers and 128 threads the
-// same system needed two oscillators per thread on 2.6 blocks per SM).
-template <int KIND>
-__global__ void __launch_bounds__(64, 12) adjoint_kernel(AdjArgs a)
+// Two compensated binary32 sums in the lanes of the paired instructions.
+struct KahanPair {
+    float2 s = {0.f, 0.f}, c = {0.f, 0.f};
+    __device__ __forceinline__ void add(float a, float b)
+    {
+        const float2 y = __fadd2_rn(make_float2(a, b), make_float2(-c.x, -c.y));
+        const float2 t = __fadd2_rn(s, y);
+        c = __fadd2_rn(__fadd2_rn(t, make_float2(-s.x, -s.y)), make_float2(-y.x, -y.y));
+        s = t;
+    }
+    __device__ __forceinline__ double first() const { return (double)s.x - (double)c.x; }
+    __device__ __forceinline__ double second() const { return (double)s.y - (double)c.y; }
+};
+
+// Where the reverse sweep's normals come from: regenerated segment by segment, or
+// kept by the forward run.
+enum { NOISE_REGEN = 0, NOISE_KEPT = 1 };
+
+// The reverse sweep is bound by the latency of its loads where the noise is kept
+// (one step's three normals at a time, 12 B from memory): with the next eight
+// steps' loads in flight and up to 128 registers, 64-thread blocks, eight a SM, 1e5
+// oscillators x 1000 steps take 1.09 ms for Hybrid Taus (1.55 with no load ahead;
+// twelve blocks at 85 registers: 1.48 with one step ahead, 1.25 with three, 1.13
+// with four, 1.17 with eight), 1.20 for Ran2 (1.75); 1e4 x 1000 0.27 (0.62).
+// Regenerated noise comes back from L2 and needs two.  Components 0 and 2 and the
+// compensated sums run in the lanes of the paired instructions.
+template <int KIND, int NOISE>
+__global__ void __launch_bounds__(64, 8) adjoint_kernel(AdjArgs a)
 {
+    constexpr int kAhead = NOISE == NOISE_REGEN ? 2 : 8;   // steps whose normals are loaded ahead
     extern __shared__ int32_t tab[];   // Ran2: [32][blockDim.x]
     __shared__ double red[4 * 32];
     constexpr int SW = KIND == GBRNG_TAUS ? 4 : 35;   // state words
@@ -121,33 +142,33 @@ __global__ void __launch_bounds__(64, 12) adjoint_kernel(AdjArgs a)
             }
         };
         // ---------------- A: forward with checkpoints
+        // components 0 and 2 in the lanes of the paired instructions (as the transform
+        // leaves their normals), component 1 by itself
         load_state(nullptr, 0);
-        Kahan loss, xsq;
+        KahanPair lx2;   // loss, |x|^2
+        float2 xp = make_float2(x[0], x[2]), vp = make_float2(v[0], v[2]);
+        float xo = x[1], vo = v[1];
+        const float2 cdt2 = splat2(c.cdt), cva2 = splat2(c.cva), nck2 = splat2(-ckx), cs2 = splat2(c.cs);
         for (int64_t seg = 0; seg < a.nseg; ++seg) {
             float* ck = a.ckpt + seg * CW * n + i;
-#pragma unroll
-            for (int q = 0; q < 3; ++q) {
-                ck[q * n] = x[q];
-                ck[(3 + q) * n] = v[q];
-            }
-            save_state(ck + 6 * n, n);
+            ck[0] = xp.x, ck[n] = xo, ck[2 * n] = xp.y;
+            ck[3 * n] = vp.x, ck[4 * n] = vo, ck[5 * n] = vp.y;
+            if (NOISE == NOISE_REGEN) save_state(ck + 6 * n, n);
             const int64_t len = min(a.P, a.S - seg * a.P);
-            for (int64_t t = 0; t < len; ++t) {
+            float* gp = a.gbuf + seg * a.P * 3 * n + i;
+            for (int64_t t = 0; t < len; ++t, gp += 3 * n) {
                 float g[3];
                 if (KIND == GBRNG_TAUS) td.normals3(g[0], g[1], g[2]); else rd.normals3(g[0], g[1], g[2]);
-                if (a.hist) {
-#pragma unroll
-                    for (int q = 0; q < 3; ++q) a.gbuf[((seg * a.P + t) * 3 + q) * n + i] = g[q];
-                }
-#pragma unroll
-                for (int q = 0; q < 3; ++q) em_component(c.cdt, c.cva, ckx, c.cs, g[q], x[q], v[q]);
-                loss.add(energy3(hK, c.hm, x[0], x[1], x[2], v[0], v[1], v[2]));
-                xsq.add(__fmaf_rn(x[2], x[2], __fmaf_rn(x[1], x[1], __fmul_rn(x[0], x[0]))));
+                if (NOISE == NOISE_KEPT) gp[0] = g[0], gp[n] = g[1], gp[2 * n] = g[2];
+                em_component2(cdt2, cva2, nck2, cs2, make_float2(g[0], g[2]), xp, vp);
+                em_component(c.cdt, c.cva, ckx, c.cs, g[1], xo, vo);
+                const float xx = norm2(xp.x, xo, xp.y);
+                lx2.add(__fmaf_rn(hK, xx, __fmul_rn(c.hm, norm2(vp.x, vo, vp.y))), xx);
             }
         }
         // end state: the system advances exactly as ld_run would
-        a.x[3 * i] = x[0], a.x[3 * i + 1] = x[1], a.x[3 * i + 2] = x[2];
-        a.v[3 * i] = v[0], a.v[3 * i + 1] = v[1], a.v[3 * i + 2] = v[2];
+        a.x[3 * i] = xp.x, a.x[3 * i + 1] = xo, a.x[3 * i + 2] = xp.y;
+        a.v[3 * i] = vp.x, a.v[3 * i + 1] = vo, a.v[3 * i + 2] = vp.y;
         if (KIND == GBRNG_TAUS) {
             a.taus[i] = td.y;
         } else {
@@ -160,74 +181,89 @@ __global__ void __launch_bounds__(64, 12) adjoint_kernel(AdjArgs a)
         }
         // ---------------- B: reverse sweep
         const float inv_ab = __frcp_rn(__fmaf_rn(ckx, c.cdt, c.cva));
-        float lx[3], lv[3];
-#pragma unroll
-        for (int q = 0; q < 3; ++q) {
-            lx[q] = Ki * x[q] * a.invS;
-            lv[q] = a.m * v[q] * a.invS;
-        }
-        Kahan dk, dg, dT;
-        float xe[3] = {x[0], x[1], x[2]}, ve[3] = {v[0], v[1], v[2]};   // segment end state
+        const float wK = a.invS * Ki, wm = a.invS * a.m;
+        const float2 ck2 = splat2(ckx), ncs2 = splat2(-c.cs), inv2 = splat2(inv_ab), ncdt2 = splat2(-c.cdt);
+        const float2 c2g2 = splat2(a.c_over_2g), nckm2 = splat2(-c.ckm);
+        float2 lxp = make_float2(wK * xp.x, wK * xp.y), lvp = make_float2(wm * vp.x, wm * vp.y);
+        float lxo = wK * xo, lvo = wm * vo;
+        KahanPair dkg;   // dK, dgamma
+        Kahan dT;
+        // the adjoint of the step from (xt, vt) with the normals g; its loss terms w
+        auto adjoint = [&](float2 xt, float xu, float2 vt, float vu, float2 g, float gu, float k, float m) {
+            const float2 pk = __fmul2_rn(lvp, xt);
+            const float2 pg = __fmul2_rn(lvp, __ffma2_rn(nckm2, vt, __fmul2_rn(c2g2, g)));
+            const float2 pT = __fmul2_rn(lvp, g);
+            const float ddk = __fmaf_rn(lvo, xu, pk.x) + pk.y;
+            const float ddg = __fmaf_rn(lvo, __fmaf_rn(-c.ckm, vu, a.c_over_2g * gu), pg.x) + pg.y;
+            const float ddT = __fmaf_rn(lvo, gu, pT.x) + pT.y;
+            const float2 lxn = __ffma2_rn(splat2(k), xt, __ffma2_rn(nck2, lvp, lxp));
+            const float2 lvn = __ffma2_rn(splat2(m), vt, __ffma2_rn(cva2, lvp, __fmul2_rn(cdt2, lxp)));
+            const float lxq = __fmaf_rn(k, xu, __fmaf_rn(-ckx, lvo, lxo));
+            const float lvq = __fmaf_rn(m, vu, __fmaf_rn(c.cva, lvo, c.cdt * lxo));
+            lxp = lxn, lvp = lvn, lxo = lxq, lvo = lvq;
+            dkg.add(-c.ckm * ddk, ddg);
+            dT.add(a.c_over_2kT * ddT);
+        };
         for (int64_t seg = a.nseg - 1; seg >= 0; --seg) {
             const float* ck = a.ckpt + seg * CW * n + i;
             const int64_t len = min(a.P, a.S - seg * a.P);
-            if (!a.hist) {
+            if (NOISE == NOISE_REGEN) {
                 load_state(ck + 6 * n, n);
-                for (int64_t t = 0; t < len; ++t) {
+                float* gp = a.gbuf + i;
+                for (int64_t t = 0; t < len; ++t, gp += 3 * n) {
                     float g[3];
                     if (KIND == GBRNG_TAUS) td.normals3(g[0], g[1], g[2]); else rd.normals3(g[0], g[1], g[2]);
-#pragma unroll
-                    for (int q = 0; q < 3; ++q) a.gbuf[(t * 3 + q) * n + i] = g[q];
+                    gp[0] = g[0], gp[n] = g[1], gp[2 * n] = g[2];
                 }
             }
-            const float* gseg = a.gbuf + (a.hist ? seg * a.P * 3 * n : 0);
-            float xn[3] = {xe[0], xe[1], xe[2]}, vn[3] = {ve[0], ve[1], ve[2]};
-            for (int64_t t = len - 1; t >= 0; --t) {
-                const int64_t tg = seg * a.P + t;   // global step index
-                float gk[3], xt[3], vt[3];
-                float ddk = 0.f, ddg = 0.f, ddT = 0.f;
+            // x, v: the state after step t; the normals of the kAhead steps below are
+            // loaded while this one is taken back
+            const float* gp = a.gbuf + ((NOISE == NOISE_REGEN ? 0 : seg * a.P) + len - 1) * 3 * n + i;   // of step t
+            float2 g, ga[kAhead];
+            float gu, gb[kAhead];
+            auto fetch = [&](int64_t d, float2& f, float& fu) {
+                const float* p = gp - d * 3 * n;
+                f = make_float2(p[0], p[2 * n]), fu = p[n];
+            };
 #pragma unroll
-                for (int q = 0; q < 3; ++q) {
-                    gk[q] = gseg[(t * 3 + q) * n + i];
-                    vt[q] = (vn[q] + ckx * xn[q] - c.cs * gk[q]) * inv_ab;
-                    xt[q] = xn[q] - c.cdt * vt[q];
-                }
-                if (t == 0) {   // the checkpoint holds the exact state
+            for (int d = 0; d < kAhead; ++d)
+                if (d < len) fetch(d, ga[d], gb[d]);
+            auto back = [&](int d) {
+                g = ga[d], gu = gb[d];
+                vp = __fmul2_rn(__ffma2_rn(ncs2, g, __ffma2_rn(ck2, xp, vp)), inv2);
+                vo = __fmaf_rn(-c.cs, gu, __fmaf_rn(ckx, xo, vo)) * inv_ab;
+                xp = __ffma2_rn(ncdt2, vp, xp);
+                xo = __fmaf_rn(-c.cdt, vo, xo);
+            };
+            int64_t t = len - 1;
+            for (; t > kAhead; t -= kAhead, gp -= kAhead * 3 * n) {
 #pragma unroll
-                    for (int q = 0; q < 3; ++q) {
-                        xt[q] = ck[q * n];
-                        vt[q] = ck[(3 + q) * n];
-                    }
-                }
-#pragma unroll
-                for (int q = 0; q < 3; ++q) {
-                    ddk += lv[q] * xt[q];
-                    ddg += lv[q] * (a.c_over_2g * gk[q] - c.ckm * vt[q]);
-                    ddT += lv[q] * gk[q];
-                    const float w = tg >= 1 ? a.invS : 0.f;
-                    const float lxn = lx[q] - ckx * lv[q] + w * Ki * xt[q];
-                    const float lvn = c.cdt * lx[q] + c.cva * lv[q] + w * a.m * vt[q];
-                    lx[q] = lxn;
-                    lv[q] = lvn;
-                }
-                dk.add(-c.ckm * ddk);
-                dg.add(ddg);
-                dT.add(a.c_over_2kT * ddT);
-#pragma unroll
-                for (int q = 0; q < 3; ++q) {
-                    xn[q] = xt[q];
-                    vn[q] = vt[q];
+                for (int d = 0; d < kAhead; ++d) {
+                    back(d);
+                    if (t - d >= kAhead) fetch(kAhead + d, ga[d], gb[d]);
+                    adjoint(xp, xo, vp, vo, g, gu, wK, wm);
                 }
             }
 #pragma unroll
-            for (int q = 0; q < 3; ++q) {
-                xe[q] = ck[q * n];
-                ve[q] = ck[(3 + q) * n];
+            for (int d = 0; d < kAhead; ++d) {
+                if (t - d <= 0) break;
+                back(d);
+                if (t - d >= kAhead) fetch(kAhead + d, ga[d], gb[d]);
+                adjoint(xp, xo, vp, vo, g, gu, wK, wm);
             }
+            // step 0's normals: the t-th of those at hand
+            const int d0 = t < kAhead ? (int)t : 0;
+#pragma unroll
+            for (int d = 0; d < kAhead; ++d)
+                if (d == d0) g = ga[d], gu = gb[d];
+            // the segment's start: the checkpoint holds the exact state
+            xp = make_float2(ck[0], ck[2 * n]), xo = ck[n];
+            vp = make_float2(ck[3 * n], ck[5 * n]), vo = ck[4 * n];
+            adjoint(xp, xo, vp, vo, g, gu, seg > 0 ? wK : 0.f, seg > 0 ? wm : 0.f);
         }
-        if (a.dK) a.dK[i] = (float)(dk.value() + 0.5 * (double)a.invS * xsq.value());
-        acc[0] += loss.value() * (double)a.invS;
-        acc[1] += dg.value();
+        if (a.dK) a.dK[i] = (float)(dkg.first() + 0.5 * (double)a.invS * lx2.second());
+        acc[0] += lx2.first() * (double)a.invS;
+        acc[1] += dkg.second();
         acc[2] += dT.value();
     }
     block_reduce_sum<4>(acc, red);
@@ -292,10 +328,11 @@ extern "C" int ld_backward(ld_system* sys, int64_t n_steps, int ckpt_every, floa
     GB_CHECK(dev_info(h->device, &di));
     const int T = 64;
     const size_t smem = h->kind == GBRNG_RAN2 ? sizeof(int32_t) * 32 * T : 0;
+    void (*fn)(AdjArgs) = h->kind == GBRNG_RAN2
+        ? (hist ? adjoint_kernel<GBRNG_RAN2, NOISE_KEPT> : adjoint_kernel<GBRNG_RAN2, NOISE_REGEN>)
+        : (hist ? adjoint_kernel<GBRNG_TAUS, NOISE_KEPT> : adjoint_kernel<GBRNG_TAUS, NOISE_REGEN>);
     int occ = 0;
-    cudaError_t e = h->kind == GBRNG_TAUS
-        ? cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, adjoint_kernel<GBRNG_TAUS>, T, smem)
-        : cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, adjoint_kernel<GBRNG_RAN2>, T, smem);
+    cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, fn, T, smem);
     if (e != cudaSuccess || occ < 1) occ = 1;
     // one full resident wave at most; oscillators i, i + W, ... per thread
     const int64_t blocks = std::min<int64_t>((int64_t)di.sms * occ, (n + T - 1) / T);
@@ -319,12 +356,8 @@ extern "C" int ld_backward(ld_system* sys, int64_t n_steps, int ckpt_every, floa
     a.streams = h->n;
     a.ckpt = scratch;
     a.gbuf = scratch + ck_bytes / sizeof(float);
-    a.hist = hist ? 1 : 0;
     a.dK = dK_per;
-    if (h->kind == GBRNG_TAUS)
-        adjoint_kernel<GBRNG_TAUS><<<(unsigned)blocks, T, smem, st>>>(a);
-    else
-        adjoint_kernel<GBRNG_RAN2><<<(unsigned)blocks, T, smem, st>>>(a);
+    fn<<<(unsigned)blocks, T, smem, st>>>(a);
     e = cudaGetLastError();
     if (e != cudaSuccess) return fail(GBRNG_ECUDA, "adjoint launch failed: %s", cudaGetErrorString(e));
     ld_stats tmp;
