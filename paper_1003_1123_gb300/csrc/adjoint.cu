@@ -101,7 +101,7 @@ __global__ void __launch_bounds__(64, 8) adjoint_kernel(AdjArgs a)
             // src == nullptr: from the generator itself
             if (KIND == GBRNG_TAUS) {
                 if (!src) {
-                    td.y = a.taus[i];
+                    td.y = taus_load(a.taus[i]);
                 } else {
                     td.y.x = __float_as_uint(src[0]);
                     td.y.y = __float_as_uint(src[stride]);

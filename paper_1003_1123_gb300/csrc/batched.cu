@@ -72,7 +72,7 @@ __global__ void __launch_bounds__(256, KIND == GBRNG_TAUS && K == 1 ? 6 : 1)
             x0[j] = d.x[3 * i], x1[j] = d.x[3 * i + 1], x2[j] = d.x[3 * i + 2];
             v0[j] = d.v[3 * i], v1[j] = d.v[3 * i + 1], v2[j] = d.v[3 * i + 2];
             if (KIND == GBRNG_TAUS) {
-                td[j].y = d.taus[i];
+                td[j].y = taus_load(d.taus[i]);
             } else {
                 rd[j].tab = tab + j * 32 * T;
                 rd[j].T = T;
@@ -87,7 +87,8 @@ __global__ void __launch_bounds__(256, KIND == GBRNG_TAUS && K == 1 ? 6 : 1)
         if constexpr (K == 2) {
             // two oscillators a thread in the lanes of the paired binary32
             // instructions (lane j = oscillator j, each lane the scalar step),
-            // two steps a loop iteration
+            // four steps a loop iteration (512 systems x 500 steps, Hybrid Taus 15.8 ms
+            // with two, 15.5 with four, 15.7 with eight)
             const float2 cdt = splat2(c.cdt), cva = splat2(c.cva), cs = splat2(c.cs);
             const float2 nckx = make_float2(-ckx[0], -ckx[1]);
             float2 X[3] = {make_float2(x0[0], x0[1]), make_float2(x1[0], x1[1]), make_float2(x2[0], x2[1])};
@@ -96,7 +97,7 @@ __global__ void __launch_bounds__(256, KIND == GBRNG_TAUS && K == 1 ? 6 : 1)
             LcgDraw lc[2];
             for (int64_t t0 = 0; t0 < n_steps; t0 += kEnergyBlock) {
                 const int nb = (int)min((int64_t)kEnergyBlock, n_steps - t0);
-#pragma unroll 2
+#pragma unroll 4
                 for (int k = 0; k < nb; ++k) {
                     float2 g[3];
                     draw3x2<KIND>(td, lc, rd, g);
@@ -135,7 +136,9 @@ __global__ void __launch_bounds__(256, KIND == GBRNG_TAUS && K == 1 ? 6 : 1)
             const int64_t i = idx[j];
             d.x[3 * i] = x0[j], d.x[3 * i + 1] = x1[j], d.x[3 * i + 2] = x2[j];
             d.v[3 * i] = v0[j], d.v[3 * i + 1] = v1[j], d.v[3 * i + 2] = v2[j];
-            if (KIND == GBRNG_TAUS) {
+            if (n_steps == 0) {
+                // nothing drawn: the state as it stands
+            } else if (KIND == GBRNG_TAUS) {
                 d.taus[i] = td[j].y;
             } else {
                 d.r2[i] = rd[j].r.idum;

@@ -22,52 +22,66 @@ __host__ __device__ __forceinline__ uint64_t splitmix64_at(uint64_t seed, uint64
 }
 
 // ------------------------------------------------------------- Hybrid Taus
-// One Tausworthe word step (Algorithm 1): b = ((y << S1) ^ y) >> S2,
-// y = ((y & C) << S3) ^ b.
-// With MUL the two left shifts are written as multiplies by 2^S (the same
-// bits), which the FMA pipe's integer multiply-add can take off the ALU pipe;
-// used where that measured faster (the two-oscillator fused kernel).
-template <int S>
-__device__ __forceinline__ uint32_t shl_mul(uint32_t y)
+// Algorithm 1 steps a Tausworthe word by b = ((y << q) ^ y) >> (k - s),
+// y = ((y & C) << s) ^ b, with (k, q, s) = (31, 13, 12), (29, 2, 4), (28, 3, 17) and C
+// the k highest bits.  A word is 32 consecutive bits b_0 (the highest), b_1, ... of
+// the sequence b_{i+k} = b_i ^ b_{i+q}, and a step moves it s bits on.  So the bits
+// after the word are (y << (32 - k)) ^ (y << (32 - k + q)), right for k - q = 18, 27
+// and 25 of them, and the next word is a funnel shift of the two by s: two
+// instructions on the ALU pipe (the left shifts run as multiplies on the FMA pipe)
+// where Algorithm 1's form takes three, and the second word's next four are
+// four shifts of one pair.  With that a particle-step's four draws are 29 ALU
+// instructions and 22 multiplies instead of 44 and 28.
+//
+// It relies on all 32 bits being of the sequence, which holds after one step; the
+// seeds' 32 - k lowest bits are arbitrary (Algorithm 1 masks them), and are replaced
+// by taus_load: the same words follow.
+__device__ __forceinline__ uint4 taus_load(uint4 s)
 {
-    uint32_t r;
-    asm("mul.lo.u32 %0, %1, %2;" : "=r"(r) : "r"(y), "n"(1u << S));
-    return r;
+    s.x = (s.x & 0xFFFFFFFEu) | (((s.x << 13) ^ s.x) >> 31);
+    s.y = (s.y & 0xFFFFFFF8u) | (((s.y << 2) ^ s.y) >> 29);
+    s.z = (s.z & 0xFFFFFFF0u) | (((s.z << 3) ^ s.z) >> 28);
+    return s;
 }
 
-template <int S1, int S2, int S3, uint32_t C, bool MUL = false>
-__device__ __forceinline__ uint32_t taus_word(uint32_t y)
+// The word's next bits.
+template <int K, int Q>
+__device__ __forceinline__ uint32_t taus_after(uint32_t y)
 {
-    if (MUL) {
-        const uint32_t b = (shl_mul<S1>(y) ^ y) >> S2;
-        return (shl_mul<S3>(y) & (C << S3)) ^ b;
-    }
-    const uint32_t b = ((y << S1) ^ y) >> S2;
-    return ((y & C) << S3) ^ b;
-}
-
-// Advance the three Tausworthe words and the LCG, return their xor.
-template <bool MUL = false>
-__device__ __forceinline__ uint32_t taus_next(uint4& s)
-{
-    s.x = taus_word<13, 19, 12, 0xFFFFFFFEu, MUL>(s.x);
-    s.y = taus_word<2, 25, 4, 0xFFFFFFF8u, MUL>(s.y);
-    s.z = taus_word<3, 11, 17, 0xFFFFFFF0u, MUL>(s.z);
-    s.w = 1664525u * s.w + 1013904223u;
-    return s.x ^ s.y ^ s.z ^ s.w;
+    return (y << (32 - K)) ^ (y << (32 - K + Q));
 }
 
 // ------------------------------------------------------ Quick and Dirty LCG
 // Eq. 1 with m = 2^32: the multiply and add wrap; the output is the new word.
-__device__ __forceinline__ uint32_t lcg_next(uint32_t& x)
+template <int N>
+__device__ __forceinline__ void lcg_draws(uint32_t& x, uint32_t (&r)[N])
 {
-    x = 1664525u * x + 1013904223u;
-    return x;
+#pragma unroll
+    for (int k = 0; k < N; ++k) r[k] = x = 1664525u * x + 1013904223u;
 }
 
-// The per-thread 32-bit generators behind one name for the fill kernels.
-__device__ __forceinline__ uint32_t next_word(uint4& y) { return taus_next(y); }
-__device__ __forceinline__ uint32_t next_word(uint32_t& x) { return lcg_next(x); }
+// The next N <= 4 draws: the xor of the three words and the LCG's.
+template <int N>
+__device__ __forceinline__ void taus_draws(uint4& s, uint32_t (&r)[N])
+{
+    lcg_draws(s.w, r);
+    const uint32_t y0 = s.y, ly = taus_after<29, 2>(y0);
+#pragma unroll
+    for (int k = 0; k < N; ++k) {
+        s.x = __funnelshift_l(taus_after<31, 13>(s.x), s.x, 12);
+        s.y = __funnelshift_l(ly, y0, 4 * (k + 1));
+        s.z = __funnelshift_l(taus_after<28, 3>(s.z), s.z, 17);
+        r[k] ^= s.x ^ s.y ^ s.z;
+    }
+}
+
+// The per-thread 32-bit generators behind one name.
+template <int N>
+__device__ __forceinline__ void word_draws(uint4& y, uint32_t (&r)[N]) { taus_draws<N>(y, r); }
+template <int N>
+__device__ __forceinline__ void word_draws(uint32_t& x, uint32_t (&r)[N]) { lcg_draws<N>(x, r); }
+__device__ __forceinline__ uint4 word_load(uint4 y) { return taus_load(y); }
+__device__ __forceinline__ uint32_t word_load(uint32_t x) { return x; }
 
 // -------------------------------------------------------------------- Ran2
 // L'Ecuyer's pair (m1, a1) = (2147483563, 40014), (m2, a2) = (2147483399,
@@ -152,6 +166,12 @@ __device__ __forceinline__ float mant_from_u32(uint32_t raw)
 __device__ __forceinline__ float open01_from_u32(uint32_t raw)
 {
     return __fsub_rn(mant_from_u32(raw), 0x1.fffffep-1f);
+}
+
+// 2^64 u for the same u, exact likewise.
+__device__ __forceinline__ float open01_scaled(uint32_t raw)
+{
+    return __fmaf_rn(mant_from_u32(raw), 0x1p64f, -0x1.fffffep+63f);
 }
 
 // 4u for the same u, in one fused step: 4m - (4 - 2^-22) = 4 k 2^-23 + 2^-22
@@ -307,11 +327,30 @@ __device__ __forceinline__ float2 splat2(float a) { return make_float2(a, a); }
 // from a paired instruction: reading such a lane's bit pattern for the
 // exponent split measured wrong in the first lane, so callers form u lane by
 // lane.
+//
+// SPLIT: the argument is 2^64 u (exact; formed in the one step that forms u), so that
+// e + 64 is a small unsigned number, and the funnel shift that extracts it also
+// sets the upper bits of 1.5 2^23: e then comes as a binary32 from one paired
+// addition instead of a conversion each, whose result a warp waits for.  Same bits.
+// Hybrid Taus, two oscillators a thread: 1e6 x 1000 steps 4.33 -> 4.09 ms; where the
+// other instructions are fewer the extra shift costs more (LCG +1%, overdamped +2%,
+// LCG normal fill +4%), and those convert.
+template <bool SPLIT = false>
 __device__ __forceinline__ float2 neg2log2(float2 u)
 {
-    const int bx = __float_as_int(u.x), by = __float_as_int(u.y);
-    const int ex = (bx - 0x3f2aaaab) >> 23, ey = (by - 0x3f2aaaab) >> 23;
-    const float2 m = make_float2(__int_as_float(bx - (ex << 23)), __int_as_float(by - (ey << 23)));
+    float2 m, ef;
+    if (SPLIT) {
+        const uint32_t bx = __float_as_uint(u.x), by = __float_as_uint(u.y);
+        const uint32_t qx = __funnelshift_r(bx - 0x3f2aaaabu, 0x4b400000u >> 9, 23);
+        const uint32_t qy = __funnelshift_r(by - 0x3f2aaaabu, 0x4b400000u >> 9, 23);
+        m = make_float2(__uint_as_float(bx - (qx << 23)), __uint_as_float(by - (qy << 23)));
+        ef = __fadd2_rn(make_float2(__uint_as_float(qx), __uint_as_float(qy)), splat2(-(0x1.8p+23f + 64.0f)));
+    } else {
+        const int bx = __float_as_int(u.x), by = __float_as_int(u.y);
+        const int ex = (bx - 0x3f2aaaab) >> 23, ey = (by - 0x3f2aaaab) >> 23;
+        m = make_float2(__int_as_float(bx - (ex << 23)), __int_as_float(by - (ey << 23)));
+        ef = make_float2((float)ex, (float)ey);
+    }
     const float2 g = __ffma2_rn(m, splat2(-2.0f), splat2(2.0f));
     const float2 g2 = __fmul2_rn(g, g);
     const float2 g4 = __fmul2_rn(g2, g2);
@@ -324,7 +363,6 @@ __device__ __forceinline__ float2 neg2log2(float2 u)
     const float2 p48 = __ffma2_rn(splat2(kLogG[8]), g4, p47);
     const float2 R = __ffma2_rn(p48, g4, p03);
     const float2 l2m = __ffma2_rn(g2, R, g);
-    const float2 ef = make_float2((float)ex, (float)ey);
     return __ffma2_rn(ef, splat2(0x1.05c610p-28f), __ffma2_rn(ef, splat2(-0x1.62e430p+0f), l2m));
 }
 
@@ -378,13 +416,15 @@ __device__ __forceinline__ void box_muller3_x(float2 m2log, float2 x, float& g0,
 }
 
 // Four raw 32-bit draws -> three normals.
+template <bool SPLIT = false>
 __device__ __forceinline__ void box_muller3_u32(uint32_t r1, uint32_t r2, uint32_t r3, uint32_t r4,
                                                 float& g0, float& g1, float& g2)
 {
-    const float2 u = make_float2(open01_from_u32(r1), open01_from_u32(r3));
+    const float2 u = SPLIT ? make_float2(open01_scaled(r1), open01_scaled(r3))
+                           : make_float2(open01_from_u32(r1), open01_from_u32(r3));
     const float2 x = __ffma2_rn(splat2(4.0f), make_float2(mant_from_u32(r2), mant_from_u32(r4)),
                                 splat2(-0x1.fffffep+1f));
-    box_muller3_x(neg2log2(u), x, g0, g1, g2);
+    box_muller3_x(neg2log2<SPLIT>(u), x, g0, g1, g2);
 }
 
 // Ran2's four uniforms -> three normals.
@@ -441,16 +481,18 @@ __device__ __forceinline__ void box_muller_2pairs(float u1, float u2, float u3, 
 // Three normals of a particle-step for each of two oscillators from their four
 // raw draws r[j][0..3]: g[k] = (normal k of oscillator 0, normal k of
 // oscillator 1).
+template <bool SPLIT = false>
 __device__ __forceinline__ void normals3x2_u32(const uint32_t (&r)[2][4], float2 (&g)[3])
 {
-    const float2 ua = make_float2(open01_from_u32(r[0][0]), open01_from_u32(r[1][0]));
-    const float2 ub = make_float2(open01_from_u32(r[0][2]), open01_from_u32(r[1][2]));
+    auto u01 = [](uint32_t raw) { return SPLIT ? open01_scaled(raw) : open01_from_u32(raw); };
+    const float2 ua = make_float2(u01(r[0][0]), u01(r[1][0]));
+    const float2 ub = make_float2(u01(r[0][2]), u01(r[1][2]));
     const float2 xa = __ffma2_rn(splat2(4.0f), make_float2(mant_from_u32(r[0][1]), mant_from_u32(r[1][1])),
                                  splat2(-0x1.fffffep+1f));
     const float2 xb = __ffma2_rn(splat2(4.0f), make_float2(mant_from_u32(r[0][3]), mant_from_u32(r[1][3])),
                                  splat2(-0x1.fffffep+1f));
-    box_muller_pair2(neg2log2(ua), xa, g[0], g[1]);
-    g[2] = box_muller_cos2(neg2log2(ub), xb);
+    box_muller_pair2(neg2log2<SPLIT>(ua), xa, g[0], g[1]);
+    g[2] = box_muller_cos2(neg2log2<SPLIT>(ub), xb);
 }
 
 // The same from Ran2's uniforms u[j][0..3].
@@ -467,11 +509,9 @@ struct TausDraw {
     uint4 y;
     __device__ __forceinline__ void normals3(float& gx, float& gy, float& gz)
     {
-        const uint32_t r1 = taus_next(y);
-        const uint32_t r2 = taus_next(y);
-        const uint32_t r3 = taus_next(y);
-        const uint32_t r4 = taus_next(y);
-        box_muller3_u32(r1, r2, r3, r4, gx, gy, gz);
+        uint32_t r[4];
+        taus_draws(y, r);
+        box_muller3_u32<true>(r[0], r[1], r[2], r[3], gx, gy, gz);
     }
 };
 
@@ -479,11 +519,9 @@ struct LcgDraw {
     uint32_t x;
     __device__ __forceinline__ void normals3(float& gx, float& gy, float& gz)
     {
-        const uint32_t r1 = lcg_next(x);
-        const uint32_t r2 = lcg_next(x);
-        const uint32_t r3 = lcg_next(x);
-        const uint32_t r4 = lcg_next(x);
-        box_muller3_u32(r1, r2, r3, r4, gx, gy, gz);
+        uint32_t r[4];
+        lcg_draws(x, r);
+        box_muller3_u32(r[0], r[1], r[2], r[3], gx, gy, gz);
     }
 };
 
@@ -510,7 +548,7 @@ struct Ran2Draw {
 // Three normals of a particle-step for each of two oscillators with their own
 // generators (lane j = oscillator j); each generator draws its four numbers
 // in order, as in draw3.
-template <int KIND, bool MUL = false>
+template <int KIND>
 __device__ __forceinline__ void draw3x2(TausDraw (&td)[2], LcgDraw (&lc)[2], Ran2Draw (&rd)[2],
                                         float2 (&g)[3])
 {
@@ -524,11 +562,13 @@ __device__ __forceinline__ void draw3x2(TausDraw (&td)[2], LcgDraw (&lc)[2], Ran
     } else {
         uint32_t r[2][4];
 #pragma unroll
-        for (int j = 0; j < 2; ++j)
-#pragma unroll
-            for (int q = 0; q < 4; ++q)
-                r[j][q] = KIND == GBRNG_TAUS ? taus_next<MUL>(td[j].y) : lcg_next(lc[j].x);
-        normals3x2_u32(r, g);
+        for (int j = 0; j < 2; ++j) {
+            if (KIND == GBRNG_TAUS)
+                taus_draws(td[j].y, r[j]);
+            else
+                lcg_draws(lc[j].x, r[j]);
+        }
+        normals3x2_u32<KIND == GBRNG_TAUS>(r, g);
     }
 }
 

@@ -13,20 +13,14 @@ namespace gb {
 
 enum { FILL_U32 = 0, FILL_UNIFORM = 1, FILL_NORMAL = 2 };
 
-template <int MODE, class State>
-__device__ __forceinline__ void emit_word(State& y, int64_t idx, void* out)
+// Item idx from its draws.
+template <int MODE>
+__device__ __forceinline__ void emit_item(uint32_t r, int64_t idx, void* out)
 {
-    if (MODE == FILL_U32) {
-        ((uint32_t*)out)[idx] = next_word(y);
-    } else if (MODE == FILL_UNIFORM) {
-        ((float*)out)[idx] = u01_from_u32(next_word(y));
-    } else {
-        const uint32_t r1 = next_word(y);
-        const uint32_t r2 = next_word(y);
-        float2 g;
-        box_muller_u32(r1, r2, g.x, g.y);
-        ((float2*)out)[idx] = g;
-    }
+    if (MODE == FILL_U32)
+        ((uint32_t*)out)[idx] = r;
+    else
+        ((float*)out)[idx] = u01_from_u32(r);
 }
 
 // n_items = numbers (u32, uniform) or pairs (normal); the items idx, idx + S, ... <
@@ -38,23 +32,35 @@ __device__ __forceinline__ void emit_chain(State& y, int64_t idx, int64_t S, int
     for (; idx + 3 * S < end; idx += 4 * S) {
         if (MODE == FILL_NORMAL) {
             // the four pairs two at a time in the paired instructions' lanes
-            uint32_t r[8];
-#pragma unroll
-            for (int q = 0; q < 8; ++q) r[q] = next_word(y);
+            uint32_t r[4];
             float2* o = (float2*)out;
             float2 ga, gb;
+            word_draws(y, r);
             box_muller_2pairs_u32(r[0], r[1], r[2], r[3], ga, gb);
             o[idx] = ga, o[idx + S] = gb;
-            box_muller_2pairs_u32(r[4], r[5], r[6], r[7], ga, gb);
+            word_draws(y, r);
+            box_muller_2pairs_u32(r[0], r[1], r[2], r[3], ga, gb);
             o[idx + 2 * S] = ga, o[idx + 3 * S] = gb;
         } else {
-            emit_word<MODE>(y, idx, out);
-            emit_word<MODE>(y, idx + S, out);
-            emit_word<MODE>(y, idx + 2 * S, out);
-            emit_word<MODE>(y, idx + 3 * S, out);
+            uint32_t r[4];
+            word_draws(y, r);
+#pragma unroll
+            for (int q = 0; q < 4; ++q) emit_item<MODE>(r[q], idx + q * S, out);
         }
     }
-    for (; idx < end; idx += S) emit_word<MODE>(y, idx, out);
+    for (; idx < end; idx += S) {
+        if (MODE == FILL_NORMAL) {
+            uint32_t r[2];
+            float2 g;
+            word_draws(y, r);
+            box_muller_u32(r[0], r[1], g.x, g.y);
+            ((float2*)out)[idx] = g;
+        } else {
+            uint32_t r[1];
+            word_draws(y, r);
+            emit_item<MODE>(r[0], idx, out);
+        }
+    }
 }
 
 // Hybrid Taus (uint4 state) and the LCG (uint32 state): one word chain per stream.
@@ -65,7 +71,7 @@ __global__ void __launch_bounds__(256) word_fill_kernel(State* __restrict__ st, 
     const int64_t active = S < n_items ? S : n_items;
     const int64_t stride = (int64_t)gridDim.x * blockDim.x;
     for (int64_t s = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; s < active; s += stride) {
-        State y = st[s];
+        State y = word_load(st[s]);
         emit_chain<MODE>(y, s, S, n_items, out);
         st[s] = y;
     }
@@ -103,7 +109,7 @@ __global__ void __launch_bounds__(kSplitThreads) word_split_kernel(State* st, in
     const bool live = s < S && first < n_items;
     State y;
     if (live) {
-        y = st[s];
+        y = word_load(st[s]);
         if (g & 7) jump_ahead(y, a.lo[g & 7]);
         if (g >> 3) jump_ahead(y, a.hi[g >> 3]);
     }

@@ -53,7 +53,7 @@ __global__ void __launch_bounds__(128, 6) ld_noalloc_kernel(NoallocArgs a)
         TausDraw td;
         Ran2Draw rd;
         if (KIND == GBRNG_TAUS) {
-            td.y = a.taus[i];
+            td.y = taus_load(a.taus[i]);
         } else {
             rd.tab = tab;
             rd.T = blockDim.x;
@@ -81,7 +81,9 @@ __global__ void __launch_bounds__(128, 6) ld_noalloc_kernel(NoallocArgs a)
         }
         a.x[3 * i] = x0, a.x[3 * i + 1] = x1, a.x[3 * i + 2] = x2;
         a.v[3 * i] = v0, a.v[3 * i + 1] = v1, a.v[3 * i + 2] = v2;
-        if (KIND == GBRNG_TAUS) {
+        if (a.n_steps == 0) {
+            // nothing drawn: the state as it stands
+        } else if (KIND == GBRNG_TAUS) {
             a.taus[i] = td.y;
         } else {
             a.r2[i] = rd.r.idum;

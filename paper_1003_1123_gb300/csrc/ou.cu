@@ -27,13 +27,13 @@ template <int KIND>
 __device__ __forceinline__ float normal1(TausDraw& td, LcgDraw& lc, Ran2Draw& rd)
 {
     if (KIND == GBRNG_TAUS) {
-        const uint32_t r1 = taus_next(td.y);
-        const uint32_t r2 = taus_next(td.y);
-        return box_muller_cos_u32(r1, r2);
+        uint32_t r[2];
+        taus_draws(td.y, r);
+        return box_muller_cos_u32(r[0], r[1]);
     } else if (KIND == GBRNG_LCG) {
-        const uint32_t r1 = lcg_next(lc.x);
-        const uint32_t r2 = lcg_next(lc.x);
-        return box_muller_cos_u32(r1, r2);
+        uint32_t r[2];
+        lcg_draws(lc.x, r);
+        return box_muller_cos_u32(r[0], r[1]);
     } else {
         const float u1 = u01_from_ran2(rd.next());
         const float u2 = u01_from_ran2(rd.next());
@@ -56,8 +56,10 @@ __device__ __forceinline__ float2 normal2(TausDraw& td, LcgDraw& lc, Ran2Draw& r
                                __fmul2_rn(splat2(4.0f), make_float2(u2, u4)));
     } else {
         uint32_t r[4];
-#pragma unroll
-        for (int q = 0; q < 4; ++q) r[q] = KIND == GBRNG_TAUS ? taus_next(td.y) : lcg_next(lc.x);
+        if (KIND == GBRNG_TAUS)
+            taus_draws(td.y, r);
+        else
+            lcg_draws(lc.x, r);
         const float2 u = make_float2(open01_from_u32(r[0]), open01_from_u32(r[2]));
         const float2 x = __ffma2_rn(splat2(4.0f), make_float2(mant_from_u32(r[1]), mant_from_u32(r[3])),
                                     splat2(-0x1.fffffep+1f));
@@ -77,7 +79,7 @@ __global__ void __launch_bounds__(256) ou_pt_kernel(OuArgs a)
     LcgDraw lc;
     Ran2Draw rd;
     if (KIND == GBRNG_TAUS) {
-        td.y = a.taus[k];
+        td.y = taus_load(a.taus[k]);
     } else if (KIND == GBRNG_LCG) {
         lc.x = a.lcg[k];
     } else {
@@ -118,7 +120,7 @@ __global__ void __launch_bounds__(256) ou_pt_kernel(OuArgs a)
             t += 1;
         }
     }
-    if (!live) return;
+    if (!live || a.n_steps == 0) return;
     a.R[i] = R;
     if (KIND == GBRNG_TAUS) {
         a.taus[i] = td.y;

@@ -35,7 +35,7 @@ __global__ void __launch_bounds__(256) step_pt_kernel(StepArgs a)
     float g0, g1, g2;
     if (KIND == GBRNG_TAUS) {
         TausDraw td;
-        td.y = a.taus[i];
+        td.y = taus_load(a.taus[i]);
         td.normals3(g0, g1, g2);
         a.taus[i] = td.y;
     } else if (KIND == GBRNG_LCG) {

@@ -89,9 +89,12 @@ __device__ __forceinline__ float2 draw_cos2(TausDraw (&td)[2], LcgDraw (&lc)[2])
 {
     uint32_t r[2][2];
 #pragma unroll
-    for (int j = 0; j < 2; ++j)
-#pragma unroll
-        for (int q = 0; q < 2; ++q) r[j][q] = KIND == GBRNG_TAUS ? taus_next(td[j].y) : lcg_next(lc[j].x);
+    for (int j = 0; j < 2; ++j) {
+        if (KIND == GBRNG_TAUS)
+            taus_draws(td[j].y, r[j]);
+        else
+            lcg_draws(lc[j].x, r[j]);
+    }
     const float2 u = make_float2(open01_from_u32(r[0][0]), open01_from_u32(r[1][0]));
     const float2 x = __ffma2_rn(splat2(4.0f), make_float2(mant_from_u32(r[0][1]), mant_from_u32(r[1][1])),
                                 splat2(-0x1.fffffep+1f));
@@ -143,7 +146,7 @@ __device__ __forceinline__ void team_produce(const TeamArgs& a, float* buf, int 
         live[j] = idx[j] < a.n;
         const int64_t i = live[j] ? idx[j] : first;   // a dead lane shadows the block's first
         if (KIND == GBRNG_TAUS)
-            td[j].y = a.taus[i];
+            td[j].y = taus_load(a.taus[i]);
         else
             lc[j].x = a.lcg[i];
     }
