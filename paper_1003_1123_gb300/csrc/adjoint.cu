@@ -94,9 +94,6 @@ __global__ void __launch_bounds__(64, 8) adjoint_kernel(AdjArgs a)
         float v[3] = {a.v[3 * i], a.v[3 * i + 1], a.v[3 * i + 2]};
         TausDraw td;
         Ran2Draw rd;
-        rd.tab = tab;
-        rd.T = blockDim.x;
-        rd.tid = threadIdx.x;
         auto load_state = [&](const float* src, int64_t stride) {
             // src == nullptr: from the generator itself
             if (KIND == GBRNG_TAUS) {
@@ -108,22 +105,10 @@ __global__ void __launch_bounds__(64, 8) adjoint_kernel(AdjArgs a)
                     td.y.z = __float_as_uint(src[2 * stride]);
                     td.y.w = __float_as_uint(src[3 * stride]);
                 }
+            } else if (!src) {
+                rd.load(a.r2 + i, a.streams, tab, blockDim.x);
             } else {
-                if (!src) {
-                    rd.r.idum = a.r2[i];
-                    rd.r.idum2 = a.r2[a.streams + i];
-                    rd.r.iy = a.r2[2 * a.streams + i];
-                    #pragma unroll 4
-                    for (int j = 0; j < 32; ++j)
-                        tab[j * blockDim.x + threadIdx.x] = a.r2[(3 + j) * a.streams + i];
-                } else {
-                    rd.r.idum = __float_as_int(src[0]);
-                    rd.r.idum2 = __float_as_int(src[stride]);
-                    rd.r.iy = __float_as_int(src[2 * stride]);
-                    #pragma unroll 4
-                    for (int j = 0; j < 32; ++j)
-                        tab[j * blockDim.x + threadIdx.x] = __float_as_int(src[(3 + j) * stride]);
-                }
+                rd.load(src, stride, tab, blockDim.x);
             }
         };
         auto save_state = [&](float* dst, int64_t stride) {
@@ -133,12 +118,7 @@ __global__ void __launch_bounds__(64, 8) adjoint_kernel(AdjArgs a)
                 dst[2 * stride] = __uint_as_float(td.y.z);
                 dst[3 * stride] = __uint_as_float(td.y.w);
             } else {
-                dst[0] = __int_as_float(rd.r.idum);
-                dst[stride] = __int_as_float(rd.r.idum2);
-                dst[2 * stride] = __int_as_float(rd.r.iy);
-                #pragma unroll 4
-                for (int j = 0; j < 32; ++j)
-                    dst[(3 + j) * stride] = __int_as_float(tab[j * blockDim.x + threadIdx.x]);
+                rd.store(dst, stride);
             }
         };
         // ---------------- A: forward with checkpoints
@@ -172,12 +152,7 @@ __global__ void __launch_bounds__(64, 8) adjoint_kernel(AdjArgs a)
         if (KIND == GBRNG_TAUS) {
             a.taus[i] = td.y;
         } else {
-            a.r2[i] = rd.r.idum;
-            a.r2[a.streams + i] = rd.r.idum2;
-            a.r2[2 * a.streams + i] = rd.r.iy;
-            #pragma unroll 4
-            for (int j = 0; j < 32; ++j)
-                a.r2[(3 + j) * a.streams + i] = tab[j * blockDim.x + threadIdx.x];
+            rd.store(a.r2 + i, a.streams);
         }
         // ---------------- B: reverse sweep
         const float inv_ab = __frcp_rn(__fmaf_rn(ckx, c.cdt, c.cva));

@@ -74,14 +74,7 @@ __global__ void __launch_bounds__(256, KIND == GBRNG_TAUS && K == 1 ? 6 : 1)
             if (KIND == GBRNG_TAUS) {
                 td[j].y = taus_load(d.taus[i]);
             } else {
-                rd[j].tab = tab + j * 32 * T;
-                rd[j].T = T;
-                rd[j].tid = tid;
-                rd[j].r.idum = d.r2[i];
-                rd[j].r.idum2 = d.r2[d.S + i];
-                rd[j].r.iy = d.r2[2 * d.S + i];
-#pragma unroll 4
-                for (int q = 0; q < 32; ++q) rd[j].tab[q * T + tid] = d.r2[(3 + q) * d.S + i];
+                rd[j].load(d.r2 + i, d.S, tab + j * 32 * T, T);
             }
         }
         if constexpr (K == 2) {
@@ -141,11 +134,7 @@ __global__ void __launch_bounds__(256, KIND == GBRNG_TAUS && K == 1 ? 6 : 1)
             } else if (KIND == GBRNG_TAUS) {
                 d.taus[i] = td[j].y;
             } else {
-                d.r2[i] = rd[j].r.idum;
-                d.r2[d.S + i] = rd[j].r.idum2;
-                d.r2[2 * d.S + i] = rd[j].r.iy;
-#pragma unroll 4
-                for (int q = 0; q < 32; ++q) d.r2[(3 + q) * d.S + i] = rd[j].tab[q * T + tid];
+                rd[j].store(d.r2 + i, d.S);
             }
             acc[0] += (double)x0[j] * x0[j] + (double)x1[j] * x1[j] + (double)x2[j] * x2[j];
             acc[1] += (double)v0[j] * v0[j] + (double)v1[j] * v1[j] + (double)v2[j] * v2[j];

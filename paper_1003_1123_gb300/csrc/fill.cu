@@ -119,27 +119,29 @@ __global__ void __launch_bounds__(kSplitThreads) word_split_kernel(State* st, in
     if (first + ((end - first - 1) / S) * S + S >= n_items) st[s] = y;   // the stream's last item
 }
 
+constexpr int kRan2Threads = 128;
+
+// The table's 32 words are loaded, and stored, all at once: at 134 draws a stream of 1e6
+// streams the state is a third of the traffic, and four words at a time its latency shows
+// (2^27 uniforms 167 us, eight or sixteen at a time 160, all 150; 2^24 70 and 62).
 template <int MODE>
-__global__ void __launch_bounds__(128) ran2_fill_kernel(int32_t* __restrict__ st, int64_t S,
+__global__ void __launch_bounds__(kRan2Threads) ran2_fill_kernel(int32_t* __restrict__ st, int64_t S,
                                                         int64_t n_items, void* __restrict__ out)
 {
     extern __shared__ int32_t tab[];      // [32][blockDim.x]
-    const int T = blockDim.x, tid = threadIdx.x;
-    auto iv = [&](int j) -> int32_t& { return tab[j * T + tid]; };
     const int64_t active = S < n_items ? S : n_items;
     const int64_t stride = (int64_t)gridDim.x * blockDim.x;
-    for (int64_t s = blockIdx.x * (int64_t)blockDim.x + tid; s < active; s += stride) {
-        Ran2Regs r{st[s], st[S + s], st[2 * S + s]};
-#pragma unroll 4
-        for (int j = 0; j < 32; ++j) iv(j) = st[(3 + j) * S + s];
+    for (int64_t s = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; s < active; s += stride) {
+        Ran2Draw rd;
+        rd.load<32>(st + s, S, tab, kRan2Threads);
         auto emit = [&](int64_t idx) {
             if (MODE == FILL_U32) {
-                ((uint32_t*)out)[idx] = (uint32_t)ran2_next(r, iv);
+                ((uint32_t*)out)[idx] = (uint32_t)-rd.next();
             } else if (MODE == FILL_UNIFORM) {
-                ((float*)out)[idx] = u01_from_ran2(ran2_next(r, iv));
+                ((float*)out)[idx] = u01_from_ran2(rd.next());
             } else {
-                const float u1 = u01_from_ran2(ran2_next(r, iv));
-                const float u2 = u01_from_ran2(ran2_next(r, iv));
+                const float u1 = u01_from_ran2(rd.next());
+                const float u2 = u01_from_ran2(rd.next());
                 float2 g;
                 box_muller(u1, u2, g.x, g.y);
                 ((float2*)out)[idx] = g;
@@ -150,14 +152,14 @@ __global__ void __launch_bounds__(128) ran2_fill_kernel(int32_t* __restrict__ st
         for (; idx + 3 * S < n_items; idx += 4 * S) {
             if (MODE == FILL_NORMAL) {
                 // the four pairs two at a time in the paired instructions' lanes
-                float u[8];
+                int32_t n[8];
 #pragma unroll
-                for (int q = 0; q < 8; ++q) u[q] = u01_from_ran2(ran2_next(r, iv));
+                for (int q = 0; q < 8; ++q) n[q] = rd.next();
                 float2* o = (float2*)out;
                 float2 ga, gb;
-                box_muller_2pairs(u[0], u[1], u[2], u[3], ga, gb);
+                box_muller_2pairs_ran2(n[0], n[1], n[2], n[3], ga, gb);
                 o[idx] = ga, o[idx + S] = gb;
-                box_muller_2pairs(u[4], u[5], u[6], u[7], ga, gb);
+                box_muller_2pairs_ran2(n[4], n[5], n[6], n[7], ga, gb);
                 o[idx + 2 * S] = ga, o[idx + 3 * S] = gb;
             } else {
                 emit(idx);
@@ -167,11 +169,7 @@ __global__ void __launch_bounds__(128) ran2_fill_kernel(int32_t* __restrict__ st
             }
         }
         for (; idx < n_items; idx += S) emit(idx);
-        st[s] = r.idum;
-        st[S + s] = r.idum2;
-        st[2 * S + s] = r.iy;
-#pragma unroll 4
-        for (int j = 0; j < 32; ++j) st[(3 + j) * S + s] = iv(j);
+        rd.store<32>(st + s, S);
     }
 }
 
@@ -235,7 +233,7 @@ static int fill_pt(Handle* h, void* dst, int64_t n_items, cudaStream_t st)
             word_fill_kernel<MODE, uint32_t><<<(unsigned)blocks, T, 0, st>>>(h->lcg, h->n, n_items,
                                                                             dst);
     } else {
-        const int T = 128;
+        const int T = kRan2Threads;
         const size_t smem = sizeof(int32_t) * 32 * T;
         const int64_t blocks = (active + T - 1) / T;
         ran2_fill_kernel<MODE><<<(unsigned)blocks, T, smem, st>>>(h->r2, h->n, n_items, dst);

@@ -52,14 +52,7 @@ __global__ void __launch_bounds__(128, KIND == GBRNG_LCG ? 7 : 6) ld_pt_kernel(L
         } else if (KIND == GBRNG_LCG) {
             lc.x = a.lcg[i];
         } else {
-            rd.tab = tab;
-            rd.T = blockDim.x;
-            rd.tid = threadIdx.x;
-            rd.r.idum = a.r2[i];
-            rd.r.idum2 = a.r2[a.S + i];
-            rd.r.iy = a.r2[2 * a.S + i];
-#pragma unroll 4
-            for (int j = 0; j < 32; ++j) tab[j * blockDim.x + threadIdx.x] = a.r2[(3 + j) * a.S + i];
+            rd.load(a.r2 + i, a.S, tab, 32);
         }
         EnergySum es;
         float hK = 0.f;
@@ -76,9 +69,10 @@ __global__ void __launch_bounds__(128, KIND == GBRNG_LCG ? 7 : 6) ld_pt_kernel(L
             hK = 0.5f * Ki;
             for (int64_t t0 = 0; t0 < a.n_steps; t0 += kEnergyBlock) {
                 const int nb = (int)min((int64_t)kEnergyBlock, a.n_steps - t0);
-                // the LCG draws cheaply enough to gain from two steps a loop
-                // iteration (3% faster); Taus and Ran2 lose 1-2%
-#pragma unroll(KIND == GBRNG_LCG ? 2 : 1)
+                // steps an iteration: the LCG 3% faster with two; Ran2, whose next
+                // draws' chain then runs beside a step's transforms, with eight (1000
+                // oscillators x 1000 steps 195 -> 191 us, 5e4 365 -> 351); Taus loses 1-2%
+#pragma unroll(KIND == GBRNG_LCG ? 2 : KIND == GBRNG_RAN2 ? 8 : 1)
                 for (int k = 0; k < nb; ++k) {
                     float g0, g1, g2;
                     draw3<KIND>(td, lc, rd, g0, g1, g2);
@@ -99,11 +93,7 @@ __global__ void __launch_bounds__(128, KIND == GBRNG_LCG ? 7 : 6) ld_pt_kernel(L
         } else if (KIND == GBRNG_LCG) {
             a.lcg[i] = lc.x;
         } else {
-            a.r2[i] = rd.r.idum;
-            a.r2[a.S + i] = rd.r.idum2;
-            a.r2[2 * a.S + i] = rd.r.iy;
-#pragma unroll 4
-            for (int j = 0; j < 32; ++j) a.r2[(3 + j) * a.S + i] = tab[j * blockDim.x + threadIdx.x];
+            rd.store(a.r2 + i, a.S);
         }
         acc[0] += (double)x0 * x0 + (double)x1 * x1 + (double)x2 * x2;
         acc[1] += (double)v0 * v0 + (double)v1 * v1 + (double)v2 * v2;
@@ -160,14 +150,7 @@ __global__ void __launch_bounds__(32) ld_pair_kernel(LdArgs a, int64_t n_pairs)
             } else if (KIND == GBRNG_LCG) {
                 lc[j].x = a.lcg[i];
             } else {
-                rd[j].tab = tab + j * 32 * blockDim.x;
-                rd[j].T = blockDim.x;
-                rd[j].tid = threadIdx.x;
-                rd[j].r.idum = a.r2[i];
-                rd[j].r.idum2 = a.r2[a.S + i];
-                rd[j].r.iy = a.r2[2 * a.S + i];
-#pragma unroll 4
-                for (int q = 0; q < 32; ++q) rd[j].tab[q * blockDim.x + threadIdx.x] = a.r2[(3 + q) * a.S + i];
+                rd[j].load(a.r2 + i, a.S, tab + j * 32 * blockDim.x, 32);
             }
         }
         nckx = make_float2(ck[0], ck[1]);
@@ -180,7 +163,8 @@ __global__ void __launch_bounds__(32) ld_pair_kernel(LdArgs a, int64_t n_pairs)
             const int nb = (int)min((int64_t)kEnergyBlock, a.n_steps - t0);
             // steps an iteration: Hybrid Taus 4.33 ms with two and converted exponents,
             // 4.09 with two, 4.05 with eight (1e6 x 1000); the LCG 3.15 and Ran2 6.04 with
-            // two, 3.11 and 5.96 with four, 3.11 and 6.13 with eight
+            // two, 3.11 and 5.96 with four, 3.11 and 6.13 with eight; since its two
+            // oscillators draw side by side Ran2 takes 5.23, 5.19 and 5.26
 #pragma unroll(KIND == GBRNG_TAUS ? 8 : 4)
             for (int k = 0; k < nb; ++k) {
                 float2 g[3];
@@ -206,11 +190,7 @@ __global__ void __launch_bounds__(32) ld_pair_kernel(LdArgs a, int64_t n_pairs)
             } else if (KIND == GBRNG_LCG) {
                 a.lcg[i] = lc[j].x;
             } else {
-                a.r2[i] = rd[j].r.idum;
-                a.r2[a.S + i] = rd[j].r.idum2;
-                a.r2[2 * a.S + i] = rd[j].r.iy;
-#pragma unroll 4
-                for (int q = 0; q < 32; ++q) a.r2[(3 + q) * a.S + i] = rd[j].tab[q * blockDim.x + threadIdx.x];
+                rd[j].store(a.r2 + i, a.S);
             }
             acc[0] += (double)x0 * x0 + (double)x1 * x1 + (double)x2 * x2;
             acc[1] += (double)v0 * v0 + (double)v1 * v1 + (double)v2 * v2;
@@ -230,7 +210,7 @@ __global__ void __launch_bounds__(32) ld_pair_kernel(LdArgs a, int64_t n_pairs)
 // Hybrid Taus against 6.13 ms for one oscillator a thread; 64-, 128- and
 // 256-thread blocks 6.06-6.60 ms; a grid trimmed so that every thread gets the
 // same number of pairs (fewer warps a SM) 6.36 ms.  With the paired
-// instructions: Taus 4.7 ms, Ran2 6.0 ms (64-thread blocks for Ran2 equal).
+// instructions: Taus 4.05 ms, Ran2 5.19 ms.
 template <int KIND>
 static int launch_pairs(const ld_system* s, int64_t n_steps, ld_stats* out, cudaStream_t st)
 {
@@ -311,22 +291,30 @@ int ld_init_pt(const ld_system* s, cudaStream_t st)
 // Which kernel runs a system.  A run's time is the steps' times the time of a
 // step, which for the thread-per-oscillator kernels goes by the warps on the
 // busiest scheduler (w1 with one oscillator a thread, w2 with two) and for the
-// teams by the oscillators a SM holds.  Measured for Hybrid Taus, ns a step:
-// one a thread 134, 206, 313, 408, 505, 602, 698, 795 for w1 = 1 .. 8; two a
-// thread 212, 377, 551, 723 for w2 = 1 .. 4 (16 warps a SM: a full wave); teams
-// 28 + 0.79 per oscillator a SM, and 8 us + 5.5 us per 1e4 oscillators more at
-// their start than the others.  The LCG's (87, 142, 210, 275, 340, 405 / 152,
-// 255, 377, 491 / 0.52) and Ran2's (763 against 740 at w1 = 6, 1000 against 957
-// at w1 = 8) stand to each other alike.
+// teams by the oscillators a SM holds, besides their start-up (the jumps).  The
+// costs are measured, ns a step over 1000 steps, one a thread by w1, two a thread by
+// w2; teams 9 + 0.67 per oscillator a SM for Hybrid Taus and 6 + 0.48 for the LCG,
+// and 2.5 us + 0.3 (LCG 0.2) us per 1000 oscillators at the start beyond the others'.
+// Above w1 = 7 two a thread are faster for every generator (155600 oscillators: 630
+// against 831, 488 against 584 and 812 against 934).
 enum LdPath { LD_ONE, LD_PAIRS, LD_TEAM };
+struct LdCost {
+    double one[7], pairs[4];
+    double team0, team, start0, start;   // ns: a step, per oscillator a SM; start, per oscillator
+};
+constexpr LdCost kCostTaus = {{119, 193, 287, 380, 469, 559, 651}, {183, 326, 478, 629}, 9, 0.67, 2500, 0.3};
+constexpr LdCost kCostLcg = {{92, 142, 208, 271, 333, 396, 458}, {166, 255, 376, 488}, 6, 0.48, 2500, 0.2};
+constexpr LdCost kCostRan2 = {{191, 254, 350, 451, 548, 645, 838}, {277, 429, 628, 812}, 1e300, 0, 0, 0};   // no team
+
 static LdPath pick_path(int kind, int64_t n, int64_t n_steps, int sms)
 {
     const int64_t w1 = (n + 128ll * sms - 1) / (128ll * sms), w2 = (n + 256ll * sms - 1) / (256ll * sms);
-    if (w1 > 8) return LD_PAIRS;
-    const double one = w1 <= 2 ? 62 + 72.0 * (double)w1 : 5 + 100.0 * (double)w1;
-    const double pairs = 38 + 172.0 * (double)w2;
-    const double team = 28 + 0.79 * (double)n / sms + (8000 + 0.55 * (double)n) / (double)std::max<int64_t>(n_steps, 1);
-    if (kind != GBRNG_RAN2 && team < std::min(one, pairs)) return LD_TEAM;
+    if (w1 > 7) return LD_PAIRS;
+    const LdCost& c = kind == GBRNG_TAUS ? kCostTaus : kind == GBRNG_LCG ? kCostLcg : kCostRan2;
+    const double one = c.one[w1 - 1], pairs = c.pairs[w2 - 1];
+    const double team = c.team0 + c.team * (double)n / sms +
+                        (c.start0 + c.start * (double)n) / (double)std::max<int64_t>(n_steps, 1);
+    if (team < std::min(one, pairs)) return LD_TEAM;
     return pairs < one ? LD_PAIRS : LD_ONE;
 }
 

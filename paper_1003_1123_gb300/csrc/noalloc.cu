@@ -55,14 +55,7 @@ __global__ void __launch_bounds__(128, 6) ld_noalloc_kernel(NoallocArgs a)
         if (KIND == GBRNG_TAUS) {
             td.y = taus_load(a.taus[i]);
         } else {
-            rd.tab = tab;
-            rd.T = blockDim.x;
-            rd.tid = threadIdx.x;
-            rd.r.idum = a.r2[i];
-            rd.r.idum2 = a.r2[a.S + i];
-            rd.r.iy = a.r2[2 * a.S + i];
-#pragma unroll 4
-            for (int j = 0; j < 32; ++j) tab[j * blockDim.x + threadIdx.x] = a.r2[(3 + j) * a.S + i];
+            rd.load(a.r2 + i, a.S, tab, blockDim.x);
         }
         const float ckx = __fmul_rn(c.ckm, Ki);
         const float hK = 0.5f * Ki;
@@ -86,11 +79,7 @@ __global__ void __launch_bounds__(128, 6) ld_noalloc_kernel(NoallocArgs a)
         } else if (KIND == GBRNG_TAUS) {
             a.taus[i] = td.y;
         } else {
-            a.r2[i] = rd.r.idum;
-            a.r2[a.S + i] = rd.r.idum2;
-            a.r2[2 * a.S + i] = rd.r.iy;
-#pragma unroll 4
-            for (int j = 0; j < 32; ++j) a.r2[(3 + j) * a.S + i] = tab[j * blockDim.x + threadIdx.x];
+            rd.store(a.r2 + i, a.S);
         }
         acc[0] += (double)x0 * x0 + (double)x1 * x1 + (double)x2 * x2;
         acc[1] += (double)v0 * v0 + (double)v1 * v1 + (double)v2 * v2;

@@ -48,12 +48,8 @@ template <int KIND>
 __device__ __forceinline__ float2 normal2(TausDraw& td, LcgDraw& lc, Ran2Draw& rd)
 {
     if (KIND == GBRNG_RAN2) {
-        const float u1 = u01_from_ran2(rd.next());
-        const float u2 = u01_from_ran2(rd.next());
-        const float u3 = u01_from_ran2(rd.next());
-        const float u4 = u01_from_ran2(rd.next());
-        return box_muller_cos2(neg2log2(make_float2(u1, u3)),
-                               __fmul2_rn(splat2(4.0f), make_float2(u2, u4)));
+        const int32_t n1 = rd.next(), n2 = rd.next(), n3 = rd.next(), n4 = rd.next();
+        return box_muller_cos2(ran2_neg2log2<false>(n1, n3), ran2_turns2(n2, n4));
     } else {
         uint32_t r[4];
         if (KIND == GBRNG_TAUS)
@@ -83,14 +79,7 @@ __global__ void __launch_bounds__(256) ou_pt_kernel(OuArgs a)
     } else if (KIND == GBRNG_LCG) {
         lc.x = a.lcg[k];
     } else {
-        rd.tab = tab;
-        rd.T = blockDim.x;
-        rd.tid = threadIdx.x;
-        rd.r.idum = a.r2[k];
-        rd.r.idum2 = a.r2[a.S + k];
-        rd.r.iy = a.r2[2 * a.S + k];
-#pragma unroll 4
-        for (int j = 0; j < 32; ++j) tab[j * blockDim.x + threadIdx.x] = a.r2[(3 + j) * a.S + k];
+        rd.load(a.r2 + k, a.S, tab, blockDim.x);
     }
     float R = live ? a.R[k] : 0.f;
     const float R0 = R;
@@ -127,11 +116,7 @@ __global__ void __launch_bounds__(256) ou_pt_kernel(OuArgs a)
     } else if (KIND == GBRNG_LCG) {
         a.lcg[i] = lc.x;
     } else {
-        a.r2[i] = rd.r.idum;
-        a.r2[a.S + i] = rd.r.idum2;
-        a.r2[2 * a.S + i] = rd.r.iy;
-#pragma unroll 4
-        for (int j = 0; j < 32; ++j) a.r2[(3 + j) * a.S + i] = tab[j * blockDim.x + threadIdx.x];
+        rd.store(a.r2 + i, a.S);
     }
 }
 

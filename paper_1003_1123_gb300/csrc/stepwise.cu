@@ -46,16 +46,16 @@ __global__ void __launch_bounds__(256) step_pt_kernel(StepArgs a)
     } else {
         int32_t* r2 = a.r2;
         const int64_t S = a.S;
-        Ran2Regs r{r2[i], r2[S + i], r2[2 * S + i]};
-        auto iv = [r2, S, i](int j) -> int32_t& { return r2[(3 + j) * S + i]; };
-        const float u1 = u01_from_ran2(ran2_next(r, iv));
-        const float u2 = u01_from_ran2(ran2_next(r, iv));
-        const float u3 = u01_from_ran2(ran2_next(r, iv));
-        const float u4 = u01_from_ran2(ran2_next(r, iv));
-        box_muller3(u1, u2, u3, u4, g0, g1, g2);
+        Ran2Regs r{r2[i], r2[S + i], -r2[2 * S + i]};
+        auto next = [&] {   // the table stays in global memory, entry j in row 3 + j
+            int32_t& e = r2[(3 + (-ran2_row(r.n) & 31)) * S + i];
+            return ran2_step(r, e, e);
+        };
+        const int32_t n[4] = {next(), next(), next(), next()};
+        box_muller3_ran2(n, g0, g1, g2);
         r2[i] = r.idum;
         r2[S + i] = r.idum2;
-        r2[2 * S + i] = r.iy;
+        r2[2 * S + i] = -r.n;
     }
     const float ckx = __fmul_rn(c.ckm, Ki);
     em_component(c.cdt, c.cva, ckx, c.cs, g0, x0, v0);
