@@ -241,8 +241,8 @@ __global__ void __launch_bounds__(64, 8) adjoint_kernel(AdjArgs a)
         acc[1] += dkg.second();
         acc[2] += dT.value();
     }
-    block_reduce_sum<4>(acc, red);
-    if (threadIdx.x < 32) store_stats(a.sink, acc);
+    const double sums = block_sums(acc, red);
+    if (threadIdx.x < 32) store_stats(a.sink, sums);
 }
 
 // Largest noise history (bytes) ld_backward keeps; -1: half the free device

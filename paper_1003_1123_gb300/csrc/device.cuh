@@ -754,45 +754,80 @@ struct EnergySum2 {
     }
 };
 
-// Deterministic block reduction of N doubles per thread (fixed tree order);
-// thread 0 receives the block totals in `v`.  smem must hold N*32 doubles.
+// Sums over a warp of N = 2 or 4 doubles a lane; sum k is in lane k.  Binary64 additions run at about one warp's in 64 cycles a scheduler, so
+// the first levels halve the values instead of the lanes: 6 additions for four sums (5 for
+// two) where one after another takes 20 (10).
 template <int N>
-__device__ __forceinline__ void block_reduce_sum(double (&v)[N], double* smem)
+__device__ __forceinline__ double warp_sums(const double (&v)[N])
+{
+    const int lane = threadIdx.x & 31;
+    double a[N];
+#pragma unroll
+    for (int k = 0; k < N; ++k) a[k] = v[k];
+    int o = 16;
+#pragma unroll
+    for (int m = N / 2; m > 0; m >>= 1, o >>= 1) {
+        const bool up = lane & o;
+#pragma unroll
+        for (int k = 0; k < m; ++k) {
+            const double other = __shfl_xor_sync(0xffffffffu, up ? a[k] : a[k + m], o);
+            a[k] = (up ? a[k + m] : a[k]) + other;
+        }
+    }
+#pragma unroll
+    for (o = 16 / N; o > 0; o >>= 1) a[0] += __shfl_xor_sync(0xffffffffu, a[0], o);
+    return __shfl_sync(0xffffffffu, a[0], lane * (32 / N) & 31);
+}
+
+// Of sums that stand in lanes k, k + N, ... (k < N): in lane k.
+template <int N>
+__device__ __forceinline__ double warp_sums_strided(double a)
+{
+#pragma unroll
+    for (int o = 16; o >= N; o >>= 1) a += __shfl_xor_sync(0xffffffffu, a, o);
+    return a;
+}
+
+// Deterministic block reduction of N = 2 or 4 doubles per thread (fixed tree order);
+// lane k of the first warp receives sum k.  smem must hold N*32 doubles.
+template <int N>
+__device__ __forceinline__ double block_sums(const double (&v)[N], double* smem)
 {
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int nwarps = (blockDim.x + 31) >> 5;
-#pragma unroll
-    for (int k = 0; k < N; ++k)
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) v[k] += __shfl_down_sync(0xffffffffu, v[k], o);
-    if (lane == 0)
-#pragma unroll
-        for (int k = 0; k < N; ++k) smem[k * 32 + warp] = v[k];
+    double a = warp_sums(v);
+    if (lane < N) smem[warp * N + lane] = a;
     __syncthreads();
     if (warp == 0) {
-#pragma unroll
-        for (int k = 0; k < N; ++k) {
-            v[k] = lane < nwarps ? smem[k * 32 + lane] : 0.0;
-#pragma unroll
-            for (int o = 16; o > 0; o >>= 1) v[k] += __shfl_down_sync(0xffffffffu, v[k], o);
-        }
+        a = 0.0;
+        for (int w = lane / N; w < nwarps; w += 32 / N) a += smem[w * N + lane % N];
+        a = warp_sums_strided<N>(a);
     }
     __syncthreads();
+    return a;
 }
 
-// Sum over a warp's first LANES lanes (a power of two), in lane 0.
-template <int LANES = 32>
+// The same with all sums in the first thread's v.
+template <int N>
+__device__ __forceinline__ void block_reduce_sum(double (&v)[N], double* smem)
+{
+    const double a = block_sums(v, smem);
+#pragma unroll
+    for (int k = 0; k < N; ++k) v[k] = __shfl_sync(0xffffffffu, a, k);
+}
+
+// Sum over a warp, in its first lane.
 __device__ __forceinline__ double warp_sum(double v)
 {
 #pragma unroll
-    for (int o = LANES / 2; o > 0; o >>= 1) v += __shfl_down_sync(0xffffffffu, v, o);
+    for (int o = 16; o > 0; o >>= 1) v += __shfl_down_sync(0xffffffffu, v, o);
     return v;
 }
 
 // A run's statistics: each block's four sums in partials[block][4]; with out (in
 // mapped host memory) the last block to finish adds them up in a fixed order and
 // leaves the ticket at zero for the next launch.  Called by one whole warp of
-// every block, v in its lane 0.  In place of a second kernel this is 4 us less
+// every block, sum k in its lane k.  In place of a second kernel this is 4 us less
 // on a call, as long as one warp's pass over the partials is short: kFuseBlocks.
 struct StatsSink {
     double* partials = nullptr;   // null: no statistics
@@ -801,32 +836,25 @@ struct StatsSink {
 };
 constexpr int64_t kFuseBlocks = 1024;
 
-__device__ __forceinline__ void store_stats(const StatsSink& s, const double (&v)[4])
+__device__ __forceinline__ void store_stats(const StatsSink& s, double v)
 {
     const int lane = threadIdx.x & 31;
-    if (lane == 0)
-#pragma unroll
-        for (int k = 0; k < 4; ++k) s.partials[4 * (int64_t)blockIdx.x + k] = v[k];
+    if (lane < 4) s.partials[4 * (int64_t)blockIdx.x + lane] = v;
     if (!s.out) return;
     int last = 0;
+    __syncwarp();
     if (lane == 0) {
         __threadfence();
         last = atomicAdd(s.ticket, 1u) == gridDim.x - 1;
         __threadfence();
     }
     if (!__shfl_sync(0xffffffffu, last, 0)) return;
-    double t[4] = {0, 0, 0, 0};
+    double t = 0;   // lane 4 j + k: sum k of blocks j, j + 8, ...
 #pragma unroll 4
-    for (unsigned b = lane; b < gridDim.x; b += 32)
-#pragma unroll
-        for (int k = 0; k < 4; ++k) t[k] += __ldcg(s.partials + 4 * (int64_t)b + k);
-#pragma unroll
-    for (int k = 0; k < 4; ++k) t[k] = warp_sum(t[k]);
-    if (lane == 0) {
-#pragma unroll
-        for (int k = 0; k < 4; ++k) s.out[k] = t[k];
-        *s.ticket = 0;
-    }
+    for (unsigned i = lane; i < 4 * gridDim.x; i += 32) t += __ldcg(s.partials + i);
+    t = warp_sums_strided<4>(t);
+    if (lane < 4) s.out[lane] = t;
+    if (lane == 0) *s.ticket = 0;
 }
 
 // Cheap global-timer read for bounded waits.

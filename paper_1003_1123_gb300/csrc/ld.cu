@@ -101,8 +101,8 @@ __global__ void __launch_bounds__(128, KIND == GBRNG_LCG ? 7 : 6) ld_pt_kernel(L
         acc[3] += es.value(hK, c.hm);
     }
     if (a.sink.partials) {
-        block_reduce_sum<4>(acc, red);
-        if (threadIdx.x < 32) store_stats(a.sink, acc);
+        const double sums = block_sums(acc, red);
+        if (threadIdx.x < 32) store_stats(a.sink, sums);
     }
 }
 
@@ -199,8 +199,8 @@ __global__ void __launch_bounds__(32) ld_pair_kernel(LdArgs a, int64_t n_pairs)
         }
     }
     if (a.sink.partials) {
-        block_reduce_sum<4>(acc, red);
-        if (threadIdx.x < 32) store_stats(a.sink, acc);
+        const double sums = block_sums(acc, red);
+        if (threadIdx.x < 32) store_stats(a.sink, sums);
     }
 }
 

@@ -48,15 +48,12 @@ __global__ void __launch_bounds__(32 * (NW + GW + 1), 1) lfg_ou_kernel(OuLfgArgs
         // sums of positions Ra (and Rb) of the unit at lane's particle j into record rec
         auto record = [&](int64_t rec, int u, int j, float Ra, float Rb) {
             const float* R0 = ou_sm + n_pad + j;
-            double m = j < nc ? (double)Ra : 0.0, q = j < nc ? (double)Ra * (double)R0[0] : 0.0;
-            if (!STEPS && j + 1 < nc) m += (double)Rb, q += (double)Rb * (double)R0[1];
-            m = warp_sum(m), q = warp_sum(q);
-            if (lane == 0) {
-                double* d = o.records + 2 * ((rec * gridDim.x + blockIdx.x) * o.slots + warp);
-                if (u == warp)
-                    d[0] = m, d[1] = q;
-                else
-                    d[0] += m, d[1] += q;
+            double v[2] = {j < nc ? (double)Ra : 0.0, j < nc ? (double)Ra * (double)R0[0] : 0.0};
+            if (!STEPS && j + 1 < nc) v[0] += (double)Rb, v[1] += (double)Rb * (double)R0[1];
+            const double sum = warp_sums(v);
+            if (lane < 2) {
+                double* d = o.records + 2 * ((rec * gridDim.x + blockIdx.x) * o.slots + warp) + lane;
+                *d = u == warp ? sum : *d + sum;
             }
         };
         if (o.records)

@@ -140,8 +140,8 @@ __global__ void __launch_bounds__(32 * (CW + GW + 1), 1) lfg_resident_kernel(Lfg
     }
     if (a.sink.partials) {
         acc[3] = e.value();
-        block_reduce_sum<4>(acc, red);
-        if (warp == 0) store_stats(a.sink, acc);
+        const double sums = block_sums(acc, red);
+        if (warp == 0) store_stats(a.sink, sums);
     }
 }
 
@@ -281,8 +281,8 @@ __global__ void __launch_bounds__(32 * (CW + GW + 1), 1) lfg_stream_kernel(LfgAr
         __syncthreads();
         if (s_failed) return;
         acc[3] = e.value();
-        block_reduce_sum<4>(acc, red);
-        if (warp == 0) store_stats(a.sink, acc);
+        const double sums = block_sums(acc, red);
+        if (warp == 0) store_stats(a.sink, sums);
     }
 }
 
@@ -322,8 +322,8 @@ __global__ void snapshot_kernel(const float* x, const float* v, int64_t n, Stats
         acc[1] += vi * vi;
         acc[2] += xi * vi;
     }
-    block_reduce_sum<4>(acc, red);
-    if (threadIdx.x < 32) store_stats(sink, acc);
+    const double sums = block_sums(acc, red);
+    if (threadIdx.x < 32) store_stats(sink, sums);
 }
 
 // The resident kernel takes a system whose step fits a round (4 N <= k D) and

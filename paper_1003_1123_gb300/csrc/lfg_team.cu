@@ -33,14 +33,20 @@ struct LfgTeamArgs {
 constexpr int kTeamUse = 15, kTeamGen = 16, kTeamThreads = 32 * (kTeamUse + kTeamGen + 1);
 constexpr int BAR_NORMALS = 3;
 
-// Sum of a double over the using warps, in their first thread; sm: kTeamUse doubles.
-__device__ __forceinline__ double use_sum(double v, double* sm)
+// Sums of N doubles over the using warps, sum k in lane k of the first; sm: N kTeamUse
+// doubles.
+template <int N>
+__device__ __forceinline__ double use_sums(const double (&v)[N], double* sm)
 {
-    v = warp_sum(v);
-    if ((threadIdx.x & 31) == 0) sm[threadIdx.x >> 5] = v;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    double t = warp_sums(v);
+    if (lane < N) sm[warp * N + lane] = t;
     bar_sync(BAR_NORMALS, 32 * kTeamUse);
-    double t = threadIdx.x < kTeamUse ? sm[threadIdx.x] : 0.0;
-    if (threadIdx.x < 32) t = warp_sum(t);
+    if (warp == 0) {
+        t = 0.0;
+        for (int i = lane; i < N * kTeamUse; i += 32) t += sm[i];
+        t = warp_sums_strided<N>(t);
+    }
     bar_sync(BAR_NORMALS, 32 * kTeamUse);
     return t;
 }
@@ -84,13 +90,9 @@ __global__ void __launch_bounds__(kTeamThreads, 1) lfg_team_kernel(LfgTeamArgs o
     Kahan2 e;   // LD: sums of x^2 and v^2
     int64_t t = 0, rec = 0, next_rec = 0;
     auto record = [&](float Rt) {
-        const double m = use_sum(live ? (double)Rt : 0.0, red);
-        const double c = use_sum(live ? (double)Rt * (double)R0 : 0.0, red);
-        if (tid == 0) {
-            double* d = o.records + 2 * (rec * gridDim.x + blockIdx.x);
-            d[0] = m;
-            d[1] = c;
-        }
+        const double v[2] = {live ? (double)Rt : 0.0, live ? (double)Rt * (double)R0 : 0.0};
+        const double sum = use_sums(v, red);
+        if (tid < 2) o.records[2 * (rec * gridDim.x + blockIdx.x) + tid] = sum;
         ++rec;
         next_rec += o.every;
     };
@@ -183,9 +185,8 @@ __global__ void __launch_bounds__(kTeamThreads, 1) lfg_team_kernel(LfgTeamArgs o
             acc[2] = (double)x * v;
             acc[3] = (double)hK * ((double)e.s.x - (double)e.c.x) + (double)a.c.hm * ((double)e.s.y - (double)e.c.y);
         }
-#pragma unroll
-        for (int k = 0; k < 4; ++k) acc[k] = use_sum(acc[k], red);
-        if (warp == 0) store_stats(a.sink, acc);
+        const double sums = use_sums(acc, red);
+        if (warp == 0) store_stats(a.sink, sums);
     }
 }
 

@@ -56,10 +56,11 @@ __device__ __forceinline__ float2 normal2(TausDraw& td, LcgDraw& lc, Ran2Draw& r
             taus_draws(td.y, r);
         else
             lcg_draws(lc.x, r);
-        const float2 u = make_float2(open01_from_u32(r[0]), open01_from_u32(r[2]));
+        const float2 u = KIND == GBRNG_TAUS ? make_float2(open01_scaled(r[0]), open01_scaled(r[2]))
+                                             : make_float2(open01_from_u32(r[0]), open01_from_u32(r[2]));
         const float2 x = __ffma2_rn(splat2(4.0f), make_float2(mant_from_u32(r[1]), mant_from_u32(r[3])),
                                     splat2(-0x1.fffffep+1f));
-        return box_muller_cos2(neg2log2(u), x);
+        return box_muller_cos2(neg2log2<KIND == GBRNG_TAUS>(u), x);
     }
 }
 
@@ -88,26 +89,26 @@ __global__ void __launch_bounds__(256) ou_pt_kernel(OuArgs a)
         if (a.partials && t == next_rec) {
             next_rec += a.every;
             double v[2] = {live ? (double)R : 0.0, live ? (double)R * (double)R0 : 0.0};
-            block_reduce_sum<2>(v, red);
-            if (threadIdx.x == 0) {
-                double* o = a.partials + 2 * (rec * gridDim.x + blockIdx.x);
-                o[0] = v[0];
-                o[1] = v[1];
-            }
+            const double sum = block_sums(v, red);
+            if (threadIdx.x < 2) a.partials[2 * (rec * gridDim.x + blockIdx.x) + threadIdx.x] = sum;
             ++rec;
         }
         if (t == a.n_steps) break;
-        if (t + 1 < a.n_steps && !(a.partials && t + 1 == next_rec)) {
-            // two steps with no record between them
+        const int64_t end = a.partials ? min(next_rec, a.n_steps) : a.n_steps;
+        int64_t pairs = (end - t) >> 1;
+// four pairs of steps an iteration (1e6 x 300, one pair / four: Hybrid Taus 602 / 553
+// us, the LCG 447 / 392, Ran2 788 / 736)
+#pragma unroll 4
+        for (; pairs > 0; --pairs) {   // two steps with no record between them
             const float2 g = normal2<KIND>(td, lc, rd);
             R = __fmaf_rn(a.c.cs, g.x, __fmaf_rn(-a.c.c1, R, R));
             R = __fmaf_rn(a.c.cs, g.y, __fmaf_rn(-a.c.c1, R, R));
-            t += 2;
-        } else {
+        }
+        if ((end - t) & 1) {
             const float g = normal1<KIND>(td, lc, rd);
             R = __fmaf_rn(a.c.cs, g, __fmaf_rn(-a.c.c1, R, R));
-            t += 1;
         }
+        t = end;
     }
     if (!live || a.n_steps == 0) return;
     a.R[i] = R;
@@ -173,16 +174,23 @@ int ou_run_pt(const ou_system* s, int64_t n_steps, int64_t every, double* mean, 
               cudaStream_t st)
 {
     Handle* h = s->rng;
-    const int T = 256;
-    const int64_t blocks = (s->n + T - 1) / T;
+    DevInfo di;
+    GB_CHECK(dev_info(h->device, &di));
     const bool rec = mean != nullptr;
     const int64_t n_rec = n_steps / every + 1;
+    // 256 threads a block, or 128 where that leaves the busiest SM fewer warps (1e4
+    // particles x 1000 steps 112 -> 84 us for Hybrid Taus, 4e4 175 -> 142, 2e5 x 200
+    // 125 -> 114; elsewhere, with twice the blocks to sum up, up to 2% slower)
+    auto too_many = [&](int64_t blocks) { return n_rec > 0x7fffffff || (double)n_rec * blocks * 16.0 > 4.0 * (1 << 30); };
+    auto busiest = [&](int64_t threads) { return threads * (((s->n + threads - 1) / threads + di.sms - 1) / di.sms); };
+    const int T = busiest(128) < busiest(256) && !(rec && too_many((s->n + 127) / 128)) ? 128 : 256;
+    const int64_t blocks = (s->n + T - 1) / T;
     int64_t team_blocks = 0;
     const int rc = ou_team(s, n_steps, every, rec, &team_blocks, st);
     if (rc < 0) return rc;
     if (rc == 1) return rec ? ou_finish(h, s->n, n_rec, team_blocks, mean, corr, st) : GBRNG_OK;
     if (rec) {
-        if (n_rec > 0x7fffffff || (double)n_rec * blocks * 16.0 > 4.0 * (1 << 30))
+        if (too_many(blocks))
             return fail(GBRNG_EINVAL, "%lld records x %lld blocks exceed the record scratch",
                         (long long)n_rec, (long long)blocks);
         GB_CHECK(ensure_partials(h, (2 * n_rec * blocks + 2 * n_rec + 3) / 4));

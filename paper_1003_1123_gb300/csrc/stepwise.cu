@@ -87,8 +87,8 @@ __global__ void step_stats_kernel(const float* x, const float* v, const float2* 
         }
         acc[3] += (double)eacc[i].x - (double)eacc[i].y;
     }
-    block_reduce_sum<4>(acc, red);
-    if (threadIdx.x < 32) store_stats(sink, acc);
+    const double sums = block_sums(acc, red);
+    if (threadIdx.x < 32) store_stats(sink, sums);
 }
 
 int stepwise_stats(Handle* h, const ld_system* s, int64_t n_steps, ld_stats* out, cudaStream_t st)

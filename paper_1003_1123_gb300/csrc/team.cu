@@ -30,8 +30,7 @@
 // 16 a block / 8 a block, us: 1000 oscillators 133 / 26.8 / 17.4; 4096 133 / 39.1
 // / 37.0; 1e4 134 / 78.1 / 72.0; 2e4 206 / 130 / 129; 5e4 312 / 286 / 303; 1e5
 // 602 / 562 / 591 (bound there by the issue of about 15% more instructions than
-// one oscillator a thread needs, the jumps and the hand-over).  Overdamped, 1000
-// steps: 1e4 117 / 45.2 / 51.4; 5e4 187 / 152 / 199; 1e5 275 / 294 / 386.
+// one oscillator a thread needs, the jumps and the hand-over).
 #include <algorithm>
 #include <type_traits>
 
@@ -375,9 +374,7 @@ __device__ __forceinline__ void team_consume_ld(const TeamArgs& a, float* buf, i
     const int64_t ie = first + lane % G;
     if (lane < 2 * G && ie < a.n)
         acc[3] = (double)(lane < G ? 0.5f * (a.Kper ? a.Kper[ie] : c.K) : c.hm) * K.value();
-#pragma unroll
-    for (int k = 0; k < 4; ++k) acc[k] = warp_sum(acc[k]);
-    store_stats(a.sink, acc);
+    store_stats(a.sink, warp_sums(acc));
 }
 
 // Consumer of the overdamped particles, a lane each; records between steps.
@@ -385,22 +382,20 @@ template <class S>
 __device__ __forceinline__ void team_consume_ou(const TeamArgs& a, float* buf, int bar_threads)
 {
     constexpr int G = S::kOsc;
-    static_assert(G <= 32, "a lane a particle");
+    static_assert(2 * G <= 32, "two lanes a particle");
     const int lane = threadIdx.x & 31;
-    const int64_t i = blockIdx.x * (int64_t)G + lane;
-    const bool live = lane < G && i < a.n;
+    // lanes beyond the first G repeat them: a record's sum of R is theirs, R R(0) the next G's
+    const int64_t i = blockIdx.x * (int64_t)G + lane % G;
+    const bool live = i < a.n;
     float R = live ? a.x[i] : 0.f;
     const float R0 = R, c1 = a.oc.c1, cs = a.oc.cs;
     int64_t t = 0, rec = 0, next_rec = 0;
     // record of the positions Rt after t steps
     auto record = [&](float Rt) {
-        const double m = warp_sum<G>(live ? (double)Rt : 0.0);
-        const double q = warp_sum<G>(live ? (double)Rt * (double)R0 : 0.0);
-        if (lane == 0) {
-            double* o = a.records + 2 * (rec * gridDim.x + blockIdx.x);
-            o[0] = m;
-            o[1] = q;
-        }
+        double v = !live ? 0.0 : lane & G ? (double)Rt * (double)R0 : (double)Rt;
+#pragma unroll
+        for (int o = G / 2; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+        if (lane == 0 || lane == G) a.records[2 * (rec * gridDim.x + blockIdx.x) + lane / G] = v;
         ++rec;
         next_rec += a.every;
     };
@@ -414,8 +409,18 @@ __device__ __forceinline__ void team_consume_ou(const TeamArgs& a, float* buf, i
         a, buf, lane % G, bar_threads, [](float*) {},
         [&](const float* p) {
             if (a.every < S::kChunk && next_rec != INT64_MAX) {   // several records a chunk
-#pragma unroll 1
-                for (int k = 0; k < S::kChunk; ++k) one(p + k * S::kStepWords);
+                // the positions take the normals' places, and the records theirs from there
+                float* pos = const_cast<float*>(p);
+                float g[S::kChunk];
+                load_chunk<S>(p, g);
+                __syncwarp();
+#pragma unroll
+                for (int k = 0; k < S::kChunk; ++k) {
+                    R = __fmaf_rn(cs, g[k], __fmaf_rn(-c1, R, R));
+                    pos[k * S::kStepWords] = R;
+                }
+                while (next_rec <= t + S::kChunk) record(pos[(next_rec - t - 1) * S::kStepWords]);
+                t += S::kChunk;
                 return;
             }
             // at most one record inside: keep the positions of its step
@@ -431,7 +436,7 @@ __device__ __forceinline__ void team_consume_ou(const TeamArgs& a, float* buf, i
             if (at > 0) record(Rt);
         },
         one, [](const float*) {});
-    if (live) a.x[i] = R;
+    if (live && lane < G) a.x[i] = R;
 }
 
 template <int MODEL, int KIND, int PAIRS, int M>
@@ -494,8 +499,10 @@ int ld_team(const ld_system* s, int64_t n_steps, ld_stats* out, cudaStream_t st)
     return finish_stats(h, a.sink, blocks, n_steps, out, st);
 }
 
-// Overdamped runs of at most 448 particles a SM (6.8e4: above, one particle a
-// thread is faster), of enough steps for the blocks' start-up (as in ld_run).
+// Overdamped runs of few particles, of enough steps for the blocks' start-up, some
+// 0.6 us per 1000 particles (Hybrid Taus, one a thread / team, us: 5000 particles x 100
+// steps 36 / 31; 1e4 x 200 41 / 43, x 400 50 / 48, x 1000 81 / 64; 2e4 x 400 63 / 63,
+// x 1000 108 / 92; 4e4 x 1000 140 / 146, x 4000 474 / 441; 6e4 x 4000 591 / 628).
 // Returns 1 and the number of blocks when it has launched, else 0 or an error.
 int ou_team(const ou_system* s, int64_t n_steps, int64_t every, bool rec, int64_t* blocks_out, cudaStream_t st)
 {
@@ -503,7 +510,8 @@ int ou_team(const ou_system* s, int64_t n_steps, int64_t every, bool rec, int64_
     if (h->kind != GBRNG_TAUS && h->kind != GBRNG_LCG) return 0;
     DevInfo di;
     GB_CHECK(dev_info(h->device, &di));
-    if (s->n > (int64_t)448 * di.sms || n_steps < 48 || n_steps < s->n / 100) return 0;
+    const int64_t per_sm = s->n / di.sms;
+    if (per_sm >= 256 || n_steps < 48 || (per_sm >= 48 && n_steps < s->n / (per_sm < 128 ? 32 : 16))) return 0;
     const bool small = s->n <= (int64_t)16 * di.sms;
     const int64_t blocks = small ? (s->n + 7) / 8 : (s->n + 15) / 16, n_rec = n_steps / every + 1;
     if (rec) {
