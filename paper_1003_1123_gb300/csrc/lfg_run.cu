@@ -288,8 +288,8 @@ __global__ void __launch_bounds__(32 * (CW + GW + 1), 1) lfg_stream_kernel(LfgAr
 
 // ------------------------------------------------------------- host side
 // Using and generating warps.  The resident kernel: 15 and 16 at 64 registers; per
-// step of 1e6 oscillators 7.4 us against 9.1 with 19 and 8, 8.3 with 19 and 12 (the
-// generating warps' loads in flight bound a phase: with none generated it takes 5.2).
+// step of 1e6 oscillators 7.1 us (when it was 7.4, 9.1 with 19 and 8, 8.3 with 19 and 12: the
+// generating warps' loads in flight bound a round: with none generated it took 5.2).
 // The streamed one has more work a word in its using warps: 15 and 8 (1e7: 159 us
 // a step, 164 with 11 and 12, 169 with 11 and 16) where a round has its full width;
 // below 2 N >= k D the narrower rounds leave less time to generate: 11 and 16 (1.2e6:
