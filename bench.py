@@ -57,8 +57,8 @@ WORKLOAD = ("N=1e6 3-D oscillators x 1e4 fused steps per generator (Taus, Ran2, 
             "systems (N 1e2..1e5) x 5000 batched steps + adjoint (Taus, Ran2) of 1e5 "
             "oscillators x 1e4 steps")
 
-# Minimal integer-ALU-pipe instructions a draw needs, given the instruction
-# set (LOP3 evaluates any three-input logic function, SHF is one shift, and
+# Integer-ALU-pipe instructions a draw needs as the algorithm is printed, given the
+# instruction set (LOP3 evaluates any three-input logic function, SHF is one shift, and
 # left shifts, multiplies and adds can run as IMAD on the FMA pipe instead):
 #   Hybrid Taus, per Tausworthe word ((y << s1) ^ y) >> s2, ((y & c) << s3) ^ b:
 #     the xor (LOP3), the right shift (SHF) and the masked xor (LOP3) = 3, the
@@ -70,8 +70,10 @@ WORKLOAD = ("N=1e6 3-D oscillators x 1e4 fused steps per generator (Taus, Ran2, 
 #     two of them 6; the slot index iy / NDIV (multiply-high on IMAD, one SHF)
 #     1; the wrap of iy as min_u32(y, y + m1 - 1) 1 -> 8 per draw, 32 per
 #     oscillator-step.
-# A lower bound on the work of the 64-lane ALU pipe, so no part can read above
-# 1.0 against it; ncu's measured ALU-pipe utilisation is reported beside it.
+# A fixed yardstick for the 64-lane ALU pipe.  The Hybrid Taus kernels need fewer since
+# they step the words by funnel shifts (29 an oscillator-step), so for them it is a rate
+# in the printed algorithm's operations and no lower bound; ncu's measured ALU-pipe
+# utilisation is reported beside it.
 INT_OPS_PER_DRAW = {"taus": 11, "ran2": 8}
 INT_OPS_PER_OSC_STEP = {k: 4 * v for k, v in INT_OPS_PER_DRAW.items()}
 # Algorithmic bytes per oscillator-step of the Lagged Fibonacci fused step at

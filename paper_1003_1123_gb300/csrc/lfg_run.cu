@@ -287,14 +287,15 @@ __global__ void __launch_bounds__(32 * (CW + GW + 1), 1) lfg_stream_kernel(LfgAr
 }
 
 // ------------------------------------------------------------- host side
-// Using and generating warps.  The resident kernel: 15 and 16 at 64 registers; per
-// step of 1e6 oscillators 7.1 us (when it was 7.4, 9.1 with 19 and 8, 8.3 with 19 and 12: the
-// generating warps' loads in flight bound a round: with none generated it took 5.2).
-// The streamed one has more work a word in its using warps: 15 and 8 (1e7: 159 us
-// a step, 164 with 11 and 12, 169 with 11 and 16) where a round has its full width;
-// below 2 N >= k D the narrower rounds leave less time to generate: 11 and 16 (1.2e6:
-// 18.4 us a step, 22.8 with 15 and 8).
-constexpr int kResWarps = 15, kResGen = 16;
+// Using and generating warps, whose sum also sets the registers a thread has.  The
+// resident kernel: 15 and 12, per step of 1e6 oscillators 6.80 us (7.08 with 15 and 16,
+// 7.04 with 14 and 13, 7.12 with 13 and 14, 7.3 with 15 or 16 and 11, 7.8 with 15 and 8:
+// the generating warps' loads in flight and the using warps' arithmetic share a round).
+// The streamed one has more work a word in its using warps: 13 and 10 (1e7: 136 us a
+// step, 138 with 15 and 8, 141 with 12 and 11, 144 with 11 and 12) where a round has its
+// full width; below 2 N >= k D the narrower rounds leave less time to generate: 11 and 12
+// (1.2e6: 17.7 us a step, 18.1 with 11 and 16, 18.0 with 13 and 14, 20.1 with 15 and 12).
+constexpr int kResWarps = 15, kResGen = 12;
 
 template <int MODE, int CW, int GW>
 static int launch_stream(Handle* h, LfgArgs& a, int k, cudaStream_t st)
@@ -385,9 +386,9 @@ int lfg_ld(const ld_system* s, int64_t n_steps, int init, ld_stats* out, cudaStr
     } else {
         a.w = (int)(std::min<int64_t>((int64_t)k * a.D, 2 * s->n) & ~(int64_t)7);
         if (2 * s->n < (int64_t)k * a.D)
-            GB_CHECK((launch_stream<LFG_LD, 11, 16>(h, a, k, st)));
+            GB_CHECK((launch_stream<LFG_LD, 11, 12>(h, a, k, st)));
         else
-            GB_CHECK((launch_stream<LFG_LD, 15, 8>(h, a, k, st)));
+            GB_CHECK((launch_stream<LFG_LD, 13, 10>(h, a, k, st)));
     }
     GB_CHECK(lfg_end(h, a, st));
     h->pos += a.n_pos;

@@ -27,10 +27,10 @@
 // Two shapes.  16 oscillators a block (16 chunks a pass, 50 KB: four blocks a SM)
 // and, for the fewest oscillators, 8 a block (32 chunks), which spreads the
 // consumers' chains wider.  Hybrid Taus x 1000 steps, one oscillator a thread /
-// 16 a block / 8 a block, us: 1000 oscillators 133 / 26.8 / 17.4; 4096 133 / 39.1
-// / 37.0; 1e4 134 / 78.1 / 72.0; 2e4 206 / 130 / 129; 5e4 312 / 286 / 303; 1e5
-// 602 / 562 / 591 (bound there by the issue of about 15% more instructions than
-// one oscillator a thread needs, the jumps and the hand-over).
+// 16 a block / 8 a block, us: 1000 oscillators 119 / 22.6 / 14.5; 4096 119 / 32.9
+// / 32.9; 1e4 119 / 67.7 / 63.6; 2e4 193 / 113 / 112; 5.8e4 287 / 287 (bound there by
+// the issue of the instructions that one oscillator a thread does not need, the jumps and
+// the hand-over).
 #include <algorithm>
 #include <type_traits>
 
