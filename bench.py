@@ -87,25 +87,27 @@ LFG_BYTES_PER_OSC_STEP = 48
 LFG_XV_BYTES_PER_OSC_STEP = 48
 L2_COPY_BYTES = 32 << 20
 FILL_BYTES_PER_NUMBER = 4
-# A Lagged Fibonacci fill number: 2 lag reads + 1 ring write + 1 output write
-# of 4 B, all through L2 (the ring stays there; the output streams on to HBM).
+# A Lagged Fibonacci fill number as the recurrence is printed: 2 lag reads + 1 ring
+# write + 1 output write of 4 B, all through L2 (the ring stays there; the output streams
+# on to HBM).  The fans read 1.5 words a number instead of 2, and L2 serves more than a
+# copy's bandwidth, so the fraction of the copy can pass 1.
 LFG_FILL_BYTES_PER_NUMBER = 16
 # DRAM bytes (read + written) of one launch of a part's kernel from the ncu
 # capture summarised in profiles/ (same kernel, same launch shape), keyed by
 # part and the batched tuner's (T, K, steps per launch); reported as the
 # roofline's `traffic` only when this run chose that shape.
-NCU_TRAFFIC = {("batched_taus", (64, 2, 0)): 303.498496e6 + 237.612032e6}
+NCU_TRAFFIC = {("batched_taus", (64, 2, 0)): 302.788864e6 + 237.262336e6}
 # ncu's ALU-pipe utilisation (sm__pipe_alu_cycles_active, % of peak sustained
 # active) of each ALU-bound part's kernel, from the captures summarised in
 # profiles/alu_pipe_by_part.md (same kernel and launch shape as the bench;
 # 100 steps of the 1e6-oscillator systems, 1000 steps of the adjoint, 2^28
 # fill numbers, the batched graph's replay; the large parts at 1e7
 # oscillators x 10 steps).
-NCU_ALU_PIPE_PCT = {"ld_taus": 69.5, "batched_taus": 69.7, "ld_ran2": 47.7,
-                    "adjoint_taus": 60.2, "adjoint_ran2": 42.2,
-                    "fill_uniform_taus": 89.1, "fill_normal_taus": 77.8,
-                    "fill_uniform_ran2": 65.5, "fill_normal_ran2": 63.3,
-                    "ld_taus_1e8": 56.0, "ld_ran2_1e8": 39.5}
+NCU_ALU_PIPE_PCT = {"ld_taus": 59.4, "batched_taus": 59.9, "ld_ran2": 51.3,
+                    "adjoint_taus": 52.4, "adjoint_ran2": 46.4,
+                    "fill_uniform_taus": 82.6, "fill_normal_taus": 70.4,
+                    "fill_uniform_ran2": 73.2, "fill_normal_ran2": 56.6,
+                    "ld_taus_1e8": 42.9, "ld_ran2_1e8": 39.3}
 
 
 def load_peaks():
@@ -370,7 +372,8 @@ def run_gpu(args, rank, world, dist):
         "data": "synthetic (seeded oscillators; equilibrium start)",
         "config": bench_config(world, extras["batched_osc"]),
         "clocks": clk,
-        "gpu_launches": gpu_launches(parts, args.steps, extras["batched_tune"]),
+        "gpu_launches": gpu_launches(parts, args.steps, extras["batched_tune"])
+        - in_kernel_statistics(parts) * args.steps,
         "batched_tune": extras["batched_tune"],
         "e2e": e2e,
         "roofline": roof,
@@ -472,6 +475,12 @@ def gpu_launches(parts, steps, batched_tune=None):
         else:
             n += 1
     return n * steps
+
+
+def in_kernel_statistics(parts):
+    """Runs whose last block adds the statistics up, with no finisher of their own: the
+    Lagged Fibonacci run, of one block an SM."""
+    return sum(name.startswith("ld_lagfib") for name, _, _ in parts)
 
 
 def compare_paths(wl, G, torch, part_ms, steps):
@@ -626,7 +635,7 @@ def part_kind(part: str) -> str:
 def roofline(part, ms, units, peaks, src, clk, l2_gbs=None):
     """Roofline of one part against its binding resource.
     - Taus/Ran2 fused, batched and adjoint: the 64-lane integer ALU pipe, with
-      the minimal ALU instructions of the generator's draws (INT_OPS_PER_DRAW;
+      the ALU instructions of the generator's printed draws (INT_OPS_PER_DRAW;
       four draws an oscillator-step, drawn twice by the adjoint, whose reverse
       sweep regenerates the noise), and ncu's measured ALU-pipe utilisation
       beside it where a capture exists.
@@ -1000,7 +1009,10 @@ def run_sweep():
         s = G.LdSystem(r, x, torch.zeros_like(x), **PARAMS)
         G.ld_init_equilibrium(s)
         sl, ll = G.rng_lfg_lags(row)
-        ring = (2 * ll + 2 * (ll - sl) + 31) // 32 * 32
+        # three rounds of the deepest fan (K of 16, 8, 4, 2 with K (ll - sl) <= 4.1e6)
+        k = next((k for k in (16, 8, 4) if k * (ll - sl) <= 4100000), 2)
+        d = ll - sl
+        ring = (max(3 * k * d, (k + 1) * d + k * sl) + 31) // 32 * 32
         lag_rows.append({"row": row, "sl": sl, "ll": ll, "ring_bytes": 4 * ring,
                          "portable_state_bytes": G.rng_state_bytes(r),
                          "ms_per_1000": timed(lambda: G.ld_run(s, steps, stats=False))})

@@ -325,8 +325,8 @@ int ld_set_adjoint_history_limit(int64_t bytes);
  * reads the statistics back and synchronises the stream (the host waits for
  * the run); on a stream in capture mode that is refused with GBRNG_EINVAL
  * before any work is queued.  It runs one oscillator a thread, so Hybrid Taus
- * systems that fill a resident wave run about 4% slower than in ld_run, which
- * takes two.  Other requirements and errors as ld_run. */
+ * and Ran2 systems that fill a resident wave run about 16 and 19% slower than in
+ * ld_run, which takes two.  Other requirements and errors as ld_run. */
 int ld_run_noalloc(ld_system* sys, int64_t n_steps, ld_stats* out_host, void* stream);
 
 /* ----------------------------------------------------------------- errors */

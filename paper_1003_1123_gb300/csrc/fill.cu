@@ -84,10 +84,11 @@ __global__ void __launch_bounds__(256) word_fill_kernel(State* __restrict__ st, 
 // that the states are read, by the cluster's barrier, before any thread replaces
 // one; clusters keep B, the streams that a row of stores covers, at least 32 (2^27
 // uniforms of 4096 streams: 434 us with 16 in one block, 148 with 32, 181 with 64 and
-// twice the blocks a cluster).  One thread a stream / segments, us: 2^20 words of
-// 4096 streams 12.4 / 6.3; 2^24 uniforms of 1024 559 / 22.7; 2^27 of 4096 1118 / 148,
-// of 2e4 233 / 173, of 5e4 176 / 140; 2^27 normals of 4096 1868 / 208.  (From 7e4
-// streams on a thread a stream is faster: 115 against 123 us.)
+// twice the blocks a cluster).  One thread a stream, then segments (in brackets with the
+// words by funnel shifts), us: 2^20 words of 4096 streams 12.4, 6.3 (6.3); 2^24 uniforms of
+// 1024 559, 22.7 (20.6); 2^27 of 4096 1118, 148 (113), of 2e4 233, 173 (131), of 5e4 176,
+// 140 (107); 2^27 normals of 4096 1868, 208 (191).  (From 7e4 streams on a thread a stream
+// is faster: 115 against 123 us.)
 constexpr int kSplitThreads = 512, kSplitMax = 64, kSplitRow = 32;
 struct SplitArgs {
     Jump lo[8], hi[kSplitMax / 8];   // g L items ahead for g = 0 .. 7, and 8g L
