@@ -224,6 +224,26 @@ __global__ void lfg_extend_kernel(LfgArgs a, int64_t q_hi, int64_t count)
     a.ring[(uint32_t)(q + R)] = a.ring[(uint32_t)(q + a.D + a.sl + R)] - a.ring[(uint32_t)(q + a.sl + R)];
 }
 
+// The whole extension of a small row in one launch, by one cluster of blocks with its
+// barrier between the pieces of sl positions: a fan of depth 16 takes 15 of them (handle of
+// row 2 made in 81 us with a launch each, 41 so).  Other blocks' values
+// come from L2.
+constexpr int kExtBlocks = 8, kExtThreads = 1024;
+__global__ void __cluster_dims__(kExtBlocks, 1, 1) __launch_bounds__(kExtThreads)
+    lfg_extend_all_kernel(LfgArgs a, int64_t q_hi, int64_t q_end)
+{
+    const uint32_t R = a.R;
+    while (q_hi > q_end) {
+        const int64_t cnt = min((int64_t)a.sl, q_hi - q_end);
+        q_hi -= cnt;
+        for (int64_t i = blockIdx.x * kExtThreads + threadIdx.x; i < cnt; i += kExtBlocks * kExtThreads) {
+            const int64_t q = q_hi + i;
+            __stcg(a.ring + (uint32_t)(q + R), __ldcg(a.ring + (uint32_t)(q + a.D + a.sl + R)) - __ldcg(a.ring + (uint32_t)(q + a.sl + R)));
+        }
+        asm volatile("barrier.cluster.arrive.aligned;\nbarrier.cluster.wait.aligned;" ::: "memory");
+    }
+}
+
 // ------------------------------------------------------------- host side
 LfgArgs lfg_args(const Handle* h)
 {
@@ -246,11 +266,17 @@ int lfg_seed(Handle* h, cudaStream_t st)
     const LfgArgs a = lfg_args(h);
     lfg_seed_kernel<<<(unsigned)((h->ll + T - 1) / T), T, 0, st>>>(h->seed, h->ll, a);
     GB_CUDA(cudaGetLastError());
-    // x_{-H} .. x_{-ll-1}, in rounds of sl positions from -ll downwards
-    for (int64_t q_hi = -(int64_t)h->ll; q_hi > -lfg_history(h);) {
-        const int64_t cnt = std::min<int64_t>(h->sl, q_hi + lfg_history(h));
-        lfg_extend_kernel<<<(unsigned)((cnt + T - 1) / T), T, 0, st>>>(a, q_hi, cnt);
-        q_hi -= cnt;
+    // x_{-H} .. x_{-ll-1}, in pieces of sl positions from -ll downwards: in one launch where
+    // a piece is at most eight words a thread of the cluster, else in one each
+    const int64_t q_end = -lfg_history(h);
+    if (h->sl <= 8 * kExtBlocks * kExtThreads) {
+        lfg_extend_all_kernel<<<kExtBlocks, kExtThreads, 0, st>>>(a, -(int64_t)h->ll, q_end);
+    } else {
+        for (int64_t q_hi = -(int64_t)h->ll; q_hi > q_end;) {
+            const int64_t cnt = std::min<int64_t>(h->sl, q_hi - q_end);
+            lfg_extend_kernel<<<(unsigned)((cnt + T - 1) / T), T, 0, st>>>(a, q_hi, cnt);
+            q_hi -= cnt;
+        }
     }
     GB_CUDA(cudaGetLastError());
     return GBRNG_OK;
