@@ -343,9 +343,11 @@ __device__ __forceinline__ float2 splat2(float a) { return make_float2(a, a); }
 // e + 64 is a small unsigned number, and the funnel shift that extracts it also
 // sets the upper bits of 1.5 2^23: e then comes as a binary32 from one paired
 // addition instead of a conversion each, whose result a warp waits for.  Same bits.
-// Hybrid Taus, two oscillators a thread: 1e6 x 1000 steps 4.33 -> 4.09 ms; where the
-// other instructions are fewer the extra shift costs more (LCG +1%, overdamped +2%,
-// LCG normal fill +4%), and those convert.
+// Hybrid Taus, two oscillators a thread: 1e6 x 1000 steps 4.33 -> 4.09 ms, overdamped
+// 1e4 x 1000 102 -> 98 us; Ran2, whose draws are converted anyway, 2^27 normals 206 ->
+// 201 us, adjoint 1e5 x 1000 1159 -> 1146.  Where the other instructions are fewer the
+// extra shift costs more (LCG +1%, overdamped LCG +2% and Ran2 +3%, LCG normal fill +4%),
+// and those convert.
 template <bool SPLIT = false>
 __device__ __forceinline__ float2 neg2log2(float2 u)
 {
