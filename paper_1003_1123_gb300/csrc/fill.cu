@@ -125,8 +125,12 @@ constexpr int kRan2Threads = 128;
 // The table's 32 words are loaded, and stored, all at once: at 134 draws a stream of 1e6
 // streams the state is a third of the traffic, and four words at a time its latency shows
 // (2^27 uniforms 167 us, eight or sixteen at a time 160, all 150; 2^24 70 and 62).
+// Eight blocks a SM, 64 registers: with the compiler's 128 half as many warps are there to
+// hide a draw's chain (2^27 from 1e6 streams, 128 registers / six / eight / ten / twelve
+// blocks: uniforms 150 / 142 / 140 / 142 / 160 us, normals 201 / 191 / 193 / 191 / 197; 2^24
+// uniforms of 4096 streams 152 / 160 / 154 / 167 / 168).
 template <int MODE>
-__global__ void __launch_bounds__(kRan2Threads) ran2_fill_kernel(int32_t* __restrict__ st, int64_t S,
+__global__ void __launch_bounds__(kRan2Threads, 8) ran2_fill_kernel(int32_t* __restrict__ st, int64_t S,
                                                         int64_t n_items, void* __restrict__ out)
 {
     extern __shared__ int32_t tab[];      // [32][blockDim.x]
