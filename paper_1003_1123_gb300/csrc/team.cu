@@ -40,6 +40,9 @@
 namespace gb {
 
 constexpr int kStages = 4;
+// Named barriers: stage s filled, 1 + s; stage s consumed, 1 + kStages + s; every
+// producer warp has loaded the generators' states.
+constexpr int BAR_LOADED = 1 + 2 * kStages;
 
 // What a team runs: the 3-D oscillators of ld_run or the overdamped particles of
 // ou_run.
@@ -77,7 +80,7 @@ struct TeamShape {
     // a half-warp's stores of one normal go to 16 / PAIRS chunks: padding a
     // chunk so that they start on different banks
     static constexpr int kChunkWords = kChunk * kStepWords + kStateWords + kOsc;
-    static constexpr int kThreads = 32 * (kStages * M + 1);
+    static constexpr int kProducers = 32 * kStages * M, kThreads = kProducers + 32;
     static constexpr size_t kBufBytes = sizeof(float) * kChunks * kChunkWords;
 };
 
@@ -149,6 +152,9 @@ __device__ __forceinline__ void team_produce(const TeamArgs& a, float* buf, int 
         else
             lc[j].x = a.lcg[i];
     }
+    // every producer warp reads these words, and the one with the run's last chunk
+    // replaces them: no warp goes on, or leaves, before all have them
+    bar_sync(BAR_LOADED, S::kProducers);
     // to the chunk's first draw: 2^l chunks ahead for every bit l of its number
     auto jump = [&](auto d) {
 #pragma unroll
@@ -445,7 +451,7 @@ __global__ void __launch_bounds__(TeamShape<MODEL, PAIRS, M>::kThreads) team_ker
     using S = TeamShape<MODEL, PAIRS, M>;
     constexpr int kBarThreads = 32 * (M + 1);
     extern __shared__ __align__(16) float team_sm[];
-    if (threadIdx.x < 32 * kStages * M)
+    if (threadIdx.x < S::kProducers)
         team_produce<MODEL, KIND, S>(a, team_sm, kBarThreads);
     else if constexpr (MODEL == TEAM_OU)
         team_consume_ou<S>(a, team_sm, kBarThreads);

@@ -65,3 +65,17 @@ def test_overdamped_team_equals_short_runs(G, kind, n, steps, every):
     assert torch.equal(a.R, b.R)
     assert G.rng_get_state(a.rng) == G.rng_get_state(b.rng)
     assert np.allclose(mean, m, rtol=0, atol=1e-12) and np.allclose(corr, c, rtol=0, atol=1e-11)
+
+
+@pytest.mark.parametrize("kind", ["taus", "lcg"])
+@pytest.mark.parametrize("n,steps", [(1000, 34), (1000, 49), (1000, 127), (1001, 128), (4865, 51), (4865, 63), (4871, 64)])
+def test_team_runs_of_one_stage(G, kind, n, steps):
+    """Runs that end in the first of the four stages (128 steps with 8 oscillators a block,
+    64 with 16): the other stages' warps leave at once, after they have loaded."""
+    a, b = system(G, kind, n), system(G, kind, n)
+    sa, sb = G.ld_run(a, steps), G.ld_run_stepwise(b, steps)
+    assert torch.equal(a.x, b.x) and torch.equal(a.v, b.v)
+    assert G.rng_get_state(a.rng) == G.rng_get_state(b.rng)
+    # binary64 sums of the same binary32 values, and two compensated binary32 sums
+    assert abs(sa["sum_v2"] / sb["sum_v2"] - 1) < 1e-12
+    assert abs(sa["energy_time_avg"] / sb["energy_time_avg"] - 1) < 1e-6

@@ -1,0 +1,38 @@
+"""Orderings that the kernels need and that no run can be relied on to miss: read from the
+sources, as which of a block's warps comes first is the hardware's choice."""
+import os
+import re
+
+CSRC = os.path.join(os.path.dirname(os.path.abspath(__file__)), "..", "paper_1003_1123_gb300", "csrc")
+
+
+def source(name):
+    """A source file without its comments."""
+    text = open(os.path.join(CSRC, name)).read()
+    return re.sub(r"//[^\n]*", "", text)
+
+
+def body(text, name):
+    """The definition of a function, from its name to the brace that closes it."""
+    at = re.search(r"\b%s\([^;{]*\)\s*\{" % name, text)
+    assert at, name
+    depth, i = 1, at.end()
+    while depth:
+        depth += {"{": 1, "}": -1}.get(text[i], 0)
+        i += 1
+    return text[at.start():i]
+
+
+def test_team_states_are_loaded_before_any_is_stored():
+    """Every producer warp of a block loads all its oscillators' generator states; the warp of
+    the run's last chunk stores the end states to the same words.  A barrier of all producer
+    warps has to lie between, and before any of them may leave."""
+    f = body(source("team.cu"), "team_produce")
+    loads = [m.end() for m in re.finditer(r"=\s*(?:taus_load\()?a\.(?:taus|lcg)\[i\]", f)]
+    stores = [m.start() for m in re.finditer(r"a\.(?:taus|lcg)\[idx\[j\]\]\s*=", f)]
+    leaves = [m.start() for m in re.finditer(r"\breturn\b", f)]
+    barrier = [m.start() for m in re.finditer(r"bar_sync\(BAR_LOADED, S::kProducers\)", f)]
+    assert len(loads) == 2 and len(stores) == 2 and len(barrier) == 1 and leaves
+    assert max(loads) < barrier[0] < min(stores + leaves)
+    s = source("team.cu")
+    assert re.search(r"threadIdx\.x < S::kProducers\)\s*team_produce", s)   # all of them, and no other warp
