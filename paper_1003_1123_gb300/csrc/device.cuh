@@ -851,6 +851,7 @@ __device__ __forceinline__ void store_stats(const StatsSink& s, double v)
         __threadfence();
     }
     if (!__shfl_sync(0xffffffffu, last, 0)) return;
+    __syncwarp();   // the other lanes' reads behind lane 0's fence (a shuffle orders no memory)
     double t = 0;   // lane 4 j + k: sum k of blocks j, j + 8, ...
 #pragma unroll 4
     for (unsigned i = lane; i < 4 * gridDim.x; i += 32) t += __ldcg(s.partials + i);

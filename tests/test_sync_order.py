@@ -36,3 +36,12 @@ def test_team_states_are_loaded_before_any_is_stored():
     assert max(loads) < barrier[0] < min(stores + leaves)
     s = source("team.cu")
     assert re.search(r"threadIdx\.x < S::kProducers\)\s*team_produce", s)   # all of them, and no other warp
+
+
+def test_last_block_reads_partials_behind_the_fence():
+    """The last block's lane 0 counts the blocks and fences; the other lanes read what the
+    other blocks left only after a warp barrier, which orders memory (a shuffle does not)."""
+    f = body(source("device.cuh"), "store_stats")
+    count, read = f.index("atomicAdd(s.ticket"), f.index("__ldcg(s.partials")
+    fence = f.index("__threadfence()", count)
+    assert count < fence < f.index("__syncwarp()", fence) < read
