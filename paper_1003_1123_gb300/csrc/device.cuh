@@ -860,6 +860,24 @@ __device__ __forceinline__ void store_stats(const StatsSink& s, double v)
     if (lane == 0) *s.ticket = 0;
 }
 
+// Barriers that a warp takes as one (bar is barrier.aligned): behind a branch or a loop that
+// its lanes may have left apart, __syncwarp brings them together first.
+__device__ __forceinline__ void bar_sync(int id, int threads)
+{
+    __syncwarp();
+    asm volatile("bar.sync %0, %1;" ::"r"(id), "r"(threads) : "memory");
+}
+__device__ __forceinline__ void bar_arrive(int id, int threads)
+{
+    __syncwarp();
+    asm volatile("bar.arrive %0, %1;" ::"r"(id), "r"(threads) : "memory");
+}
+__device__ __forceinline__ void cluster_sync()
+{
+    __syncwarp();
+    asm volatile("barrier.cluster.arrive.aligned;\nbarrier.cluster.wait.aligned;" ::: "memory");
+}
+
 // Cheap global-timer read for bounded waits.
 __device__ __forceinline__ uint64_t global_ns()
 {

@@ -114,7 +114,7 @@ __global__ void __launch_bounds__(kSplitThreads) word_split_kernel(State* st, in
         if (g & 7) jump_ahead(y, a.lo[g & 7]);
         if (g >> 3) jump_ahead(y, a.hi[g >> 3]);
     }
-    asm volatile("barrier.cluster.arrive.aligned;\nbarrier.cluster.wait.aligned;" ::: "memory");
+    cluster_sync();
     if (!live) return;
     emit_chain<MODE>(y, first, S, end, out);
     if (first + ((end - first - 1) / S) * S + S >= n_items) st[s] = y;   // the stream's last item

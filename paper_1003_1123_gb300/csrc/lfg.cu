@@ -72,7 +72,6 @@ __global__ void __launch_bounds__(32 * (kFillWarps + 1), 1) lfg_fill_kernel(LfgA
             }
         }
         if (r + 1 < n_rounds) {
-            __syncwarp();
             bar_arrive(BAR_STORED, T);
         }
         if (MODE == LFG_NORMAL) {
@@ -240,7 +239,7 @@ __global__ void __cluster_dims__(kExtBlocks, 1, 1) __launch_bounds__(kExtThreads
             const int64_t q = q_hi + i;
             __stcg(a.ring + (uint32_t)(q + R), __ldcg(a.ring + (uint32_t)(q + a.D + a.sl + R)) - __ldcg(a.ring + (uint32_t)(q + a.sl + R)));
         }
-        asm volatile("barrier.cluster.arrive.aligned;\nbarrier.cluster.wait.aligned;" ::: "memory");
+        cluster_sync();
     }
 }
 

@@ -117,15 +117,6 @@ __device__ inline bool barrier_thread(const LfgArgs& a, uint64_t target, bool ar
     return true;
 }
 
-__device__ __forceinline__ void bar_sync(int id, int threads)
-{
-    asm volatile("bar.sync %0, %1;" ::"r"(id), "r"(threads) : "memory");
-}
-__device__ __forceinline__ void bar_arrive(int id, int threads)
-{
-    asm volatile("bar.arrive %0, %1;" ::"r"(id), "r"(threads) : "memory");
-}
-
 // The warps of a CTA.  Generating warps arrive at BAR_STORED when the CTA's share
 // of round r is stored; the waiting warp meets them there, takes the CTA through
 // the grid barrier and meets every warp at BAR_GO: the using warps, which then use
@@ -274,7 +265,6 @@ __device__ __forceinline__ void gen_warps(const LfgArgs& a, int warp, int64_t n_
             fan_load<K>(a, slot_add(s_round, (uint32_t)(g * FO), a.R), g * FO, f);
             fan_store<K>(a, n_off, n, f, [](int, int, uint32_t) {});
         }
-        __syncwarp();
         bar_arrive(BAR_STORED, 32 * (GW + 1));
         s_round = slot_add(s_round, (uint32_t)n, a.R);
         bar_sync(BAR_GO, threads);

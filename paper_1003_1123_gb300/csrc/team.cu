@@ -103,15 +103,6 @@ __device__ __forceinline__ float2 draw_cos2(TausDraw (&td)[2], LcgDraw (&lc)[2])
     return box_muller_cos2(neg2log2(u), x);
 }
 
-__device__ __forceinline__ void bar_sync(int id, int threads)
-{
-    asm volatile("bar.sync %0, %1;" ::"r"(id), "r"(threads) : "memory");
-}
-__device__ __forceinline__ void bar_arrive(int id, int threads)
-{
-    asm volatile("bar.arrive %0, %1;" ::"r"(id), "r"(threads) : "memory");
-}
-
 // em_component with cs g formed beforehand: of one oscillator, or of two in the
 // lanes of the paired instructions.
 __device__ __forceinline__ void team_update(float cdt, float cva, float nck, float csg, float& x, float& v)
@@ -233,7 +224,6 @@ __device__ __forceinline__ void team_produce(const TeamArgs& a, float* buf, int 
                         a.lcg[idx[j]] = lc[j].x;
                 }
         }
-        __syncwarp();
         bar_arrive(1 + stage, bar_threads);
         // to the same chunk of the next pass
         if (t + S::kPassSteps < a.n_steps) jump(std::integral_constant<uint64_t, D*(S::kChunks - 1)>{});
@@ -243,7 +233,6 @@ __device__ __forceinline__ void team_produce(const TeamArgs& a, float* buf, int 
         if (!energies) return;
         bar_sync(1 + kStages + stage, bar_threads);
         chunk_energy(t0 - S::kPassSteps + (int64_t)chunk * S::kChunk);
-        __syncwarp();
         bar_arrive(1 + stage, bar_threads);
     }
 }
@@ -283,7 +272,6 @@ __device__ __forceinline__ void team_consume(const TeamArgs& a, float* buf, int 
         }
         // hand the stage back if it is looked at or filled again
         if (ENERGIES || t0 + S::kPassSteps < a.n_steps) {
-            __syncwarp();
             bar_arrive(1 + kStages + stage, bar_threads);
         }
         t0 += n_stage;

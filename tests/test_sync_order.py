@@ -45,3 +45,18 @@ def test_last_block_reads_partials_behind_the_fence():
     count, read = f.index("atomicAdd(s.ticket"), f.index("__ldcg(s.partials")
     fence = f.index("__threadfence()", count)
     assert count < fence < f.index("__syncwarp()", fence) < read
+
+
+def test_aligned_barriers_are_taken_by_whole_warps():
+    """The aligned barriers want the warp converged: each stands in a helper that brings it
+    together first, and nowhere else."""
+    helpers = ("bar_sync", "bar_arrive", "cluster_sync")
+    device = source("device.cuh")
+    for name in helpers:
+        f = body(device, name)
+        assert "__syncwarp()" in f and f.index("__syncwarp()") < f.index("asm volatile"), name
+        device = device.replace(f, "")
+    texts = {n: source(n) for n in sorted(os.listdir(CSRC)) if n.endswith((".cu", ".cuh"))}
+    texts["device.cuh"] = device
+    for n, text in texts.items():
+        assert not re.search(r'"[^"]*\bbar(?:rier)?\.', text), n
