@@ -27,12 +27,12 @@ template <int MODE, int K>
 __global__ void __launch_bounds__(32 * (kFillWarps + 1), 1) lfg_fill_kernel(LfgArgs a)
 {
     extern __shared__ __align__(16) uint32_t fill_sm[];   // [K][units of the CTA][offsets of a unit]
-    __shared__ int s_failed;
+    __shared__ int64_t s_failed;
     __shared__ uint32_t over[K];
     constexpr int J = fan_j<K>(), FO = 32 * J, T = 32 * (kFillWarps + 1), WORK = 32 * kFillWarps;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int64_t n_rounds = (a.n_pos + a.w - 1) / a.w;
-    if (threadIdx.x == 0) s_failed = 0;
+    if (threadIdx.x == 0) s_failed = kNoRound;
     __syncthreads();
     if (warp == kFillWarps) {
         wait_warp(a, n_rounds - 1, T, T, &s_failed);
@@ -121,7 +121,7 @@ __global__ void __launch_bounds__(32 * (kFillWarps + 1), 1) lfg_fill_kernel(LfgA
         sU = slot_add(sU, (uint32_t)n, a.R);
         if (r + 1 < n_rounds) {
             bar_sync(BAR_GO, T);
-            if (*(volatile int*)&s_failed) return;
+            if (round_failed(&s_failed, r)) return;
         }
     }
 }

@@ -123,11 +123,21 @@ __device__ inline bool barrier_thread(const LfgArgs& a, uint64_t target, bool ar
 // round r, and the generating ones, which then generate round r + 1.  A using warp
 // comes to BAR_GO with round r - 1 used, so the arrival that follows says that the
 // CTA is done with it: R >= 3 W keeps it until then.
+//
+// A wait that ran out is told by its round (kNoRound: none did).  Past BAR_GO of
+// round r the waiting warp needs only the generating warps to be in round r + 1, and
+// to fail there; a using warp that looks late must not leave for that before BAR_GO of
+// round r + 1, which counts on it.  So warps leave by round_failed(r), the same for all.
+constexpr int64_t kNoRound = INT64_MAX;
+__device__ __forceinline__ bool round_failed(const int64_t* failed, int64_t r)
+{
+    return *(volatile const int64_t*)failed <= r;
+}
 enum { BAR_STORED = 1, BAR_GO = 2 };
 
 // The waiting warp: one barrier for each of `count` rounds, `stored` threads at
 // BAR_STORED and `threads` at BAR_GO.
-__device__ __forceinline__ void wait_warp(const LfgArgs& a, int64_t count, int stored, int threads, int* failed)
+__device__ __forceinline__ void wait_warp(const LfgArgs& a, int64_t count, int stored, int threads, int64_t* failed)
 {
     const bool arrive_here = (int)blockIdx.x != a.stall_cta;
     for (int64_t r = 0; r < count; ++r) {
@@ -135,7 +145,7 @@ __device__ __forceinline__ void wait_warp(const LfgArgs& a, int64_t count, int s
         int ok = 1;
         if ((threadIdx.x & 31) == 0) {
             ok = barrier_thread(a, (uint64_t)gridDim.x * (uint64_t)(r + 1), arrive_here);
-            if (!ok) *(volatile int*)failed = 1;
+            if (!ok) *(volatile int64_t*)failed = r;
         }
         ok = __shfl_sync(0xffffffffu, ok, 0);
         bar_sync(BAR_GO, threads);
@@ -245,7 +255,7 @@ __device__ __forceinline__ void fan_store(const LfgArgs& a, int n_off, int n, Fa
 // contiguous share, a warp every GW-th unit of it.
 template <int K, int GW>
 __device__ __forceinline__ void gen_warps(const LfgArgs& a, int warp, int64_t n_rounds, int threads,
-                                          const int* failed)
+                                          const int64_t* failed)
 {
     constexpr int FO = fan_offsets<K>();
     uint32_t s_round = a.base_slot;
@@ -268,7 +278,7 @@ __device__ __forceinline__ void gen_warps(const LfgArgs& a, int warp, int64_t n_
         bar_arrive(BAR_STORED, 32 * (GW + 1));
         s_round = slot_add(s_round, (uint32_t)n, a.R);
         bar_sync(BAR_GO, threads);
-        if (*(volatile const int*)failed) return;
+        if (round_failed(failed, r)) return;
     }
 }
 

@@ -28,7 +28,7 @@ template <int K, int NW, int GW, bool STEPS>
 __global__ void __launch_bounds__(32 * (NW + GW + 1), 1) lfg_ou_kernel(OuLfgArgs o)
 {
     extern __shared__ __align__(16) float ou_sm[];   // [2][n_pad]
-    __shared__ int s_failed;
+    __shared__ int64_t s_failed;
     constexpr int T = 32 * (NW + GW + 1), UP = STEPS ? 32 : 64, ST = STEPS ? 2 : 1;
     const LfgArgs& a = o.l;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -37,7 +37,7 @@ __global__ void __launch_bounds__(32 * (NW + GW + 1), 1) lfg_ou_kernel(OuLfgArgs
     const int n_pad = (o.n_c + 63) & ~63, n_units = (nc + UP - 1) / UP;
     const int S = a.w / (int)(2 * a.N);   // steps a round
     const int64_t n_rounds = (a.n_pos + a.w - 1) / a.w;
-    if (threadIdx.x == 0) s_failed = 0;
+    if (threadIdx.x == 0) s_failed = kNoRound;
     for (int i = threadIdx.x; i < nc; i += T) ou_sm[i] = ou_sm[n_pad + i] = o.R[j0 + i];
     __syncthreads();
     if (warp >= NW + GW) {
@@ -76,7 +76,7 @@ __global__ void __launch_bounds__(32 * (NW + GW + 1), 1) lfg_ou_kernel(OuLfgArgs
             // first record of the phase: its number, and the steps of the phase taken by then
             const int64_t rec0 = p * S / o.every + 1, at0 = rec0 * o.every - p * S;
             bar_sync(BAR_GO, T);
-            if (*(volatile int*)&s_failed) break;
+            if (round_failed(&s_failed, p)) break;
             uint32_t su = s_first;
             uint4 w;   // raw words are loaded one item ahead
             if (warp < n_units) w = fetch(su);
@@ -113,7 +113,7 @@ __global__ void __launch_bounds__(32 * (NW + GW + 1), 1) lfg_ou_kernel(OuLfgArgs
         }
     }
     __syncthreads();
-    if (s_failed) return;
+    if (s_failed != kNoRound) return;
     for (int i = threadIdx.x; i < nc; i += T) o.R[j0 + i] = ou_sm[i];
 }
 

@@ -48,7 +48,7 @@ template <int K, int CW, int GW>
 __global__ void __launch_bounds__(32 * (CW + GW + 1), 1) lfg_resident_kernel(LfgArgs a, int n_c)
 {
     extern __shared__ __align__(16) float res_sm[];   // [unit][kUnitWords]
-    __shared__ int s_failed;
+    __shared__ int64_t s_failed;
     __shared__ double red[4 * 32];
     constexpr int T = 32 * (CW + GW + 1);
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -56,7 +56,7 @@ __global__ void __launch_bounds__(32 * (CW + GW + 1), 1) lfg_resident_kernel(Lfg
     const int nc = (int)max((int64_t)0, min(a.N - j0, (int64_t)n_c));
     const int n_units = (nc + 63) >> 6;
     const int64_t n_rounds = (a.n_pos + a.w - 1) / a.w;
-    if (threadIdx.x == 0) s_failed = 0;
+    if (threadIdx.x == 0) s_failed = kNoRound;
     // word q of oscillator j of the CTA (q: x, then v)
     auto at = [](int j, int q) { return (j >> 6) * kUnitWords + 64 * q + (j & 63); };
     for (int i = threadIdx.x; i < 3 * nc; i += T) {
@@ -80,7 +80,7 @@ __global__ void __launch_bounds__(32 * (CW + GW + 1), 1) lfg_resident_kernel(Lfg
             const int steps = (int)min((int64_t)S, left);
             left -= steps;
             bar_sync(BAR_GO, T);
-            if (*(volatile int*)&s_failed) break;
+            if (round_failed(&s_failed, p)) break;
             // raw words are loaded one item (a unit's step) ahead
             uint4 w0, w1;
             uint32_t su = s_first;
@@ -127,7 +127,7 @@ __global__ void __launch_bounds__(32 * (CW + GW + 1), 1) lfg_resident_kernel(Lfg
         }
     }
     __syncthreads();
-    if (s_failed) return;
+    if (s_failed != kNoRound) return;
     double acc[4] = {0, 0, 0, 0};
     for (int i = threadIdx.x; i < 3 * nc; i += T) {
         const int j = i / 3, q = i - 3 * j;
@@ -153,12 +153,12 @@ __global__ void __launch_bounds__(32 * (CW + GW + 1), 1) lfg_resident_kernel(Lfg
 template <int MODE, int K, int CW, int GW>
 __global__ void __launch_bounds__(32 * (CW + GW + 1), 1) lfg_stream_kernel(LfgArgs a)
 {
-    __shared__ int s_failed;
+    __shared__ int64_t s_failed;
     __shared__ double red[4 * 32];
     constexpr int T = 32 * (CW + GW + 1);
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int64_t n_rounds = (a.n_pos + a.w - 1) / a.w;
-    if (threadIdx.x == 0) s_failed = 0;
+    if (threadIdx.x == 0) s_failed = kNoRound;
     __syncthreads();
     Kahan2 e;
     double acc[4] = {0, 0, 0, 0};
@@ -203,7 +203,7 @@ __global__ void __launch_bounds__(32 * (CW + GW + 1), 1) lfg_stream_kernel(LfgAr
                 }
             };
             bar_sync(BAR_GO, T);
-            if (*(volatile int*)&s_failed) break;
+            if (round_failed(&s_failed, p)) break;
             uint4 w0, w1;
             float2 X[3], V[3];
             if (u0 < u1) {
@@ -279,7 +279,7 @@ __global__ void __launch_bounds__(32 * (CW + GW + 1), 1) lfg_stream_kernel(LfgAr
     }
     if (MODE == LFG_LD && a.sink.partials) {
         __syncthreads();
-        if (s_failed) return;
+        if (s_failed != kNoRound) return;
         acc[3] = e.value();
         const double sums = block_sums(acc, red);
         if (warp == 0) store_stats(a.sink, sums);

@@ -55,7 +55,7 @@ template <int MODEL, int K>
 __global__ void __launch_bounds__(kTeamThreads, 1) lfg_team_kernel(LfgTeamArgs o)
 {
     extern __shared__ __align__(16) float team_sm[];   // [steps][normal][n_c]
-    __shared__ int s_failed;
+    __shared__ int64_t s_failed;
     __shared__ double red[4 * kTeamUse];
     constexpr int Q = MODEL == LFG_TEAM_LD ? 3 : 1, WORDS = MODEL == LFG_TEAM_LD ? 4 : 2;   // a step's normals, draws
     constexpr int USE = 32 * kTeamUse, T = kTeamThreads;
@@ -64,7 +64,7 @@ __global__ void __launch_bounds__(kTeamThreads, 1) lfg_team_kernel(LfgTeamArgs o
     const int64_t j0 = (int64_t)blockIdx.x * n2;
     const int nc = (int)max((int64_t)0, min(a.N - j0, (int64_t)n2));
     const int64_t n_rounds = (a.n_pos + a.w - 1) / a.w;
-    if (threadIdx.x == 0) s_failed = 0;
+    if (threadIdx.x == 0) s_failed = kNoRound;
     __syncthreads();
     if (warp >= kTeamUse + kTeamGen) {
         wait_warp(a, n_rounds, 32 * (kTeamGen + 1), T, &s_failed);
@@ -110,7 +110,7 @@ __global__ void __launch_bounds__(kTeamThreads, 1) lfg_team_kernel(LfgTeamArgs o
     for (int64_t p = 0; p < n_rounds; ++p) {
         const int steps = (int)min((int64_t)S, a.n_steps - p * S);
         bar_sync(BAR_GO, T);
-        if (*(volatile int*)&s_failed) return;
+        if (round_failed(&s_failed, p)) return;
         if (nc > 0) {
             auto fetch = [&](int i, int s, uint4& w0, uint4& w1) {
                 const uint32_t sl = slot_add(slot_add(s_cta, (uint32_t)s * step_slots, a.R), (uint32_t)(2 * WORDS * i), a.R);

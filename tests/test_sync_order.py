@@ -60,3 +60,19 @@ def test_aligned_barriers_are_taken_by_whole_warps():
     texts["device.cuh"] = device
     for n, text in texts.items():
         assert not re.search(r'"[^"]*\bbar(?:rier)?\.', text), n
+
+
+def test_warps_leave_a_failed_launch_by_its_round():
+    """A wait that ran out in round r + 1 can be recorded before a using warp has looked past
+    round r's barrier; it may leave only for round r's failure, as round r + 1's barrier
+    counts on it.  So no flag: the round, and every warp inside the rounds asks for its own."""
+    head = source("lfg.cuh")
+    assert "<= r" in body(head, "round_failed")
+    assert re.search(r"failed\s*=\s*r;", body(head, "wait_warp"))
+    for name, kernels in (("lfg.cu", 1), ("lfg_run.cu", 2), ("lfg_ou.cu", 1), ("lfg_team.cu", 1)):
+        text = source(name)
+        assert text.count("__shared__ int64_t s_failed;") == kernels == text.count("s_failed = kNoRound;")
+        assert not re.search(r"if \((?:\*\(volatile[^)]*\)&)?s_failed\)", text)      # as a flag
+        # past each BAR_GO, the round of the loop that it closes
+        for at in (m.end() for m in re.finditer(r"bar_sync\(BAR_GO, T\);", text)):
+            assert re.match(r"\s*if \(round_failed\(&s_failed, [rp]\)\) (?:break|return);", text[at:]), name
