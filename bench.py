@@ -1017,6 +1017,20 @@ def run_sweep():
                          "portable_state_bytes": G.rng_state_bytes(r),
                          "ms_per_1000": timed(lambda: G.ld_run(s, steps, stats=False))})
         del s, x, r
+    # Lagged Fibonacci systems beyond the SMs' shared memory, even and odd N (their x and v
+    # rows change alignment from step to step), one spring constant and one each
+    stream_rows = []
+    for n in (1200000, 1200001, 10**7, 10**7 + 1):
+        for per_k in (False, True):
+            r = G.rng_init("lagfib", SEED, n)
+            x = torch.zeros((n, 3), dtype=torch.float32, device="cuda")
+            K = torch.linspace(0.5, 2.0, n, device="cuda") if per_k else None
+            s = G.LdSystem(r, x, torch.zeros_like(x), K_per=K, **PARAMS)
+            G.ld_init_equilibrium(s)
+            stream_rows.append({"n": n, "K_per": per_k,
+                                "ms_per_1000": timed(lambda: G.ld_run(s, steps, stats=False))})
+            del s, x, r, K
+    torch.cuda.empty_cache()
     # the overdamped 1-D test of Sec. IV (Eq. 4-5) at the paper's parameters
     # (k_sp = 0.01 pN/nm, T = 300 K, D = 0.25 nm^2/ns, dt = 1 ps, R0 = 10 nm):
     # 1000 steps with a record every 100, at the paper's N = 1e4 and at 1e6
@@ -1033,8 +1047,9 @@ def run_sweep():
                        "particle_steps_per_s": n * steps / (ms * 1e-3)})
             del o, R, r
     return {"sweep": "time per 1000 steps vs N (E2), state bytes (E3), RNG share (E4), "
-                     "Table I rows at N = 1000, overdamped runs (Sec. IV)",
-            "params": PARAMS, "rows": rows, "lag_rows": lag_rows, "ou_params": ou_params,
+                     "Table I rows at N = 1000, streamed Lagged Fibonacci runs, overdamped runs (Sec. IV)",
+            "params": PARAMS, "rows": rows, "lag_rows": lag_rows,
+            "stream_rows": stream_rows, "ou_params": ou_params,
             "ou": ou, "clocks": clocks.stop()}
 
 

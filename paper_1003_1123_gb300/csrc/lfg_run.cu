@@ -145,14 +145,46 @@ __global__ void __launch_bounds__(32 * (CW + GW + 1), 1) lfg_resident_kernel(Lfg
     }
 }
 
-// The runs whose data streams through global memory: Langevin steps of systems
-// beyond the resident kernel and the equilibrium start.  A round is shared out in
-// units of 64 quads of words (oscillator-steps, two a lane); a Langevin round holds at most half a step (W <= 2 N), so that an
-// oscillator's next step comes two phases later at the earliest, after the
-// barrier that its last update's stores precede.
+// The runs whose data streams through global memory: Langevin steps of systems beyond the
+// resident kernel and the equilibrium start.  A round is shared out in units of 64 quads
+// of words (oscillator-steps, two a lane); a Langevin round holds at most half a step (W <=
+// 2 N), so that an oscillator's next step comes two phases later at the earliest, after
+// the barrier that its last update's stores precede.
+//
+// A unit's x, v and K pass through shared memory, copied in (cp.async) while the warp works
+// on the unit before, and out again, side by side over the warp: 16, 8 or 4 bytes a lane as
+// the unit's first words are aligned, which for an odd N changes from step to step.  A lane's
+// six words taken straight from x and v are strided, three accesses from an 8-byte boundary
+// and up to six elsewhere, and K was waited for at its use: us a step before / so, even N,
+// odd N, odd N with K_per: 2e6 26.1 / 22.7, 43.5 / 23.7, 46.2 / 26.7; 1e7 139 / 129, 231 /
+// 138, 230 / 146.  (4 bytes a lane always 151 at 1e7, at most 8 139; three stages instead
+// of two 1 to 2% slower.)
+constexpr int kStreamStages = 2, kStageWords = 7 * 64;   // of a warp: x, v [64][3], K [64]
+template <int CW>
+constexpr size_t stream_smem() { return sizeof(float) * kStageWords * kStreamStages * CW; }
+
+template <int BYTES>
+using Width = std::integral_constant<int, BYTES>;
+template <int BYTES>
+using Words = typename std::conditional<BYTES == 4, float, typename std::conditional<BYTES == 8, float2, float4>::type>::type;
+
+template <int BYTES>
+__device__ __forceinline__ void copy_words(float* to, const float* from, Width<BYTES>)
+{
+    asm volatile("cp.async.ca.shared.global [%0], [%1], %2;" ::"r"((uint32_t)__cvta_generic_to_shared(to)), "l"(from),
+                 "n"(BYTES)
+                 : "memory");
+}
+template <int BYTES>
+__device__ __forceinline__ void store_words(float* to, const float* from, Width<BYTES>)
+{
+    *reinterpret_cast<Words<BYTES>*>(to) = *reinterpret_cast<const Words<BYTES>*>(from);
+}
+
 template <int MODE, int K, int CW, int GW>
 __global__ void __launch_bounds__(32 * (CW + GW + 1), 1) lfg_stream_kernel(LfgArgs a)
 {
+    extern __shared__ __align__(16) float str_sm[];   // LD: [using warp][stage][kStageWords]
     __shared__ int64_t s_failed;
     __shared__ double red[4 * 32];
     constexpr int T = 32 * (CW + GW + 1);
@@ -168,12 +200,9 @@ __global__ void __launch_bounds__(32 * (CW + GW + 1), 1) lfg_stream_kernel(LfgAr
         gen_warps<K, GW>(a, warp - CW, n_rounds, T, &s_failed);
     } else {
         uint32_t s_round = a.base_slot;
-        // a lane's two oscillators as 8-byte words: x and v so aligned, and every pair
-        // an even oscillator and the next (N and a round's oscillators even)
-        const bool vec2 = a.N % 2 == 0 && a.w % 8 == 0 &&
-                          (((uintptr_t)a.x | (uintptr_t)a.v) & 7) == 0;
         int64_t j_round = 0, t_round = 0;   // oscillator and step of the round's first quad
         int n = 0, quads = 0, u0 = 0, u1 = 0;
+        float* const stages = str_sm + warp * kStreamStages * kStageWords;
         for (int64_t p = 0; p < n_rounds; ++p) {
             const int64_t U = p * a.w;   // launch offset of the round
             if (p == 0 || p == n_rounds - 1) {
@@ -186,92 +215,102 @@ __global__ void __launch_bounds__(32 * (CW + GW + 1), 1) lfg_stream_kernel(LfgAr
             // the quads from `wrap` on belong to the next step
             const int wrap = (int)min(a.N - j_round, (int64_t)INT_MAX);
             auto index = [&](int qd) { return j_round + qd - (qd >= wrap ? a.N : 0); };
-            auto fetch_xv = [&](int uu, float2 (&x)[3], float2 (&v)[3]) {
-                const int qd = min(64 * uu + 2 * lane, quads - 1), qe = min(qd + 1, quads - 1);
-                const float* x0 = a.x + 3 * index(qd);
-                const float* v0 = a.v + 3 * index(qd);
-                if (vec2 && qd < qe) {
-                    const float2* x2 = reinterpret_cast<const float2*>(x0);
-                    const float2* v2 = reinterpret_cast<const float2*>(v0);
+            // f(k, i, width): this lane passes `width` bytes of unit uu's words from the k-th of
+            // 64 x 3 on, which is word i of x and of v
+            auto words = [&](int uu, auto&& f) {
+                const int q0 = 64 * uu;
+                if (q0 + 64 <= quads && (q0 >= wrap || q0 + 64 <= wrap)) {
+                    const int64_t i = 3 * index(q0);
+                    const uint32_t low = (uint32_t)(uintptr_t)(a.x + i) | (uint32_t)(uintptr_t)(a.v + i);
+                    if (low % 16 == 0) {
+                        f(4 * lane, i + 4 * lane, Width<16>{});
+                        if (lane < 16) f(128 + 4 * lane, i + 128 + 4 * lane, Width<16>{});
+                    } else if (low % 8 == 0) {
 #pragma unroll
-                    for (int q = 0; q < 3; ++q) x[q] = x2[q], v[q] = v2[q];   // (x0, y0), (z0, x1), (y1, z1)
+                        for (int c = 0; c < 3; ++c) f(64 * c + 2 * lane, i + 64 * c + 2 * lane, Width<8>{});
+                    } else {
+#pragma unroll
+                        for (int c = 0; c < 6; ++c) f(32 * c + lane, i + 32 * c + lane, Width<4>{});
+                    }
                 } else {
-                    const float* x1 = a.x + 3 * index(qe);
-                    const float* v1 = a.v + 3 * index(qe);
-                    x[0] = make_float2(x0[0], x0[1]), x[1] = make_float2(x0[2], x1[0]), x[2] = make_float2(x1[1], x1[2]);
-                    v[0] = make_float2(v0[0], v0[1]), v[1] = make_float2(v0[2], v1[0]), v[2] = make_float2(v1[1], v1[2]);
+#pragma unroll 1
+                    for (int k = lane; k < 192; k += 32)
+                        if (q0 + k / 3 < quads) f(k, 3 * index(q0 + k / 3) + k % 3, Width<4>{});
                 }
+            };
+            auto copy_in = [&](int uu, float* st) {
+                if (uu < u1) {
+                    words(uu, [&](int k, int64_t i, auto w) {
+                        copy_words(st + k, a.x + i, w);
+                        copy_words(st + 192 + k, a.v + i, w);
+                    });
+                    if (a.Kper)
+#pragma unroll
+                        for (int k = lane; k < 64; k += 32)
+                            if (64 * uu + k < quads) copy_words(st + 384 + k, a.Kper + index(64 * uu + k), Width<4>{});
+                }
+                asm volatile("cp.async.commit_group;" ::: "memory");
             };
             bar_sync(BAR_GO, T);
             if (round_failed(&s_failed, p)) break;
             uint4 w0, w1;
-            float2 X[3], V[3];
-            if (u0 < u1) {
-                ring_octet(a, slot_add(s_round, (uint32_t)(256 * u0), a.R), w0, w1);
-                if (MODE == LFG_LD) fetch_xv(u0, X, V);
-            }
+            if (u0 < u1) ring_octet(a, slot_add(s_round, (uint32_t)(256 * u0), a.R), w0, w1);
+            int stage = 0;
+            if (MODE == LFG_LD) copy_in(u0, stages);
 #pragma unroll 1
             for (int u = u0; u < u1; u += CW) {
                 const int qd = 64 * u + 2 * lane;   // first quad of this lane
                 const bool live0 = qd < quads, live1 = qd + 1 < quads;
                 uint4 n0, n1;
-                float2 nx[3], nv[3];
-                if (u + CW < u1) {
-                    ring_octet(a, slot_add(s_round, (uint32_t)(256 * (u + CW)), a.R), n0, n1);
-                    if (MODE == LFG_LD) fetch_xv(u + CW, nx, nv);
-                }
-                {
+                if (u + CW < u1) ring_octet(a, slot_add(s_round, (uint32_t)(256 * (u + CW)), a.R), n0, n1);
+                if (MODE == LFG_LD) {
+                    float* const st = stages + stage * kStageWords;
+                    stage ^= 1;
+                    __syncwarp();   // the warp has left the unit before's stage
+                    copy_in(u + CW, stages + stage * kStageWords);
+                    asm volatile("cp.async.wait_group 1;" ::: "memory");
+                    __syncwarp();
+                    float2* const xs = reinterpret_cast<float2*>(st) + 3 * lane;
+                    float2* const vs = xs + 96;
+                    const float2 k = a.Kper ? reinterpret_cast<const float2*>(st + 384)[lane] : splat2(a.c.K);
+                    const float2 x0 = xs[0], x1 = xs[1], x2 = xs[2], v0 = vs[0], v1 = vs[1], v2 = vs[2];
+                    float2 x[3] = {make_float2(x0.x, x1.y), make_float2(x0.y, x2.x), make_float2(x1.x, x2.y)};
+                    float2 v[3] = {make_float2(v0.x, v1.y), make_float2(v0.y, v2.x), make_float2(v1.x, v2.y)};
+                    float2 en = pair_step(a.c, make_float2(-__fmul_rn(a.c.ckm, k.x), -__fmul_rn(a.c.ckm, k.y)),
+                                          make_float2(0.5f * k.x, 0.5f * k.y), w0, w1, x, v);
+                    if (!live0) en.x = 0.f;
+                    if (!live1) en.y = 0.f;
+                    e.add(en);
+                    const bool la = t_round + (qd >= wrap) == a.n_steps - 1;
+                    const bool lb = t_round + (qd + 1 >= wrap) == a.n_steps - 1;
+                    if (la || lb) final_sums(x, v, live0 && la, live1 && lb, acc);
+                    xs[0] = make_float2(x[0].x, x[1].x), xs[1] = make_float2(x[2].x, x[0].y), xs[2] = make_float2(x[1].y, x[2].y);
+                    vs[0] = make_float2(v[0].x, v[1].x), vs[1] = make_float2(v[2].x, v[0].y), vs[2] = make_float2(v[1].y, v[2].y);
+                    __syncwarp();
+                    words(u, [&](int k, int64_t i, auto w) {
+                        store_words(a.x + i, st + k, w);
+                        store_words(a.v + i, st + 192 + k, w);
+                    });
+                } else {
+                    // draw-step 0 -> x = sqrt(kT/K_i) g, draw-step 1 -> v = sqrt(kT/m) g
                     const int64_t ja = index(live0 ? qd : 0), jb = index(live1 ? qd + 1 : 0);
                     const float k0 = a.Kper ? __ldg(a.Kper + ja) : a.c.K, k1 = a.Kper ? __ldg(a.Kper + jb) : a.c.K;
-                    if (MODE == LFG_LD) {
-                        float2 x[3] = {make_float2(X[0].x, X[1].y), make_float2(X[0].y, X[2].x),
-                                       make_float2(X[1].x, X[2].y)};
-                        float2 v[3] = {make_float2(V[0].x, V[1].y), make_float2(V[0].y, V[2].x),
-                                       make_float2(V[1].x, V[2].y)};
-                        float2 en = pair_step(a.c, make_float2(-__fmul_rn(a.c.ckm, k0), -__fmul_rn(a.c.ckm, k1)),
-                                              make_float2(0.5f * k0, 0.5f * k1), w0, w1, x, v);
-                        if (!live0) en.x = 0.f;
-                        if (!live1) en.y = 0.f;
-                        e.add(en);
-                        const bool la = t_round + (qd >= wrap) == a.n_steps - 1;
-                        const bool lb = t_round + (qd + 1 >= wrap) == a.n_steps - 1;
-                        if (la || lb) final_sums(x, v, live0 && la, live1 && lb, acc);
-                        float* xa = a.x + 3 * ja;
-                        float* va = a.v + 3 * ja;
-                        if (vec2 && live1) {
-                            float2* x2 = reinterpret_cast<float2*>(xa);
-                            float2* v2 = reinterpret_cast<float2*>(va);
-                            x2[0] = make_float2(x[0].x, x[1].x), x2[1] = make_float2(x[2].x, x[0].y);
-                            x2[2] = make_float2(x[1].y, x[2].y);
-                            v2[0] = make_float2(v[0].x, v[1].x), v2[1] = make_float2(v[2].x, v[0].y);
-                            v2[2] = make_float2(v[1].y, v[2].y);
-                        } else {
+                    float g[2][3];
+                    box_muller3_u32(w0.x, w0.y, w0.z, w0.w, g[0][0], g[0][1], g[0][2]);
+                    box_muller3_u32(w1.x, w1.y, w1.z, w1.w, g[1][0], g[1][1], g[1][2]);
 #pragma unroll
-                            for (int q = 0; q < 3; ++q) {
-                                if (live0) xa[q] = x[q].x, va[q] = v[q].x;
-                                if (live1) a.x[3 * jb + q] = x[q].y, a.v[3 * jb + q] = v[q].y;
-                            }
-                        }
-                    } else {
-                        // draw-step 0 -> x = sqrt(kT/K_i) g, draw-step 1 -> v = sqrt(kT/m) g
-                        float g[2][3];
-                        box_muller3_u32(w0.x, w0.y, w0.z, w0.w, g[0][0], g[0][1], g[0][2]);
-                        box_muller3_u32(w1.x, w1.y, w1.z, w1.w, g[1][0], g[1][1], g[1][2]);
+                    for (int h = 0; h < 2; ++h) {
+                        if (!(h ? live1 : live0)) continue;
+                        const int64_t j = h ? jb : ja;
+                        const bool pos = t_round + (qd + h >= wrap) == 0;
+                        const float f = pos ? __fsqrt_rn(__fdiv_rn(a.c.kT, h ? k1 : k0)) : a.c.sv;
 #pragma unroll
-                        for (int h = 0; h < 2; ++h) {
-                            if (!(h ? live1 : live0)) continue;
-                            const int64_t j = h ? jb : ja;
-                            const bool pos = t_round + (qd + h >= wrap) == 0;
-                            const float f = pos ? __fsqrt_rn(__fdiv_rn(a.c.kT, h ? k1 : k0)) : a.c.sv;
-#pragma unroll
-                            for (int q = 0; q < 3; ++q) (pos ? a.x : a.v)[3 * j + q] = __fmul_rn(f, g[h][q]);
-                        }
+                        for (int q = 0; q < 3; ++q) (pos ? a.x : a.v)[3 * j + q] = __fmul_rn(f, g[h][q]);
                     }
                 }
                 w0 = n0, w1 = n1;
-#pragma unroll
-                for (int q = 0; q < 3; ++q) X[q] = nx[q], V[q] = nv[q];
             }
+            if (MODE == LFG_LD) __syncwarp();   // the stages are left before the next round's copies
             s_round = slot_add(s_round, (uint32_t)n, a.R);
             j_round += n >> 2;
             if (j_round >= a.N) j_round -= a.N, ++t_round;
@@ -291,10 +330,10 @@ __global__ void __launch_bounds__(32 * (CW + GW + 1), 1) lfg_stream_kernel(LfgAr
 // resident kernel: 15 and 12, per step of 1e6 oscillators 6.80 us (7.08 with 15 and 16,
 // 7.04 with 14 and 13, 7.12 with 13 and 14, 7.3 with 15 or 16 and 11, 7.8 with 15 and 8:
 // the generating warps' loads in flight and the using warps' arithmetic share a round).
-// The streamed one has more work a word in its using warps: 13 and 10 (1e7: 136 us a
-// step, 138 with 15 and 8, 141 with 12 and 11, 144 with 11 and 12) where a round has its
-// full width; below 2 N >= k D the narrower rounds leave less time to generate: 11 and 12
-// (1.2e6: 17.7 us a step, 18.1 with 11 and 16, 18.0 with 13 and 14, 20.1 with 15 and 12).
+// The streamed one (us a step at 1.1e6, 1.2e6, 1500001, 2e6, 1e7 oscillators): 11 and 12
+// 15.6, 15.4, 20.2, 24.6, 134; 12 and 10 16.5, 16.9, 18.6, 22.7, 129; 13 and 10 ., ., ., 24.5,
+// 130; 10 and 13 15.0, 16.2, 19.8, 25.6, 139.  A round holds at most 2 N of its k D
+// positions, so the narrow ones leave less time to generate: 11 and 12 up to 3 N = k D.
 constexpr int kResWarps = 15, kResGen = 12;
 
 template <int MODE, int CW, int GW>
@@ -307,7 +346,8 @@ static int launch_stream(Handle* h, LfgArgs& a, int k, cudaStream_t st)
     void* args[] = {&a};
     return with_depth(k, [&](auto kk) {
         constexpr int K = decltype(kk)::value;
-        return lfg_cooperative((const void*)lfg_stream_kernel<MODE, K, CW, GW>, G, 32 * (CW + GW + 1), args, 0, st);
+        return lfg_cooperative((const void*)lfg_stream_kernel<MODE, K, CW, GW>, G, 32 * (CW + GW + 1), args,
+                               MODE == LFG_LD ? stream_smem<CW>() : 0, st);
     });
 }
 
@@ -384,11 +424,12 @@ int lfg_ld(const ld_system* s, int64_t n_steps, int init, ld_stats* out, cudaStr
                                    smem, st);
         }));
     } else {
-        a.w = (int)(std::min<int64_t>((int64_t)k * a.D, 2 * s->n) & ~(int64_t)7);
-        if (2 * s->n < (int64_t)k * a.D)
+        // whole groups of four oscillators, whose x and v start on 16 bytes
+        a.w = (int)(std::min<int64_t>((int64_t)k * a.D, 2 * s->n) & ~(int64_t)15);
+        if (3 * s->n < (int64_t)k * a.D)
             GB_CHECK((launch_stream<LFG_LD, 11, 12>(h, a, k, st)));
         else
-            GB_CHECK((launch_stream<LFG_LD, 13, 10>(h, a, k, st)));
+            GB_CHECK((launch_stream<LFG_LD, 12, 10>(h, a, k, st)));
     }
     GB_CHECK(lfg_end(h, a, st));
     h->pos += a.n_pos;

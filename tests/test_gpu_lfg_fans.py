@@ -119,3 +119,53 @@ def test_small_system_timeout(G):
     st = G.ld_run(s, 100)
     xx = (s.x.double() ** 2).sum().item()
     assert abs(st["sum_x2"] / xx - 1) < 1e-12
+
+
+def shifted(t, words):
+    """A copy of t that starts `words` 4-byte words behind a 16-byte boundary."""
+    flat = torch.empty(t.numel() + 4, dtype=t.dtype, device=t.device)[words:words + t.numel()]
+    flat.copy_(t.reshape(-1))
+    return flat.view(t.shape)
+
+
+@pytest.mark.parametrize("n,row,steps,order", [
+    (400, 0, 7, 1), (401, 0, 9, 1), (403, 0, 6, 1),                  # units that cross a step's end, partial ones
+    (2000001, -1, 3, 0), (2000002, -1, 3, 0), (1200003, -1, 5, 0),   # whole units, either split of the warps
+])
+@pytest.mark.parametrize("at_x,at_v", [(0, 0), (1, 1), (2, 0), (2, 3)])
+def test_streamed_runs_at_any_alignment(G, n, row, steps, order, at_x, at_v):
+    """x and v through global memory, at every alignment of their first words (an odd N or one
+    that is no multiple of 4 moves it from step to step), each oscillator with its own K."""
+    try:
+        G.gbrng_set_lfg_order(4)          # a ring for the paper form at 4 N > 2 (ll - sl)
+        b = system(G, n, row, 2)
+        sb = G.ld_run_stepwise(b, steps)
+        G.gbrng_set_lfg_order(order)
+        a = system(G, n, row, 2)
+        a = G.LdSystem(a.rng, shifted(a.x, at_x), shifted(a.v, at_v), K_per=a.K_per)
+        sa = G.ld_run(a, steps)
+    finally:
+        G.gbrng_set_lfg_order(0)
+    assert torch.equal(a.x, b.x) and torch.equal(a.v, b.v)
+    assert G.rng_get_state(a.rng) == G.rng_get_state(b.rng)
+    assert abs(sa["sum_v2"] / sb["sum_v2"] - 1) < 1e-12          # binary64 sums
+    assert abs(sa["energy_time_avg"] / sb["energy_time_avg"] - 1) < 1e-6
+
+
+@pytest.mark.parametrize("n", [1200000, 2000000, 5000000])
+def test_streamed_runs_cost_no_more_for_odd_n(G, n):
+    """Per oscillator-step an odd N takes at most 1.3 times what the even one beside it does
+    (1.02 to 1.07 measured; 1.6 to 1.7 with a lane's words loaded one by one)."""
+    ms = {}
+    for m in (n, n + 1):
+        s = G.LdSystem(G.rng_init("lagfib", 3, m), torch.zeros((m, 3), device="cuda"), torch.zeros((m, 3), device="cuda"))
+        G.ld_run(s, 20, stats=False)
+        ev = [torch.cuda.Event(enable_timing=True) for _ in range(2)]
+        ms[m] = 1e9
+        for _ in range(5):
+            ev[0].record()
+            G.ld_run(s, 40, stats=False)
+            ev[1].record()
+            ev[1].synchronize()
+            ms[m] = min(ms[m], ev[0].elapsed_time(ev[1]) / m)
+    assert ms[n + 1] < 1.3 * ms[n]
