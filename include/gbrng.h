@@ -242,7 +242,8 @@ typedef struct {
  * 2n <= ll - sl below position ll and <= 2(ll - sl) after, else GBRNG_ELAGS and
  * nothing runs.  Requirements: n >= 1, n_steps >= 0, every >= 1, k_sp > 0,
  * xi > 0, kT >= 0, dt > 0.  Synchronises the stream when records are
- * requested; scratch (16 bytes per record per 256 particles) is the handle's. */
+ * requested.  Scratch is the handle's: 16 bytes per record per 256 particles,
+ * or up to 256 MiB where that is more; GBRNG_EINVAL beyond 4 GiB of the former. */
 int ou_run(ou_system* sys, int64_t n_steps, int64_t every, double* mean_host, double* corr_host,
            void* stream);
 

@@ -339,11 +339,11 @@ int lfg_end(Handle* h, const LfgArgs& a, cudaStream_t st);
 int lfg_cooperative(const void* fn, int64_t G, int T, void** args, size_t smem, cudaStream_t st);
 enum { LFG_U32 = 0, LFG_UNIFORM = 1, LFG_NORMAL = 2, LFG_LD = 3, LFG_LD_INIT = 4 };
 // Small systems (lfg_team.cu): 1 and launched (a.w set), 0 where they do not fit, or
-// an error.  a: of the run, x = R for the overdamped one; n_rec: its records, one
-// slot a CTA (h->partials), or 0.
+// an error.  a: of the run, x = R for the overdamped one; R0: R(0); n_rec: its
+// records, one slot a CTA (h->partials), or 0.
 int lfg_team_ld(Handle* h, LfgArgs& a, int k, int64_t n_steps, cudaStream_t st);
-int lfg_team_ou(Handle* h, LfgArgs& a, int k, OuCoef c, int64_t n_steps, int64_t every, int64_t n_rec,
-                cudaStream_t st);
+int lfg_team_ou(Handle* h, LfgArgs& a, int k, OuCoef c, const float* R0, int64_t n_steps, int64_t every,
+                int64_t n_rec, cudaStream_t st);
 
 // f(integral constant K) for a depth k.
 template <class F>

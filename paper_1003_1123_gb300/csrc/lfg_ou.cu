@@ -3,6 +3,7 @@
 #include <algorithm>
 
 #include "lfg.cuh"
+#include "records.h"
 
 namespace gb {
 
@@ -19,6 +20,7 @@ struct OuLfgArgs {
     LfgArgs l;
     OuCoef c;
     float* R;
+    const float* R0;   // R(0): R itself, or a copy where a run takes several launches
     int64_t every;     // steps between records
     double* records;   // or null
     int n_c, slots;    // particles and record slots of a CTA
@@ -38,7 +40,7 @@ __global__ void __launch_bounds__(32 * (NW + GW + 1), 1) lfg_ou_kernel(OuLfgArgs
     const int S = a.w / (int)(2 * a.N);   // steps a round
     const int64_t n_rounds = (a.n_pos + a.w - 1) / a.w;
     if (threadIdx.x == 0) s_failed = kNoRound;
-    for (int i = threadIdx.x; i < nc; i += T) ou_sm[i] = ou_sm[n_pad + i] = o.R[j0 + i];
+    for (int i = threadIdx.x; i < nc; i += T) ou_sm[i] = o.R[j0 + i], ou_sm[n_pad + i] = o.R0[j0 + i];
     __syncthreads();
     if (warp >= NW + GW) {
         wait_warp(a, n_rounds, 32 * (GW + 1), T, &s_failed);
@@ -117,26 +119,19 @@ __global__ void __launch_bounds__(32 * (NW + GW + 1), 1) lfg_ou_kernel(OuLfgArgs
     for (int i = threadIdx.x; i < nc; i += T) o.R[j0 + i] = ou_sm[i];
 }
 
-constexpr int kOuWarps = 15, kOuGen = 16;
+constexpr int kOuGen = 16;
 
-int lfg_ou(const ou_system* s, int64_t n_steps, int64_t every, double* mean, double* corr, cudaStream_t st)
+// One launch: n_steps steps, records after 0, every, ... of them.
+static int launch_ou(const ou_system* s, const float* R0, int64_t n_steps, int64_t every, double* mean, double* corr,
+                     cudaStream_t st)
 {
     Handle* h = s->rng;
     const int64_t two_n = 2 * s->n, D = (int64_t)h->ll - h->sl;
-    if (two_n > lfg_step_width(h))
-        return fail(GBRNG_ELAGS,
-                    "one round per step needs 2N = %lld within %lld times the lag distance "
-                    "(ll - sl = %lld)",
-                    (long long)two_n, (long long)(lfg_step_width(h) / D), (long long)D);
     DevInfo di;
     GB_CHECK(dev_info(h->device, &di));
     const int64_t G = di.sms;
     const bool rec = mean != nullptr;
     const int64_t n_rec = n_steps / every + 1;
-    if (rec && (n_rec > 0x7fffffff ||
-                (double)n_rec * (double)std::min<int64_t>(4 * G, (s->n + 255) / 256) * 16.0 > 4.0 * (1 << 30)))
-        return fail(GBRNG_EINVAL, "%lld records of %lld particles exceed the record scratch", (long long)n_rec,
-                    (long long)s->n);
     // the depth set may be below the width a step needs (whole quads): no deeper than D allows
     const int k = lfg_depth(h);
     OuLfgArgs o{};
@@ -146,7 +141,7 @@ int lfg_ou(const ou_system* s, int64_t n_steps, int64_t every, double* mean, dou
     o.l.n_pos = two_n * n_steps;
     o.l.vec = o.l.vec && s->n % 2 == 0;   // every step from a multiple of 4 on
     o.l.x = s->R;
-    if (const int rc = lfg_team_ou(h, o.l, k, make_ou_coef(s), n_steps, every, rec ? n_rec : 0, st)) {
+    if (const int rc = lfg_team_ou(h, o.l, k, make_ou_coef(s), R0, n_steps, every, rec ? n_rec : 0, st)) {
         if (rc < 0) return rc;
         GB_CHECK(lfg_end(h, o.l, st));
         h->pos += o.l.n_pos;
@@ -156,11 +151,11 @@ int lfg_ou(const ou_system* s, int64_t n_steps, int64_t every, double* mean, dou
     o.l.w = (int)(two_n * S);
     o.c = make_ou_coef(s);
     o.R = s->R;
+    o.R0 = R0;
     o.every = every;
-    o.n_c = (int)(((s->n + G - 1) / G + 1) & ~(int64_t)1);
+    o.n_c = (int)lfg_share(s->n, di.sms);
     const bool steps = S >= 4 && o.n_c <= 32 * kOuWarps * 2;
-    const int up = steps ? 32 : 64;
-    o.slots = std::min(kOuWarps, (o.n_c + up - 1) / up);
+    o.slots = lfg_record_slots(o.n_c, steps ? 32 : 64);
     if (rec) {
         const int64_t blocks = G * o.slots;
         GB_CHECK(ensure_partials(h, (2 * n_rec * blocks + 2 * n_rec + 3) / 4));
@@ -181,6 +176,37 @@ int lfg_ou(const ou_system* s, int64_t n_steps, int64_t every, double* mean, dou
         h->pos += o.l.n_pos;
     }
     if (rec) return ou_finish(h, s->n, n_rec, G * o.slots, mean, corr, st);
+    return GBRNG_OK;
+}
+
+int lfg_ou(const ou_system* s, int64_t n_steps, int64_t every, double* mean, double* corr, cudaStream_t st)
+{
+    Handle* h = s->rng;
+    const int64_t two_n = 2 * s->n, D = (int64_t)h->ll - h->sl;
+    const int order = (int)((lfg_step_width(h) + D - 1) / D);
+    if (two_n > lfg_step_width(h))
+        return fail(GBRNG_ELAGS,
+                    "one round per step needs 2N = %lld within %lld times the lag distance "
+                    "(ll - sl = %lld)",
+                    (long long)two_n, (long long)(lfg_step_width(h) / D), (long long)D);
+    DevInfo di;
+    GB_CHECK(dev_info(h->device, &di));
+    const int64_t n_rec = n_steps / every + 1;
+    if (mean && records_refused(n_rec, lfg_record_blocks(s->n, di.sms, order)))
+        return fail(GBRNG_EINVAL, "%lld records of %lld particles exceed the record scratch", (long long)n_rec,
+                    (long long)s->n);
+    const int64_t most = lfg_launch_records(s->n, di.sms);
+    if (!mean || n_rec <= most) return launch_ou(s, s->R, n_steps, every, mean, corr, st);
+    // launches of `most` records, the first of each the last of the one before, all against
+    // R(0) of the run
+    GB_CHECK(ensure_eacc(h, s->n));
+    float* R0 = reinterpret_cast<float*>(h->eacc);
+    GB_CUDA(cudaMemcpyAsync(R0, s->R, sizeof(float) * s->n, cudaMemcpyDeviceToDevice, st));
+    for (int64_t r = 0; r < n_rec - 1; r += most - 1) {
+        const int64_t left = n_steps - r * every;
+        const int64_t steps = r + most - 1 < n_rec - 1 ? (most - 1) * every : left;
+        GB_CHECK(launch_ou(s, R0, steps, every, mean + r, corr + r, st));
+    }
     return GBRNG_OK;
 }
 

@@ -25,6 +25,7 @@ enum { LFG_TEAM_LD = 0, LFG_TEAM_OU = 1 };
 struct LfgTeamArgs {
     LfgArgs l;
     OuCoef oc;
+    const float* R0;   // OU: R(0)
     int64_t every;     // OU: steps between records
     double* records;   // OU: [record][CTA][2] or null
     int n_c;           // oscillators of a CTA, even
@@ -86,7 +87,7 @@ __global__ void __launch_bounds__(kTeamThreads, 1) lfg_team_kernel(LfgTeamArgs o
         nck = -__fmul_rn(a.c.ckm, k);
         hK = 0.5f * k;
     }
-    const float R0 = x;
+    const float R0 = MODEL == LFG_TEAM_OU && live ? o.R0[at] : 0.f;
     Kahan2 e;   // LD: sums of x^2 and v^2
     int64_t t = 0, rec = 0, next_rec = 0;
     auto record = [&](float Rt) {
@@ -224,8 +225,8 @@ int lfg_team_ld(Handle* h, LfgArgs& a, int k, int64_t n_steps, cudaStream_t st)
     return 1;
 }
 
-int lfg_team_ou(Handle* h, LfgArgs& a, int k, OuCoef c, int64_t n_steps, int64_t every, int64_t n_rec,
-                cudaStream_t st)
+int lfg_team_ou(Handle* h, LfgArgs& a, int k, OuCoef c, const float* R0, int64_t n_steps, int64_t every,
+                int64_t n_rec, cudaStream_t st)
 {
     DevInfo di;
     GB_CHECK(dev_info(h->device, &di));
@@ -233,6 +234,7 @@ int lfg_team_ou(Handle* h, LfgArgs& a, int k, OuCoef c, int64_t n_steps, int64_t
     size_t smem = 0;
     if (!team_fits(LFG_TEAM_OU, a, k, n_steps, di, &o.n_c, &smem)) return 0;
     o.oc = c;
+    o.R0 = R0;
     o.every = every;
     if (n_rec) {
         GB_CHECK(ensure_partials(h, (2 * n_rec * di.sms + 2 * n_rec + 3) / 4));

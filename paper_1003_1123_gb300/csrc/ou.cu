@@ -8,6 +8,7 @@
 
 #include "device.cuh"
 #include "internal.cuh"
+#include "records.h"
 
 namespace gb {
 
@@ -181,20 +182,17 @@ int ou_run_pt(const ou_system* s, int64_t n_steps, int64_t every, double* mean, 
     // 256 threads a block, or 128 where that leaves the busiest SM fewer warps (1e4
     // particles x 1000 steps 112 -> 84 us for Hybrid Taus, 4e4 175 -> 142, 2e5 x 200
     // 125 -> 114; elsewhere, with twice the blocks to sum up, up to 2% slower)
-    auto too_many = [&](int64_t blocks) { return n_rec > 0x7fffffff || (double)n_rec * blocks * 16.0 > 4.0 * (1 << 30); };
     auto busiest = [&](int64_t threads) { return threads * (((s->n + threads - 1) / threads + di.sms - 1) / di.sms); };
-    const int T = busiest(128) < busiest(256) && !(rec && too_many((s->n + 127) / 128)) ? 128 : 256;
+    const int T = busiest(128) < busiest(256) && (!rec || records_fit(n_rec, (s->n + 127) / 128, s->n)) ? 128 : 256;
     const int64_t blocks = (s->n + T - 1) / T;
+    if (rec && records_refused(n_rec, record_blocks(s->n)))
+        return fail(GBRNG_EINVAL, "%lld records x %lld blocks exceed the record scratch",
+                    (long long)n_rec, (long long)record_blocks(s->n));
     int64_t team_blocks = 0;
     const int rc = ou_team(s, n_steps, every, rec, &team_blocks, st);
     if (rc < 0) return rc;
     if (rc == 1) return rec ? ou_finish(h, s->n, n_rec, team_blocks, mean, corr, st) : GBRNG_OK;
-    if (rec) {
-        if (too_many(blocks))
-            return fail(GBRNG_EINVAL, "%lld records x %lld blocks exceed the record scratch",
-                        (long long)n_rec, (long long)blocks);
-        GB_CHECK(ensure_partials(h, (2 * n_rec * blocks + 2 * n_rec + 3) / 4));
-    }
+    if (rec) GB_CHECK(ensure_partials(h, (2 * n_rec * blocks + 2 * n_rec + 3) / 4));
     OuArgs a;
     a.n = s->n;
     a.n_steps = n_steps;

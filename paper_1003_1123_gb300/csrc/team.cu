@@ -36,6 +36,7 @@
 
 #include "jump.cuh"
 #include "internal.cuh"
+#include "records.h"
 
 namespace gb {
 
@@ -509,7 +510,7 @@ int ou_team(const ou_system* s, int64_t n_steps, int64_t every, bool rec, int64_
     const bool small = s->n <= (int64_t)16 * di.sms;
     const int64_t blocks = small ? (s->n + 7) / 8 : (s->n + 15) / 16, n_rec = n_steps / every + 1;
     if (rec) {
-        if (n_rec > 0x7fffffff || (double)n_rec * blocks * 16.0 > 4.0 * (1 << 30)) return 0;
+        if (!records_fit(n_rec, blocks, s->n)) return 0;
         GB_CHECK(ensure_partials(h, (2 * n_rec * blocks + 2 * n_rec + 3) / 4));
     }
     TeamArgs a{};
