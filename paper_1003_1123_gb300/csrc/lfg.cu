@@ -301,11 +301,17 @@ int lfg_depth(const Handle* h)
     return o ? std::min(o, h->depth) : h->depth;
 }
 
-// k D positions (whole quads), k the order set, or 2.
-int64_t lfg_step_width(const Handle* h)
+// The order set, at most the handle's, or 2.
+int lfg_step_order(const Handle* h)
 {
     const int o = g_lfg_order.load();
-    return ((o ? std::min(o, h->order_max) : 2) * ((int64_t)h->ll - h->sl)) & ~(int64_t)3;
+    return o ? std::min(o, h->order_max) : 2;
+}
+
+// k D positions of that order k (whole quads).
+int64_t lfg_step_width(const Handle* h)
+{
+    return (lfg_step_order(h) * ((int64_t)h->ll - h->sl)) & ~(int64_t)3;
 }
 
 // Barrier counter, status words, wait limit and test hook of one launch.
@@ -383,9 +389,9 @@ int lfg_ld_stepwise(const ld_system* s, int64_t n_steps, ld_stats* out, cudaStre
     const int64_t four_n = 4 * s->n;
     if (four_n > lfg_step_width(h))
         return fail(GBRNG_ELAGS,
-                    "one launch per step needs 4N = %lld within %lld times the lag distance "
+                    "one launch per step needs 4N = %lld within %d times the lag distance "
                     "(ll - sl = %lld)",
-                    (long long)four_n, (long long)(lfg_step_width(h) / (h->ll - h->sl)), (long long)(h->ll - h->sl));
+                    (long long)four_n, lfg_step_order(h), (long long)(h->ll - h->sl));
     GB_CHECK(ensure_eacc(h, s->n));
     GB_CUDA(cudaMemsetAsync(h->eacc, 0, sizeof(float2) * s->n, st));
     LfgArgs a = lfg_args(h);

@@ -330,7 +330,8 @@ struct Kahan2 {
 LfgArgs lfg_args(const Handle* h);
 // Fan depth of a launch: the process-wide setting, else the ring's own.
 int lfg_depth(const Handle* h);
-// The widest step (positions) of the paper form and of the overdamped run.
+// Order and width (positions) of the widest step of the paper form and the overdamped run.
+int lfg_step_order(const Handle* h);
 int64_t lfg_step_width(const Handle* h);
 // Barrier counter, status words, wait limit and test hook of a launch of G CTAs.
 int lfg_begin(Handle* h, LfgArgs& a, int64_t G, cudaStream_t st);

@@ -183,16 +183,15 @@ int lfg_ou(const ou_system* s, int64_t n_steps, int64_t every, double* mean, dou
 {
     Handle* h = s->rng;
     const int64_t two_n = 2 * s->n, D = (int64_t)h->ll - h->sl;
-    const int order = (int)((lfg_step_width(h) + D - 1) / D);
     if (two_n > lfg_step_width(h))
         return fail(GBRNG_ELAGS,
-                    "one round per step needs 2N = %lld within %lld times the lag distance "
+                    "one round per step needs 2N = %lld within %d times the lag distance "
                     "(ll - sl = %lld)",
-                    (long long)two_n, (long long)(lfg_step_width(h) / D), (long long)D);
+                    (long long)two_n, lfg_step_order(h), (long long)D);
     DevInfo di;
     GB_CHECK(dev_info(h->device, &di));
     const int64_t n_rec = n_steps / every + 1;
-    if (mean && records_refused(n_rec, lfg_record_blocks(s->n, di.sms, order)))
+    if (mean && records_refused(n_rec, lfg_record_blocks(s->n, di.sms, lfg_step_order(h))))
         return fail(GBRNG_EINVAL, "%lld records of %lld particles exceed the record scratch", (long long)n_rec,
                     (long long)s->n);
     const int64_t most = lfg_launch_records(s->n, di.sms);

@@ -169,3 +169,19 @@ def test_streamed_runs_cost_no_more_for_odd_n(G, n):
             ev[1].synchronize()
             ms[m] = min(ms[m], ev[0].elapsed_time(ev[1]) / m)
     assert ms[n + 1] < 1.3 * ms[n]
+
+
+@pytest.mark.parametrize("order", [1, 2, 4])
+def test_too_wide_a_step_names_the_order(G, order):
+    """A step beyond k (ll - sl) positions is refused, and the message says which k."""
+    try:
+        G.gbrng_set_lfg_order(order)
+        sl, ll = G.rng_lfg_lags(0)
+        n = order * (ll - sl) // 2 + 1
+        R = torch.zeros(n, device="cuda")
+        s = system(G, n, 0, 0)
+        for call in (lambda: G.ou_run(G.OuSystem(s.rng, R), 1), lambda: G.ld_run_stepwise(s, 1)):
+            with pytest.raises(G.GbrngError, match="within %d times the lag distance" % order):
+                call()
+    finally:
+        G.gbrng_set_lfg_order(0)
