@@ -33,3 +33,54 @@ def test_split_equals_short_fills(G, kind, op, streams, items):
     assert torch.equal(whole.view(torch.int32), parts.view(torch.int32))
     # a partial last row leaves the streams' own counts: compare the next draws too
     assert G.rng_get_state(a) == G.rng_get_state(b)
+
+
+@pytest.mark.parametrize("kind", ["taus", "lcg"])
+@pytest.mark.parametrize("op", ["u32", "uniform"])
+@pytest.mark.parametrize("streams,words,offset", [
+    (2051, 777, 0),       # segments, 64 streams a cluster, the last cluster and item partial
+    (5001, 0, 0), (20001, 5, 3),
+    (60799, 60000, 0),    # few segments, or one thread a stream
+    (100001, 1, 0), (999999, 999998, 0),   # one thread a stream
+    (4096, 11, 1),        # rows of whole sectors, from an address that is not
+])
+def test_ragged_rows_of_long_fills(G, kind, op, streams, words, offset):
+    """Rows that are not whole sectors in fills larger than the L2 keeps, whose threads stay
+    together: equal to short fills, with nothing written beside them."""
+    fill = {"u32": G.rng_fill_u32, "uniform": G.rng_fill_uniform}[op]
+    dtype = torch.int32 if op == "u32" else torch.float32
+    n = (192 << 20) // 4 + words
+    a, b = G.rng_init(kind, 43, streams), G.rng_init(kind, 43, streams)
+    room = torch.full((n + 64,), -1, dtype=dtype, device="cuda")
+    whole = room[16 + offset:16 + offset + n]
+    fill(a, n, out=whole)
+    row = max(1, 2**21 // streams) * streams
+    part = torch.empty(row, dtype=dtype, device="cuda")
+    for k in range(0, n, row):
+        m = min(row, n - k)
+        fill(b, m, out=part[:m])
+        assert torch.equal(whole[k:k + m].view(torch.int32), part[:m].view(torch.int32))
+    assert bool((room[:16 + offset] == -1).all()) and bool((room[16 + offset + n:] == -1).all())
+    assert G.rng_get_state(a) == G.rng_get_state(b)
+
+
+@pytest.mark.parametrize("kind,op", [("taus", "u32"), ("lcg", "uniform")])
+@pytest.mark.parametrize("streams", [24001, 33691, 208529, 500001])
+def test_ragged_rows_cost_little(G, kind, op, streams):
+    """2^28 items of an odd number of streams take at most 1.6 times what the next multiple of 8,
+    whose rows are whole sectors, takes (1.1 to 1.3 measured; 1.8 to 2.5 with the warps apart)."""
+    fill = {"u32": G.rng_fill_u32, "uniform": G.rng_fill_uniform}[op]
+    out = torch.empty(2**28, dtype=torch.int32 if op == "u32" else torch.float32, device="cuda")
+    ms = []
+    for s in (streams, (streams + 7) // 8 * 8):
+        r = G.rng_init(kind, 3, s)
+        ev = [torch.cuda.Event(enable_timing=True) for _ in range(2)]
+        best = 1e9
+        for _ in range(6):
+            ev[0].record()
+            fill(r, 2**28, out=out)
+            ev[1].record()
+            ev[1].synchronize()
+            best = min(best, ev[0].elapsed_time(ev[1]))
+        ms.append(best)
+    assert ms[0] < 1.6 * ms[1]
