@@ -106,9 +106,9 @@ __global__ void __launch_bounds__(64, 8) adjoint_kernel(AdjArgs a)
                     td.y.w = __float_as_uint(src[3 * stride]);
                 }
             } else if (!src) {
-                rd.load(a.r2 + i, a.streams, tab, blockDim.x);
+                rd.load<16>(a.r2 + i, a.streams, tab, blockDim.x);
             } else {
-                rd.load(src, stride, tab, blockDim.x);
+                rd.load<16>(src, stride, tab, blockDim.x);
             }
         };
         auto save_state = [&](float* dst, int64_t stride) {
@@ -118,7 +118,7 @@ __global__ void __launch_bounds__(64, 8) adjoint_kernel(AdjArgs a)
                 dst[2 * stride] = __uint_as_float(td.y.z);
                 dst[3 * stride] = __uint_as_float(td.y.w);
             } else {
-                rd.store(dst, stride);
+                rd.store<16>(dst, stride);
             }
         };
         // ---------------- A: forward with checkpoints
@@ -152,7 +152,7 @@ __global__ void __launch_bounds__(64, 8) adjoint_kernel(AdjArgs a)
         if (KIND == GBRNG_TAUS) {
             a.taus[i] = td.y;
         } else {
-            rd.store(a.r2 + i, a.streams);
+            rd.store<16>(a.r2 + i, a.streams);
         }
         // ---------------- B: reverse sweep
         const float inv_ab = __frcp_rn(__fmaf_rn(ckx, c.cdt, c.cva));

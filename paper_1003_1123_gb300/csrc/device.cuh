@@ -549,7 +549,10 @@ struct LcgDraw {
 
 // Ran2 with its shuffle table in a column of shared memory.  A stored state is 35
 // words at a stride: idum, idum2, iy and the entries (int32_t in the generator, their
-// bits as float in a checkpoint).
+// bits as float in a checkpoint).  AT_ONCE entries are in flight together: 16 where a run may
+// have few steps, or a checkpoint each, to hide them behind (one step of 3e6 oscillators,
+// two a thread, 266 us with four, 246 with 16, 235 with 32; adjoint of 3e5 x 20 with 20
+// checkpoints 775, 573, 576; ld_run of 1e6 x 100 570, 558, 574).
 __device__ __forceinline__ int32_t word_bits(int32_t w) { return w; }
 __device__ __forceinline__ int32_t word_bits(float w) { return __float_as_int(w); }
 __device__ __forceinline__ void put_bits(int32_t& w, int32_t b) { w = b; }

@@ -150,7 +150,7 @@ __global__ void __launch_bounds__(32) ld_pair_kernel(LdArgs a, int64_t n_pairs)
             } else if (KIND == GBRNG_LCG) {
                 lc[j].x = a.lcg[i];
             } else {
-                rd[j].load(a.r2 + i, a.S, tab + j * 32 * blockDim.x, 32);
+                rd[j].load<16>(a.r2 + i, a.S, tab + j * 32 * blockDim.x, 32);
             }
         }
         nckx = make_float2(ck[0], ck[1]);
@@ -190,7 +190,7 @@ __global__ void __launch_bounds__(32) ld_pair_kernel(LdArgs a, int64_t n_pairs)
             } else if (KIND == GBRNG_LCG) {
                 a.lcg[i] = lc[j].x;
             } else {
-                rd[j].store(a.r2 + i, a.S);
+                rd[j].store<16>(a.r2 + i, a.S);
             }
             acc[0] += (double)x0 * x0 + (double)x1 * x1 + (double)x2 * x2;
             acc[1] += (double)v0 * v0 + (double)v1 * v1 + (double)v2 * v2;
