@@ -292,29 +292,42 @@ int ld_init_pt(const ld_system* s, cudaStream_t st)
 // step, which for the thread-per-oscillator kernels goes by the warps on the
 // busiest scheduler (w1 with one oscillator a thread, w2 with two) and for the
 // teams by the oscillators a SM holds, besides their start-up (the jumps).  The
-// costs are measured, ns a step over 1000 steps, one a thread by w1, two a thread by
-// w2; teams 9 + 0.67 per oscillator a SM for Hybrid Taus and 6 + 0.48 for the LCG,
-// and 2.5 us + 0.3 (LCG 0.2) us per 1000 oscillators at the start beyond the others'.
-// Above w1 = 7 two a thread are faster for every generator (155600 oscillators: 630
-// against 831, 488 against 584 and 812 against 934).
+// costs are measured, ns a step over 3000 steps, one a thread by w1, two a thread by w2;
+// teams with statistics repeat every update in their producer warps, a fifth more a step
+// (the thread-per-oscillator kernels sum the energies in any case).  Without that in the
+// rule, runs with statistics took a team too far: 1.1e5 LCG oscillators 522 ns a step instead
+// of 365 by two a thread, 58368 257 instead of 198 by one.  Above w1 = 8 two a thread.
 enum LdPath { LD_ONE, LD_PAIRS, LD_TEAM };
 struct LdCost {
-    double one[7], pairs[4];
-    double team0, team, start0, start;   // ns: a step, per oscillator a SM; start, per oscillator
+    double one[8], pairs[4], pairs_start;
+    // ns: a step, and per oscillator a SM; the start, and per oscillator
+    struct Team {
+        double step0, step, start0, start;
+    } team[2];   // without statistics, with
 };
-constexpr LdCost kCostTaus = {{119, 193, 287, 380, 469, 559, 651}, {183, 326, 478, 629}, 9, 0.67, 2500, 0.3};
-constexpr LdCost kCostLcg = {{92, 142, 208, 271, 333, 396, 458}, {166, 255, 376, 488}, 6, 0.48, 2500, 0.2};
-constexpr LdCost kCostRan2 = {{191, 254, 350, 451, 548, 645, 838}, {277, 429, 628, 812}, 1e300, 0, 0, 0};   // no team
+constexpr LdCost kCostTaus = {{113, 188, 286, 375, 467, 557, 649, 739}, {175, 320, 471, 621}, 1500,
+                              {{4, 0.755, 1500, 0.3}, {5, 0.89, 6000, 0.44}}};
+constexpr LdCost kCostLcg = {{86, 132, 198, 259, 320, 382, 443, 504}, {151, 246, 365, 477}, 1500,
+                             {{3, 0.56, 1000, 0.18}, {4, 0.665, 4000, 0.34}}};
+constexpr LdCost kCostRan2 = {{183, 245, 340, 440, 537, 631, 729, 824}, {266, 418, 615, 800}, 400,
+                              {{1e300, 0, 0, 0}, {1e300, 0, 0, 0}}};   // no team
 
-static LdPath pick_path(int kind, int64_t n, int64_t n_steps, int sms)
+static LdPath pick_path(int kind, int64_t n, int64_t n_steps, bool stats, int sms)
 {
     const int64_t w1 = (n + 128ll * sms - 1) / (128ll * sms), w2 = (n + 256ll * sms - 1) / (256ll * sms);
-    if (w1 > 7) return LD_PAIRS;
+    if (w1 > 8) return LD_PAIRS;
     const LdCost& c = kind == GBRNG_TAUS ? kCostTaus : kind == GBRNG_LCG ? kCostLcg : kCostRan2;
-    const double one = c.one[w1 - 1], pairs = c.pairs[w2 - 1];
-    const double team = c.team0 + c.team * (double)n / sms +
-                        (c.start0 + c.start * (double)n) / (double)std::max<int64_t>(n_steps, 1);
-    if (team < std::min(one, pairs)) return LD_TEAM;
+    const LdCost::Team& t = c.team[stats];
+    const double steps = (double)n_steps;
+    // the blocks' sums, added up by the last block or by a second kernel
+    auto sums = [&](int64_t blocks) { return !stats ? 0.0 : blocks <= kFuseBlocks ? 11.5 * (double)blocks : 4000.0; };
+    const double one = c.one[w1 - 1] * steps + sums(n / (w1 <= 2 || kind == GBRNG_RAN2 ? 32 : 128));
+    const double pairs = c.pairs[w2 - 1] * steps + c.pairs_start + sums(n / 64);
+    // a start counts in full up to some 80 steps; in long runs the blocks drift apart, and the
+    // jumps of one pass beside another's steps: less than nothing from 290 on
+    const double seen = std::min(1.0, std::max(-0.35, 1.0 - (steps - 80.0) / 210.0));
+    const double team = (t.step0 + t.step * (double)n / sms) * steps + (t.start0 + t.start * (double)n) * seen;
+    if (n_steps > 0 && team < std::min(one, pairs)) return LD_TEAM;
     return pairs < one ? LD_PAIRS : LD_ONE;
 }
 
@@ -333,7 +346,7 @@ int ld_run_pt(const ld_system* s, int64_t n_steps, ld_stats* out, cudaStream_t s
     }
     DevInfo di;
     GB_CHECK(dev_info(s->rng->device, &di));
-    const LdPath path = pick_path(s->rng->kind, s->n, n_steps, di.sms);
+    const LdPath path = pick_path(s->rng->kind, s->n, n_steps, out != nullptr, di.sms);
     if (path == LD_TEAM) return ld_team(s, n_steps, out, st);
     if (s->rng->kind == GBRNG_TAUS) return run_kind<GBRNG_TAUS>(s, path, n_steps, out, st);
     if (s->rng->kind == GBRNG_LCG) return run_kind<GBRNG_LCG>(s, path, n_steps, out, st);
