@@ -127,17 +127,19 @@ __global__ void __launch_bounds__(32 * (kFillWarps + 1), 1) lfg_fill_kernel(LfgA
 }
 
 // -------------------------------------------------------- single positions
-// The value of the position in slot s that lies k D to (k + 1) D after the first
-// position not in the ring, computed by itself: k + 1 applications of the
-// recurrence, x_q = sum_i C(k + 1, i) x_{q - (k+1) D - i sl}.
-__device__ __forceinline__ uint32_t lag_value(const LfgArgs& a, uint32_t s, int k)
+// The value of the position in slot s that lies p < 4 D after the first position not in the
+// ring, computed by itself: n = p div D + 1 applications of the recurrence, x_q = sum_i C(n,
+// i) x_{q - n D - i sl}, its n + 1 loads side by side.
+__device__ __forceinline__ uint32_t lag_value(const LfgArgs& a, uint32_t s, int64_t p)
 {
-    uint32_t t = s;
-    for (int i = 0; i <= k; ++i) t = slot_sub(t, a.D, a.R);
-    uint32_t sum = 0, c = 1;
-    for (int i = 0; i <= k + 1; ++i) {
-        sum += c * __ldcg(a.ring + t);
-        c = c * (uint32_t)(k + 1 - i) / (uint32_t)(i + 1);
+    const int n = 1 + (p >= a.D) + (p >= 2ll * a.D) + (p >= 3ll * a.D);
+    const uint32_t binom = n == 1 ? 0x11u : n == 2 ? 0x121u : n == 3 ? 0x1331u : 0x14641u;   // C(n, i), a digit each
+    uint32_t t = s, sum = 0;
+#pragma unroll
+    for (int i = 0; i < 4; ++i) t = i < n ? slot_sub(t, a.D, a.R) : t;
+#pragma unroll
+    for (int i = 0; i <= 4; ++i) {
+        if (i <= n) sum += (binom >> (4 * i) & 15u) * __ldcg(a.ring + t);
         t = slot_sub(t, a.sl, a.R);
     }
     return sum;
@@ -156,26 +158,30 @@ __global__ void __launch_bounds__(256) lfg_step_kernel(LfgArgs a, uint32_t sP, f
     if (j >= a.N) return;
     const uint32_t s = slot_add(sP, (uint32_t)(4 * j), a.R);   // 4j < 4N < R
     uint32_t w[4];
-    // all four by one application of the recurrence or all by two, as nearly everywhere:
-    // the loads then stand side by side (one after another 1e4 oscillators take 6.2 us a
-    // step instead of a launch's 4.1, 1e6 26.7 instead of 20.6)
+    // all four by one application of the recurrence, or each by one or two, as nearly
+    // everywhere: the loads then stand side by side (one after another 1e4 oscillators take 6.2
+    // us a step instead of a launch's 4.1, 1e6 26.7 instead of 20.9).  The quad across D is
+    // among the latter: by itself its words' loops kept a step of any small row at 6.3 us.
     if (4 * j + 3 < a.D) {
 #pragma unroll
         for (int r = 0; r < 4; ++r) {
             const uint32_t t = slot_sub(slot_add(s, r, a.R), a.D, a.R);
             w[r] = __ldcg(a.ring + t) + __ldcg(a.ring + slot_sub(t, a.sl, a.R));
         }
-    } else if (4 * j >= a.D && 4 * j + 3 < 2ll * a.D) {
+    } else if (4 * j + 3 < 2ll * a.D) {
 #pragma unroll
         for (int r = 0; r < 4; ++r) {
-            uint32_t t = slot_sub(slot_sub(slot_add(s, r, a.R), a.D, a.R), a.D, a.R);
+            const bool two = 4 * j + r >= a.D;
+            uint32_t t = slot_sub(slot_add(s, r, a.R), a.D, a.R);
+            if (two) t = slot_sub(t, a.D, a.R);
             const uint32_t b0 = __ldcg(a.ring + t);
             t = slot_sub(t, a.sl, a.R);
-            w[r] = b0 + 2 * __ldcg(a.ring + t) + __ldcg(a.ring + slot_sub(t, a.sl, a.R));
+            const uint32_t b1 = __ldcg(a.ring + t), b2 = two ? __ldcg(a.ring + slot_sub(t, a.sl, a.R)) : 0u;
+            w[r] = b0 + b1 + (two ? b1 + b2 : 0u);
         }
     } else {
 #pragma unroll
-        for (int r = 0; r < 4; ++r) w[r] = lag_value(a, slot_add(s, r, a.R), (int)((4 * j + r) / a.D));
+        for (int r = 0; r < 4; ++r) w[r] = lag_value(a, slot_add(s, r, a.R), 4 * j + r);
     }
 #pragma unroll
     for (int r = 0; r < 4; ++r) __stcg(a.ring + slot_add(s, r, a.R), w[r]);

@@ -185,3 +185,41 @@ def test_too_wide_a_step_names_the_order(G, order):
                 call()
     finally:
         G.gbrng_set_lfg_order(0)
+
+
+@pytest.mark.parametrize("row,n", [(0, 500), (4, 4195), (6, 30000)])
+def test_paper_form_steps_across_d_cost_no_more(G, row, n):
+    """A step whose 4 N positions pass the lag distance D takes a launch's time, as one of
+    fewer: at most 1.25 times that (1.0 measured; 1.5 with the quad across D word by word)."""
+    sl, ll = G.rng_lfg_lags(row)
+    assert ll - sl < 4 * n < 2 * (ll - sl)
+    us = []
+    for m in ((ll - sl) // 4 - 10, n):
+        s = system(G, m, row, 0)
+        best = 1e9
+        G.ld_run_stepwise(s, 200, stats=False)
+        for _ in range(5):
+            ev = [torch.cuda.Event(enable_timing=True) for _ in range(2)]
+            ev[0].record()
+            G.ld_run_stepwise(s, 400, stats=False)
+            ev[1].record()
+            ev[1].synchronize()
+            best = min(best, ev[0].elapsed_time(ev[1]))
+        us.append(best)
+    assert us[1] < 1.25 * us[0]
+
+
+@pytest.mark.parametrize("row,n", [(0, 700), (0, 1028), (2, 4186), (3, 9841), (4, 6087)])
+@pytest.mark.parametrize("skip", [0, 3])
+def test_paper_form_of_wide_steps(G, row, n, skip):
+    """Steps of 2 to 4 lag distances (order 4): quads within and across each of them."""
+    try:
+        G.gbrng_set_lfg_order(4)
+        a = system(G, n, row, skip)
+        G.ld_run_stepwise(a, 7)
+    finally:
+        G.gbrng_set_lfg_order(0)
+    b = system(G, n, row, skip)
+    G.ld_run(b, 7)
+    assert torch.equal(a.x, b.x) and torch.equal(a.v, b.v)
+    assert G.rng_get_state(a.rng) == G.rng_get_state(b.rng)
