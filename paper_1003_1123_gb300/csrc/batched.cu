@@ -539,7 +539,7 @@ extern "C" int ld_run_batched(ld_system* sys, int n_sys, int64_t n_steps, const 
         h = copy.data();
     }
     GB_CUDA(cudaMemcpyAsync(h, p->dstats, bytes, cudaMemcpyDeviceToHost, st));
-    GB_CUDA(cudaStreamSynchronize(st));
+    GB_CHECK(sync_results(st));
     for (int s = 0; s < n_sys; ++s) {
         out[s].sum_x2 = h[4 * s];
         out[s].sum_v2 = h[4 * s + 1];

@@ -144,6 +144,8 @@ int ou_team(const ou_system* s, int64_t n_steps, int64_t every, bool rec, int64_
 // before it returns.  Null if it cannot be allocated.
 constexpr size_t kHostBlock = 65536;
 void* host_block();
+// Wait for st before the block is read (a failure leaves the thread without that block).
+int sync_results(cudaStream_t st);
 
 // Statistics.  make_sink: where a launch of `blocks` blocks leaves its sums
 // (partials grown if needed).  finish_stats: add them up if the launch has not,

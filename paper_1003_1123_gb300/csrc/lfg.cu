@@ -339,7 +339,7 @@ int lfg_begin(Handle* h, LfgArgs& a, int64_t G, cudaStream_t st)
 
 int lfg_end(Handle* h, const LfgArgs& a, cudaStream_t st)
 {
-    GB_CUDA(cudaStreamSynchronize(st));
+    GB_CHECK(sync_results(st));
     if (*(volatile int*)a.host_status == DEV_TIMEOUT) {
         // some CTAs may have counted themselves into the statistics
         GB_CUDA(cudaMemsetAsync(h->dstatus, 0, 2 * sizeof(int), st));

@@ -163,7 +163,7 @@ int ou_finish(Handle* h, int64_t n, int64_t n_rec, int64_t blocks, double* mean,
         host = copy.data();
         GB_CUDA(cudaMemcpyAsync(host, out, bytes, cudaMemcpyDeviceToHost, st));
     }
-    GB_CUDA(cudaStreamSynchronize(st));
+    GB_CHECK(sync_results(st));
     for (int64_t r = 0; r < n_rec; ++r) {
         mean[r] = host[2 * r];
         corr[r] = host[2 * r + 1];

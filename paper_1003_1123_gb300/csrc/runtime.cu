@@ -280,22 +280,68 @@ __global__ void finish_stats_kernel(const double* partials, int64_t blocks, doub
 
 // Results come back through mapped pinned memory, so that they need no copy
 // after the kernel: a 32-byte copy to pageable memory costs a call 6 to 9 us
-// (ld_run of 1000 oscillators x 10 steps with statistics 34.4 -> 28.2 us).  One
-// block a host thread, freed when the thread ends.
+// (ld_run of 1000 oscillators x 10 steps with statistics 34.4 -> 28.2 us).  One block a
+// host thread, from the first such call on.  A thread that ends leaves its block to the next
+// (at most kSpareBlocks, 4 MB; more are freed): freeing it there would end a stream capture
+// that another thread has begun, and wait for the device.
 namespace {
+constexpr size_t kSpareBlocks = 64;
+std::mutex g_spare_mu;
+std::vector<void*>& spare_blocks()
+{
+    static auto* v = new std::vector<void*>;   // outlives the threads
+    return *v;
+}
+
+// Allocating and freeing pinned memory does not touch captures in progress.
+struct RelaxedCapture {
+    cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;
+    RelaxedCapture() { cudaThreadExchangeStreamCaptureMode(&mode); }
+    ~RelaxedCapture() { cudaThreadExchangeStreamCaptureMode(&mode); }
+};
+
 struct HostBlock {
     void* p = nullptr;
     ~HostBlock()
     {
-        if (p) cudaFreeHost(p);
+        if (!p) return;
+        {
+            std::lock_guard<std::mutex> lk(g_spare_mu);
+            if (spare_blocks().size() < kSpareBlocks) {
+                spare_blocks().push_back(p);
+                return;
+            }
+        }
+        RelaxedCapture relaxed;
+        cudaFreeHost(p);
     }
 };
 }  // namespace
 
+static thread_local HostBlock t_block;
+
+int sync_results(cudaStream_t st)
+{
+    const cudaError_t e = cudaStreamSynchronize(st);
+    if (e == cudaSuccess) return GBRNG_OK;
+    t_block.p = nullptr;   // refused, and the kernel may still write there: nobody else's
+    return fail(GBRNG_ECUDA, "cudaStreamSynchronize failed: %s", cudaGetErrorString(e));
+}
+
 void* host_block()
 {
-    static thread_local HostBlock t;
-    if (!t.p && cudaHostAlloc(&t.p, kHostBlock, cudaHostAllocMapped | cudaHostAllocPortable) != cudaSuccess) {
+    HostBlock& t = t_block;
+    if (t.p) return t.p;
+    {
+        std::lock_guard<std::mutex> lk(g_spare_mu);
+        if (!spare_blocks().empty()) {
+            t.p = spare_blocks().back();
+            spare_blocks().pop_back();
+            return t.p;
+        }
+    }
+    RelaxedCapture relaxed;
+    if (cudaHostAlloc(&t.p, kHostBlock, cudaHostAllocMapped | cudaHostAllocPortable) != cudaSuccess) {
         cudaGetLastError();
         t.p = nullptr;
     }
@@ -326,7 +372,7 @@ int finish_stats(Handle* h, const StatsSink& sink, int64_t blocks, int64_t n_ste
         finish_stats_kernel<<<1, 256, 0, st>>>(h->partials, blocks, host);
         GB_CUDA(cudaGetLastError());
     }
-    GB_CUDA(cudaStreamSynchronize(st));
+    GB_CHECK(sync_results(st));
     out->sum_x2 = host[0];
     out->sum_v2 = host[1];
     out->sum_xv = host[2];
