@@ -89,7 +89,6 @@ __device__ __forceinline__ uint32_t word_load(uint32_t x) { return x; }
 constexpr int32_t kR2M1 = 2147483563, kR2A1 = 40014, kR2Q1 = 53668, kR2R1 = 12211;
 constexpr int32_t kR2M2 = 2147483399, kR2A2 = 40692, kR2Q2 = 52774, kR2R2 = 3791;
 constexpr int32_t kR2Imm1 = kR2M1 - 1;
-constexpr int32_t kR2Ndiv = 1 + kR2Imm1 / 32;
 static_assert(kR2Q1 == kR2M1 / kR2A1 && kR2R1 == kR2M1 % kR2A1, "Schrage constants");
 static_assert(kR2Q2 == kR2M2 / kR2A2 && kR2R2 == kR2M2 % kR2A2, "Schrage constants");
 
@@ -821,14 +820,6 @@ __device__ __forceinline__ void block_reduce_sum(double (&v)[N], double* smem)
     for (int k = 0; k < N; ++k) v[k] = __shfl_sync(0xffffffffu, a, k);
 }
 
-// Sum over a warp, in its first lane.
-__device__ __forceinline__ double warp_sum(double v)
-{
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) v += __shfl_down_sync(0xffffffffu, v, o);
-    return v;
-}
-
 // A run's statistics: each block's four sums in partials[block][4]; with out (in
 // mapped host memory) the last block to finish adds them up in a fixed order and
 // leaves the ticket at zero for the next launch.  Called by one whole warp of
@@ -892,18 +883,6 @@ __device__ __forceinline__ uint64_t global_ns()
 __device__ __forceinline__ void red_release_add_u64(uint64_t* p, uint64_t v)
 {
     asm volatile("red.release.gpu.global.add.u64 [%0], %1;" ::"l"(p), "l"(v) : "memory");
-}
-
-__device__ __forceinline__ void st_release_u64(uint64_t* p, uint64_t v)
-{
-    asm volatile("st.release.gpu.global.u64 [%0], %1;" ::"l"(p), "l"(v) : "memory");
-}
-
-__device__ __forceinline__ uint64_t ld_relaxed_u64(const uint64_t* p)
-{
-    uint64_t v;
-    asm volatile("ld.relaxed.gpu.global.u64 %0, [%1];" : "=l"(v) : "l"(p) : "memory");
-    return v;
 }
 
 __device__ __forceinline__ uint64_t ld_acquire_u64(const uint64_t* p)

@@ -30,7 +30,7 @@ void clear_error();
         if (rc_ != GBRNG_OK) return rc_;                                                \
     } while (0)
 
-// Status values written by kernels into the handle's device status word.
+// Status values of a Lagged Fibonacci launch.
 enum : int { DEV_OK = 0, DEV_TIMEOUT = 1 };
 
 // NVTX range named after the C ABI call, open for the call's duration (a
@@ -67,7 +67,7 @@ struct Handle {
     // scratch owned by the handle
     uint64_t* progress = nullptr;   // grid-barrier arrival counter, status (LFG)
     int64_t progress_cap = 0;
-    int* dstatus = nullptr;         // device status word, then the statistics' ticket
+    unsigned* ticket = nullptr;     // blocks that have left their statistics (0 between launches)
     double* partials = nullptr;     // per-block reduction partials
     int64_t partials_cap = 0;
     float2* eacc = nullptr;         // paper-form runs: per-oscillator energy sum (Kahan s, c)

@@ -342,7 +342,7 @@ int lfg_end(Handle* h, const LfgArgs& a, cudaStream_t st)
     GB_CHECK(sync_results(st));
     if (*(volatile int*)a.host_status == DEV_TIMEOUT) {
         // some CTAs may have counted themselves into the statistics
-        GB_CUDA(cudaMemsetAsync(h->dstatus, 0, 2 * sizeof(int), st));
+        GB_CUDA(cudaMemsetAsync(h->ticket, 0, sizeof(unsigned), st));
         return fail(GBRNG_ETIMEOUT, "Lagged Fibonacci grid barrier wait exceeded %llu ns",
                     (unsigned long long)wait_limit_ns());
     }

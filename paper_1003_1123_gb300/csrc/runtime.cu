@@ -196,7 +196,7 @@ static void free_handle(Handle* h)
     cudaFree(h->lcg);
     cudaFree(h->ring);
     cudaFree(h->progress);
-    cudaFree(h->dstatus);
+    cudaFree(h->ticket);
     cudaFree(h->partials);
     cudaFree(h->eacc);
     cudaFree(h->adj);
@@ -216,13 +216,13 @@ static int alloc_state(Handle* h)
         if (h->depth == 0) lfg_new_handle(h);   // a clone has its source's ring
         e = cudaMalloc(&h->ring, sizeof(uint32_t) * h->ring_size);
     }
-    if (e == cudaSuccess) e = cudaMalloc(&h->dstatus, sizeof(int) * 2);
+    if (e == cudaSuccess) e = cudaMalloc(&h->ticket, sizeof(unsigned));
     if (e != cudaSuccess) {
         cudaGetLastError();
         return fail(GBRNG_ENOMEM, "cannot allocate generator state for %lld streams: %s",
                     (long long)h->n, cudaGetErrorString(e));
     }
-    GB_CUDA(cudaMemset(h->dstatus, 0, sizeof(int) * 2));
+    GB_CUDA(cudaMemset(h->ticket, 0, sizeof(unsigned)));
     return GBRNG_OK;
 }
 
@@ -354,7 +354,7 @@ int make_sink(Handle* h, int64_t blocks, bool want, StatsSink* out)
     if (!want) return GBRNG_OK;
     GB_CHECK(ensure_partials(h, blocks));
     out->partials = h->partials;
-    out->ticket = reinterpret_cast<unsigned*>(h->dstatus + 1);
+    out->ticket = h->ticket;
     if (blocks <= kFuseBlocks) {
         out->out = (double*)host_block();
         if (!out->out) return fail(GBRNG_ENOMEM, "cannot allocate pinned host memory");
