@@ -351,7 +351,8 @@ int lfg_end(Handle* h, const LfgArgs& a, cudaStream_t st)
 
 int lfg_cooperative(const void* fn, int64_t G, int T, void** args, size_t smem, cudaStream_t st)
 {
-    if (smem > 48 * 1024)
+    // beyond 48 KB with the kernel's own, at most 2 KB, the limit has to be raised
+    if (smem > 46 * 1024)
         GB_CUDA(cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
     GB_CUDA(cudaLaunchCooperativeKernel(fn, dim3((unsigned)G), dim3(T), args, smem, st));
     return GBRNG_OK;
