@@ -230,21 +230,40 @@ __global__ void lfg_extend_kernel(LfgArgs a, int64_t q_hi, int64_t count)
 }
 
 // The whole extension of a small row in one launch, by one cluster of blocks with its
-// barrier between the pieces of sl positions: a fan of depth 16 takes 15 of them (handle of
-// row 2 made in 81 us with a launch each, 41 so).  Other blocks' values
-// come from L2.
+// barrier between the pieces (other blocks' values come from L2).  n applications of the
+// reverse, x_q = sum_i (-1)^i C(n, i) x_{q + (n-i) ll + i sl}, give pieces of n sl positions once
+// every read lies below 0, from q = -n ll on: a fan of depth 16 takes 7 or 8 pieces with n up to
+// 4 where it takes 15 with one (handle of row 0, 3, 6 made in 32, 37, 60 us with one; 28, 32, 55
+// with two; 26, 30, 56 with four; a launch each 81 for row 2).
 constexpr int kExtBlocks = 8, kExtThreads = 1024;
+template <int N>
+__device__ __forceinline__ void extend_piece(const LfgArgs& a, int64_t q, int64_t cnt)
+{
+    constexpr uint32_t binom = N == 1 ? 0x11u : N == 2 ? 0x121u : 0x14641u;   // C(N, i), a digit each
+    const uint32_t s0 = (uint32_t)(q + a.R), ll = a.D + a.sl;
+#pragma unroll 4
+    for (uint32_t i = blockIdx.x * kExtThreads + threadIdx.x; i < (uint32_t)cnt; i += kExtBlocks * kExtThreads) {
+        uint32_t sum = 0;
+#pragma unroll
+        for (int k = 0; k <= N; ++k) {
+            const uint32_t v = (binom >> (4 * k) & 15u) * __ldcg(a.ring + s0 + i + (N - k) * ll + k * a.sl);
+            sum += k & 1 ? 0u - v : v;
+        }
+        __stcg(a.ring + s0 + i, sum);
+    }
+}
+
 __global__ void __cluster_dims__(kExtBlocks, 1, 1) __launch_bounds__(kExtThreads)
     lfg_extend_all_kernel(LfgArgs a, int64_t q_hi, int64_t q_end)
 {
-    const uint32_t R = a.R;
+    const int64_t ll = (int64_t)a.D + a.sl;
     while (q_hi > q_end) {
-        const int64_t cnt = min((int64_t)a.sl, q_hi - q_end);
+        const int n = q_hi <= -4 * ll ? 4 : q_hi <= -2 * ll ? 2 : 1;
+        const int64_t cnt = min((int64_t)n * a.sl, q_hi - q_end);
         q_hi -= cnt;
-        for (int64_t i = blockIdx.x * kExtThreads + threadIdx.x; i < cnt; i += kExtBlocks * kExtThreads) {
-            const int64_t q = q_hi + i;
-            __stcg(a.ring + (uint32_t)(q + R), __ldcg(a.ring + (uint32_t)(q + a.D + a.sl + R)) - __ldcg(a.ring + (uint32_t)(q + a.sl + R)));
-        }
+        if (n == 4) extend_piece<4>(a, q_hi, cnt);
+        else if (n == 2) extend_piece<2>(a, q_hi, cnt);
+        else extend_piece<1>(a, q_hi, cnt);
         cluster_sync();
     }
 }

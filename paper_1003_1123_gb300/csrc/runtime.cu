@@ -188,6 +188,66 @@ static int launch_seed(Handle* h, cudaStream_t st)
     return GBRNG_OK;
 }
 
+// Rings of destroyed Lagged Fibonacci handles, for the next handle of the row on the device:
+// three rounds of the deepest fan are 0.2 to 48 MB, and cudaMalloc takes 100 us and more where
+// no block that it holds has the room (handle of row 3 made in 155 us, 30 with a kept ring;
+// of row 9 165, 26).  At most kKeptRings and kKeptRingBytes of them, the oldest given back
+// first, all where an allocation fails.  A ring is kept only once the device has been waited
+// for, so no stream still uses it.
+namespace {
+constexpr size_t kKeptRings = 8, kKeptRingBytes = (size_t)100 << 20;
+struct KeptRing {
+    int device;
+    uint32_t words;
+    uint32_t* p;
+};
+std::mutex g_ring_mu;
+std::vector<KeptRing>& kept_rings()
+{
+    static auto* v = new std::vector<KeptRing>;   // outlives handles of static storage
+    return *v;
+}
+
+uint32_t* take_ring(int device, uint32_t words)
+{
+    std::lock_guard<std::mutex> lk(g_ring_mu);
+    auto& v = kept_rings();
+    for (size_t i = v.size(); i-- > 0;)
+        if (v[i].device == device && v[i].words == words) {
+            uint32_t* p = v[i].p;
+            v.erase(v.begin() + i);
+            return p;
+        }
+    return nullptr;
+}
+
+// Give back the oldest until at most `rings` of `bytes` are left.
+void trim_rings(size_t rings, size_t bytes)
+{
+    auto& v = kept_rings();
+    size_t sum = 0;
+    for (const KeptRing& r : v) sum += sizeof(uint32_t) * (size_t)r.words;
+    while (!v.empty() && (v.size() > rings || sum > bytes)) {
+        sum -= sizeof(uint32_t) * (size_t)v[0].words;
+        cudaFree(v[0].p);
+        v.erase(v.begin());
+    }
+}
+
+void keep_ring(const KeptRing& r)
+{
+    std::lock_guard<std::mutex> lk(g_ring_mu);
+    kept_rings().push_back(r);
+    trim_rings(kKeptRings, kKeptRingBytes);
+}
+
+void give_rings_back()
+{
+    std::lock_guard<std::mutex> lk(g_ring_mu);
+    trim_rings(0, 0);
+}
+}  // namespace
+
 static void free_handle(Handle* h)
 {
     if (!h) return;
@@ -206,15 +266,23 @@ static void free_handle(Handle* h)
 static int alloc_state(Handle* h)
 {
     cudaError_t e = cudaSuccess;
+    auto get = [&](auto** p, size_t bytes) {
+        e = cudaMalloc(p, bytes);
+        if (e != cudaErrorMemoryAllocation) return;
+        cudaGetLastError();
+        give_rings_back();
+        e = cudaMalloc(p, bytes);
+    };
     if (h->kind == GBRNG_TAUS) {
-        e = cudaMalloc(&h->taus, sizeof(uint4) * h->n);
+        get(&h->taus, sizeof(uint4) * h->n);
     } else if (h->kind == GBRNG_RAN2) {
-        e = cudaMalloc(&h->r2, sizeof(int32_t) * 35 * h->n);
+        get(&h->r2, sizeof(int32_t) * 35 * h->n);
     } else if (h->kind == GBRNG_LCG) {
-        e = cudaMalloc(&h->lcg, sizeof(uint32_t) * h->n);
+        get(&h->lcg, sizeof(uint32_t) * h->n);
     } else {
         if (h->depth == 0) lfg_new_handle(h);   // a clone has its source's ring
-        e = cudaMalloc(&h->ring, sizeof(uint32_t) * h->ring_size);
+        h->ring = take_ring(h->device, h->ring_size);
+        if (!h->ring) get(&h->ring, sizeof(uint32_t) * h->ring_size);
     }
     if (e == cudaSuccess) e = cudaMalloc(&h->ticket, sizeof(unsigned));
     if (e != cudaSuccess) {
@@ -467,6 +535,10 @@ int rng_destroy(gbrng_t rng)
     cudaGetDevice(&dev);
     cudaSetDevice(rng->device);
     cudaError_t e = cudaDeviceSynchronize();
+    if (e == cudaSuccess && rng->ring) {
+        keep_ring({rng->device, rng->ring_size, rng->ring});
+        rng->ring = nullptr;
+    }
     free_handle(rng);
     cudaSetDevice(dev);
     if (e != cudaSuccess) return fail(GBRNG_ECUDA, "pending work failed: %s", cudaGetErrorString(e));
