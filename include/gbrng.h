@@ -25,7 +25,9 @@
  *  - Device pointers passed in (dst, x, v, K_per, dK_per) are owned by the
  *    caller and must be device-accessible memory of the handle's device.
  *  - The library owns generator state and scratch.  A handle allocates its
- *    state in rng_init* and frees everything in rng_destroy.
+ *    state in rng_init* and frees everything in rng_destroy; the rings of
+ *    destroyed Lagged Fibonacci handles are kept for the next ones (at most
+ *    eight and 100 MB in the process, given back when an allocation fails).
  *  - A handle is not thread-safe; calls on one handle must not overlap.
  *  - Device errors map to GBRNG_ECUDA; a device-side wait that exceeded its
  *    limit (Lagged Fibonacci grid barrier) maps to GBRNG_ETIMEOUT, after which
@@ -85,7 +87,8 @@ int rng_init(gbrng_t* out, int kind, uint64_t seed, int64_t n_streams, void* str
  * sl = 12470 gives a reducible trinomial.  GBRNG_ELAGS for a row outside 0-9. */
 int rng_init_lfg(gbrng_t* out, uint64_t seed, int64_t n_threads, int lag_row, void* stream);
 
-/* Free the handle and everything it owns (waits for its pending work). */
+/* Free the handle and everything it owns (waits for its pending work; a Lagged
+ * Fibonacci handle's ring may stay for the next handle, see above). */
 int rng_destroy(gbrng_t rng);
 
 /* New handle with an identical copy of src's state (device-to-device). */
@@ -239,8 +242,8 @@ typedef struct {
  * (1/n) sum_i R_i R_i(0), R(0) the positions on entry (the paper's <R(t)> and
  * <R(t)R(0)>); both are host arrays of n_steps/every + 1 doubles, or both NULL
  * (no records).  Lagged Fibonacci: every step is one round of 2n positions,
- * 2n <= ll - sl below position ll and <= 2(ll - sl) after, else GBRNG_ELAGS and
- * nothing runs.  Requirements: n >= 1, n_steps >= 0, every >= 1, k_sp > 0,
+ * 2n <= k (ll - sl) with k = 2 or the order set (gbrng_set_lfg_order), else
+ * GBRNG_ELAGS and nothing runs.  Requirements: n >= 1, n_steps >= 0, every >= 1, k_sp > 0,
  * xi > 0, kT >= 0, dt > 0.  Synchronises the stream when records are
  * requested.  Scratch is the handle's: 16 bytes per record per 256 particles,
  * or up to 256 MiB where that is more; GBRNG_EINVAL beyond 4 GiB of the former. */
@@ -254,9 +257,8 @@ int ou_run(ou_system* sys, int64_t n_steps, int64_t every, double* mean_host, do
  * Same draws, stream positions and binary32 operations as ld_run, so x, v and
  * the generator state come out bit for bit equal to ld_run's; the statistics
  * equal ld_run's up to summation order.  Lagged Fibonacci: a step's 4N
- * positions must be independent of each other, 4N <= ll - sl while the
- * generator is below position ll and 4N <= 2 (ll - sl) after (the leap form),
- * else GBRNG_ELAGS and nothing runs.  Owns 8 bytes of scratch per oscillator
+ * positions must be independent of each other, 4N <= k (ll - sl) with k = 2 or
+ * the order set (gbrng_set_lfg_order), else GBRNG_ELAGS and nothing runs.  Owns 8 bytes of scratch per oscillator
  * (grown on demand, freed in rng_destroy).  out_host as in ld_run. */
 int ld_run_stepwise(ld_system* sys, int64_t n_steps, ld_stats* out_host, void* stream);
 
@@ -326,7 +328,7 @@ int ld_set_adjoint_history_limit(int64_t bytes);
  * reads the statistics back and synchronises the stream (the host waits for
  * the run); on a stream in capture mode that is refused with GBRNG_EINVAL
  * before any work is queued.  It runs one oscillator a thread, so Hybrid Taus
- * and Ran2 systems that fill a resident wave run about 16 and 19% slower than in
+ * and Ran2 systems that fill a resident wave run about 16 and 18% slower than in
  * ld_run, which takes two.  Other requirements and errors as ld_run. */
 int ld_run_noalloc(ld_system* sys, int64_t n_steps, ld_stats* out_host, void* stream);
 

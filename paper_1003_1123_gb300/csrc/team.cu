@@ -24,13 +24,14 @@
 // A stage is filled by M warps, handed to the consumer by a named barrier, and
 // handed back by another, so the producers refill it as soon as it is consumed.
 //
-// Two shapes.  16 oscillators a block (16 chunks a pass, 50 KB: four blocks a SM)
-// and, for the fewest oscillators, 8 a block (32 chunks), which spreads the
+// Two shapes, of 55 KB each (four blocks a SM).  16 oscillators a block (16 chunks a
+// pass) and, for the fewest oscillators, 8 a block (32 chunks), which spreads the
 // consumers' chains wider.  Hybrid Taus x 1000 steps, one oscillator a thread /
 // 16 a block / 8 a block, us: 1000 oscillators 119 / 22.6 / 14.5; 4096 119 / 32.9
 // / 32.9; 1e4 119 / 67.7 / 63.6; 2e4 193 / 113 / 112; 5.8e4 287 / 287 (bound there by
 // the issue of the instructions that one oscillator a thread does not need, the jumps and
-// the hand-over).
+// the hand-over).  With statistics a step costs a fifth more: 1e4 66 ns instead of 55, 5.8e4
+// 343 instead of 291, where one oscillator a thread takes 286 either way.
 #include <algorithm>
 #include <type_traits>
 
