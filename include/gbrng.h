@@ -27,7 +27,7 @@
  *  - The library owns generator state and scratch.  A handle allocates its
  *    state in rng_init* and frees everything in rng_destroy; the rings of
  *    destroyed Lagged Fibonacci handles are kept for the next ones (at most
- *    eight and 100 MB in the process, given back when an allocation fails).
+ *    eight and 100 MB in the process, given back when an allocation here fails).
  *  - A handle is not thread-safe; calls on one handle must not overlap.
  *  - Device errors map to GBRNG_ECUDA; a device-side wait that exceeded its
  *    limit (Lagged Fibonacci grid barrier) maps to GBRNG_ETIMEOUT, after which

@@ -306,11 +306,11 @@ static int make_plan(int device, int kind, const std::vector<int64_t>& sizes, Tu
         return fail(GBRNG_EINVAL, "batched launch shape T=%d K=%d does not fit", tune.T, tune.K);
     }
     p->grid = std::min<int64_t>((int64_t)di.sms * occ, p->n_tiles);
-    cudaError_t e = cudaMalloc(&p->dsys, sizeof(SysDesc) * p->n_sys);
-    if (e == cudaSuccess) e = cudaMalloc(&p->dtiles, sizeof(Tile) * p->n_tiles);
-    if (e == cudaSuccess) e = cudaMalloc(&p->dbegin, sizeof(int64_t) * (p->n_sys + 1));
-    if (e == cudaSuccess) e = cudaMalloc(&p->dpartials, sizeof(double) * 4 * p->n_tiles);
-    if (e == cudaSuccess) e = cudaMalloc(&p->dstats, sizeof(double) * 4 * p->n_sys);
+    cudaError_t e = device_alloc((void**)&p->dsys, sizeof(SysDesc) * p->n_sys);
+    if (e == cudaSuccess) e = device_alloc((void**)&p->dtiles, sizeof(Tile) * p->n_tiles);
+    if (e == cudaSuccess) e = device_alloc((void**)&p->dbegin, sizeof(int64_t) * (p->n_sys + 1));
+    if (e == cudaSuccess) e = device_alloc((void**)&p->dpartials, sizeof(double) * 4 * p->n_tiles);
+    if (e == cudaSuccess) e = device_alloc((void**)&p->dstats, sizeof(double) * 4 * p->n_sys);
     if (e == cudaSuccess)
         e = cudaMemcpy(p->dtiles, p->tiles.data(), sizeof(Tile) * p->n_tiles, cudaMemcpyHostToDevice);
     if (e == cudaSuccess)
@@ -391,7 +391,7 @@ static int autotune(const ld_system* sys, int n_sys, int kind, const std::vector
         bytes += up(kind == GBRNG_TAUS ? sizeof(uint4) * S : sizeof(int32_t) * 35 * S);
     }
     char* scratch = nullptr;
-    if (cudaMalloc(&scratch, bytes) != cudaSuccess) {
+    if (device_alloc((void**)&scratch, bytes) != cudaSuccess) {
         cudaGetLastError();
         return fail(GBRNG_ENOMEM, "autotune scratch (%zu bytes) allocation failed", bytes);
     }

@@ -87,6 +87,8 @@ struct DevInfo {
 };
 int dev_info(int device, DevInfo* out);
 
+// cudaMalloc, a second time without the kept rings (runtime.cu) where memory has run out.
+cudaError_t device_alloc(void** p, size_t bytes);
 int ensure_partials(Handle* h, int64_t count);
 int ensure_progress(Handle* h, int64_t count);
 

@@ -54,13 +54,86 @@ uint64_t wait_limit_ns() { return g_wait_ns.load(); }
 static std::atomic<int64_t> g_stall_chunk{-1};
 int64_t test_stall_chunk() { return g_stall_chunk.load(); }
 
+// Rings of destroyed Lagged Fibonacci handles, for the next handle of the row on the device:
+// three rounds of the deepest fan are 0.2 to 48 MB, and cudaMalloc takes 100 us and more where
+// no block that it holds has the room (handle of row 3 made in 155 us, 30 with a kept ring;
+// of row 9 165, 26).  At most kKeptRings and kKeptRingBytes of them, the oldest given back
+// first, all where an allocation of this library fails.  A ring is kept only once the device
+// has been waited for, so no stream still uses it.
+namespace {
+constexpr size_t kKeptRings = 8, kKeptRingBytes = (size_t)100 << 20;
+struct KeptRing {
+    int device;
+    uint32_t words;
+    uint32_t* p;
+};
+std::mutex g_ring_mu;
+std::vector<KeptRing>& kept_rings()
+{
+    static auto* v = [] {   // outlives handles of static storage; never grows
+        auto* r = new std::vector<KeptRing>;
+        r->reserve(kKeptRings + 1);
+        return r;
+    }();
+    return *v;
+}
+
+uint32_t* take_ring(int device, uint32_t words)
+{
+    std::lock_guard<std::mutex> lk(g_ring_mu);
+    auto& v = kept_rings();
+    for (size_t i = v.size(); i-- > 0;)
+        if (v[i].device == device && v[i].words == words) {
+            uint32_t* p = v[i].p;
+            v.erase(v.begin() + i);
+            return p;
+        }
+    return nullptr;
+}
+
+// Give back the oldest until at most `rings` of `bytes` are left.
+void trim_rings(size_t rings, size_t bytes)
+{
+    auto& v = kept_rings();
+    size_t sum = 0;
+    for (const KeptRing& r : v) sum += sizeof(uint32_t) * (size_t)r.words;
+    while (!v.empty() && (v.size() > rings || sum > bytes)) {
+        sum -= sizeof(uint32_t) * (size_t)v[0].words;
+        cudaFree(v[0].p);
+        v.erase(v.begin());
+    }
+}
+
+void keep_ring(const KeptRing& r)
+{
+    std::lock_guard<std::mutex> lk(g_ring_mu);
+    kept_rings().push_back(r);
+    trim_rings(kKeptRings, kKeptRingBytes);
+}
+
+void give_rings_back()
+{
+    std::lock_guard<std::mutex> lk(g_ring_mu);
+    trim_rings(0, 0);
+}
+}  // namespace
+
+cudaError_t device_alloc(void** p, size_t bytes)
+{
+    cudaError_t e = cudaMalloc(p, bytes);
+    if (e != cudaErrorMemoryAllocation) return e;
+    cudaGetLastError();
+    give_rings_back();
+    return cudaMalloc(p, bytes);
+}
+
 int ensure_partials(Handle* h, int64_t count)
 {
     if (count <= h->partials_cap) return GBRNG_OK;
     if (h->partials) cudaFree(h->partials);
     h->partials = nullptr;
     h->partials_cap = 0;
-    if (cudaMalloc(&h->partials, sizeof(double) * 4 * count) != cudaSuccess) {
+    if (device_alloc((void**)&h->partials, sizeof(double) * 4 * count) != cudaSuccess) {
         cudaGetLastError();
         return fail(GBRNG_ENOMEM, "cannot allocate %lld reduction partials", (long long)count);
     }
@@ -74,7 +147,7 @@ int ensure_eacc(Handle* h, int64_t n)
     if (h->eacc) cudaFree(h->eacc);
     h->eacc = nullptr;
     h->eacc_cap = 0;
-    if (cudaMalloc(&h->eacc, sizeof(float2) * n) != cudaSuccess) {
+    if (device_alloc((void**)&h->eacc, sizeof(float2) * n) != cudaSuccess) {
         cudaGetLastError();
         return fail(GBRNG_ENOMEM, "cannot allocate %lld energy sums", (long long)n);
     }
@@ -88,7 +161,7 @@ int ensure_adj(Handle* h, size_t bytes)
     if (h->adj) cudaFree(h->adj);
     h->adj = nullptr;
     h->adj_bytes = 0;
-    if (cudaMalloc((void**)&h->adj, bytes) != cudaSuccess) {
+    if (device_alloc((void**)&h->adj, bytes) != cudaSuccess) {
         cudaGetLastError();
         return fail(GBRNG_ENOMEM, "adjoint scratch of %zu bytes", bytes);
     }
@@ -102,7 +175,7 @@ int ensure_progress(Handle* h, int64_t count)
     if (h->progress) cudaFree(h->progress);
     h->progress = nullptr;
     h->progress_cap = 0;
-    if (cudaMalloc(&h->progress, sizeof(uint64_t) * count) != cudaSuccess) {
+    if (device_alloc((void**)&h->progress, sizeof(uint64_t) * count) != cudaSuccess) {
         cudaGetLastError();
         return fail(GBRNG_ENOMEM, "cannot allocate %lld progress counters", (long long)count);
     }
@@ -188,66 +261,6 @@ static int launch_seed(Handle* h, cudaStream_t st)
     return GBRNG_OK;
 }
 
-// Rings of destroyed Lagged Fibonacci handles, for the next handle of the row on the device:
-// three rounds of the deepest fan are 0.2 to 48 MB, and cudaMalloc takes 100 us and more where
-// no block that it holds has the room (handle of row 3 made in 155 us, 30 with a kept ring;
-// of row 9 165, 26).  At most kKeptRings and kKeptRingBytes of them, the oldest given back
-// first, all where an allocation fails.  A ring is kept only once the device has been waited
-// for, so no stream still uses it.
-namespace {
-constexpr size_t kKeptRings = 8, kKeptRingBytes = (size_t)100 << 20;
-struct KeptRing {
-    int device;
-    uint32_t words;
-    uint32_t* p;
-};
-std::mutex g_ring_mu;
-std::vector<KeptRing>& kept_rings()
-{
-    static auto* v = new std::vector<KeptRing>;   // outlives handles of static storage
-    return *v;
-}
-
-uint32_t* take_ring(int device, uint32_t words)
-{
-    std::lock_guard<std::mutex> lk(g_ring_mu);
-    auto& v = kept_rings();
-    for (size_t i = v.size(); i-- > 0;)
-        if (v[i].device == device && v[i].words == words) {
-            uint32_t* p = v[i].p;
-            v.erase(v.begin() + i);
-            return p;
-        }
-    return nullptr;
-}
-
-// Give back the oldest until at most `rings` of `bytes` are left.
-void trim_rings(size_t rings, size_t bytes)
-{
-    auto& v = kept_rings();
-    size_t sum = 0;
-    for (const KeptRing& r : v) sum += sizeof(uint32_t) * (size_t)r.words;
-    while (!v.empty() && (v.size() > rings || sum > bytes)) {
-        sum -= sizeof(uint32_t) * (size_t)v[0].words;
-        cudaFree(v[0].p);
-        v.erase(v.begin());
-    }
-}
-
-void keep_ring(const KeptRing& r)
-{
-    std::lock_guard<std::mutex> lk(g_ring_mu);
-    kept_rings().push_back(r);
-    trim_rings(kKeptRings, kKeptRingBytes);
-}
-
-void give_rings_back()
-{
-    std::lock_guard<std::mutex> lk(g_ring_mu);
-    trim_rings(0, 0);
-}
-}  // namespace
-
 static void free_handle(Handle* h)
 {
     if (!h) return;
@@ -266,13 +279,7 @@ static void free_handle(Handle* h)
 static int alloc_state(Handle* h)
 {
     cudaError_t e = cudaSuccess;
-    auto get = [&](auto** p, size_t bytes) {
-        e = cudaMalloc(p, bytes);
-        if (e != cudaErrorMemoryAllocation) return;
-        cudaGetLastError();
-        give_rings_back();
-        e = cudaMalloc(p, bytes);
-    };
+    auto get = [&](auto** p, size_t bytes) { e = device_alloc((void**)p, bytes); };
     if (h->kind == GBRNG_TAUS) {
         get(&h->taus, sizeof(uint4) * h->n);
     } else if (h->kind == GBRNG_RAN2) {
@@ -284,7 +291,7 @@ static int alloc_state(Handle* h)
         h->ring = take_ring(h->device, h->ring_size);
         if (!h->ring) get(&h->ring, sizeof(uint32_t) * h->ring_size);
     }
-    if (e == cudaSuccess) e = cudaMalloc(&h->ticket, sizeof(unsigned));
+    if (e == cudaSuccess) get(&h->ticket, sizeof(unsigned));
     if (e != cudaSuccess) {
         cudaGetLastError();
         return fail(GBRNG_ENOMEM, "cannot allocate generator state for %lld streams: %s",
@@ -357,7 +364,11 @@ constexpr size_t kSpareBlocks = 64;
 std::mutex g_spare_mu;
 std::vector<void*>& spare_blocks()
 {
-    static auto* v = new std::vector<void*>;   // outlives the threads
+    static auto* v = [] {   // outlives the threads; never grows
+        auto* r = new std::vector<void*>;
+        r->reserve(kSpareBlocks);
+        return r;
+    }();
     return *v;
 }
 
