@@ -370,9 +370,15 @@ int lfg_end(Handle* h, const LfgArgs& a, cudaStream_t st)
 
 int lfg_cooperative(const void* fn, int64_t G, int T, void** args, size_t smem, cudaStream_t st)
 {
-    // beyond 48 KB with the kernel's own, at most 2 KB, the limit has to be raised
-    if (smem > 46 * 1024)
-        GB_CUDA(cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+    // beyond 48 KB with the kernel's own, at most 2 KB, the limit has to be raised: to one
+    // value, as another thread may launch the same kernel with more in between
+    if (smem > 46 * 1024) {
+        int device = 0;
+        DevInfo di;
+        GB_CUDA(cudaGetDevice(&device));
+        GB_CHECK(dev_info(device, &di));
+        GB_CUDA(cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)di.smem_optin - 2048));
+    }
     GB_CUDA(cudaLaunchCooperativeKernel(fn, dim3((unsigned)G), dim3(T), args, smem, st));
     return GBRNG_OK;
 }

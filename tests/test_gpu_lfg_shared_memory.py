@@ -50,3 +50,36 @@ def test_first_launch_of_48_kb(what):
     code = "import torch\nfrom paper_1003_1123_gb300 import gbrng as G\n" + RUNS[what] + "torch.cuda.synchronize()\n"
     r = subprocess.run([sys.executable, "-c", code], cwd=ROOT, capture_output=True, text=True, timeout=120)
     assert r.returncode == 0, r.stderr[-600:]
+
+
+def test_threads_with_launches_of_several_sizes():
+    """Threads that launch the same kernels with more and with less shared memory: neither takes
+    the other's limit away."""
+    if not torch.cuda.is_available():
+        pytest.skip("needs a CUDA GPU")
+    import threading
+    from paper_1003_1123_gb300 import gbrng as G
+    errors = []
+    fills = [(G.rng_init_lfg(k, 1000, 9), n) for k, n in enumerate((10**6, 15 * 10**5, 21 * 10**5))]
+    runs = []
+    for n in (310000, 600000, 900000):
+        runs.append(G.LdSystem(G.rng_init("lagfib", 3, n), torch.zeros((n, 3), device="cuda"),
+                               torch.zeros((n, 3), device="cuda")))
+    torch.cuda.synchronize()
+
+    def work(f):
+        try:
+            with torch.cuda.stream(torch.cuda.Stream()):
+                for _ in range(60):
+                    f()
+        except G.GbrngError as e:
+            errors.append(str(e))
+
+    jobs = [lambda r=r, n=n: G.rng_fill_uniform(r, n) for r, n in fills]
+    jobs += [lambda s=s: G.ld_run(s, 2, stats=False) for s in runs]
+    threads = [threading.Thread(target=work, args=(f,)) for f in jobs]
+    for t in threads:
+        t.start()
+    for t in threads:
+        t.join()
+    assert not errors, errors[0]
